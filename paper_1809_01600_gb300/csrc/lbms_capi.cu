@@ -259,6 +259,10 @@ size_t x_word(int precision) { return precision == LBMS_FP64 ? sizeof(double) : 
 // swapping, so the state is unchanged; the X copy of cur ^ 1 is restored.
 lbms_status autotune(lbms_ctx* c) {
     Launch& L = c->L;
+    if (L.tiled) {   // chosen by rule at create
+        c->tuned = true;
+        return LBMS_OK;
+    }
     if (c->opt.step_variant > 0) {
         const int v = c->opt.step_variant - 1;
         if (kVariantNb[v] == kNbOffset16 && !L.b.nbr16)
@@ -915,6 +919,10 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
     L.drift = c->opt.coupling == LBMS_COUPLING_MS ? 1 : 0;
     L.grad_forward = c->opt.grad_stencil == LBMS_GRAD_FORWARD ? 1 : 0;
     L.outlet_extrap = c->opt.outlet_bc == LBMS_OUTLET_EXTRAPOLATED ? 1 : 0;
+    // the default step: the paper's default readings, element offsets of all
+    // populations in 32 bits, enough cells to fill the GPU
+    L.tiled = c->opt.step_variant == 0 && !L.grad_forward && !L.outlet_extrap && L.ncells >= kTileMinCells &&
+              3 * (int64_t)c->Q * (L.S + kTile) < (int64_t)1 << 32;
 
     // reduction segments and block -> case tables
     std::vector<int2> segs, case_segs(n_cases), case_rows(n_cases);
@@ -989,7 +997,8 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
             max_n = std::max<int64_t>(max_n, cs.N);
             max_nf = std::max<int64_t>(max_nf, cs.nf);
         }
-        int16_t* nb16 = static_cast<int16_t*>(dev_alloc(c, (size_t)nbw16 * L.S * sizeof(int16_t)));
+        int16_t* nb16 =
+            L.tiled ? nullptr : static_cast<int16_t*>(dev_alloc(c, (size_t)nbw16 * L.S * sizeof(int16_t)));
         int* d_index = static_cast<int*>(dev_alloc(c, (size_t)max_n * sizeof(int)));
         int64_t* d_cells = static_cast<int64_t*>(dev_alloc(c, (size_t)max_nf * sizeof(int64_t)));
         unsigned long long* d_counts = static_cast<unsigned long long*>(dev_alloc(c, 2 * sizeof(unsigned long long)));
@@ -1036,16 +1045,18 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
         for (const auto& cs : c->cases) {
             ok_rm = ok_rm && !cs.periodic_x && cs.nx <= kRowMaskMaxNx && cs.ny <= kRowMaskMaxNy &&
                     cs.nz <= kRowMaskMaxNz;
-            entries += (int64_t)cs.ny * cs.nz * ((cs.nx + 31) / 32);
+            entries += (int64_t)cs.ny * cs.nz * (L.tiled ? (cs.nx + 15) / 16 : (cs.nx + 31) / 32);
         }
         ok_rm = ok_rm && entries < (int64_t)std::numeric_limits<int>::max();
         if (ok_rm) {
             std::vector<uint32_t> code((size_t)L.S, 0xFFFFFFFFu);
-            std::vector<uint4> tab((size_t)entries);
+            std::vector<uint4> tab(L.tiled ? 0 : (size_t)entries);
+            std::vector<uint2> tab16(L.tiled ? (size_t)entries : 0);
             int64_t next_tab = 0;
             for (int k = 0; k < n_cases; ++k) {
                 CaseHost& cs = c->cases[k];
-                cs.wpr = (cs.nx + 31) / 32;
+                const int words32 = (cs.nx + 31) / 32;
+                cs.wpr = L.tiled ? (cs.nx + 15) / 16 : words32;
                 cs.tab = (int)next_tab;
                 next_tab += (int64_t)cs.ny * cs.nz * cs.wpr;
                 for (int li = 0; li < cs.nf; ++li) {
@@ -1055,13 +1066,24 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
                     const uint32_t z = (uint32_t)(cell / ((int64_t)cs.nx * cs.ny));
                     code[(size_t)cs.base + li] = x | (y << 11) | (z << 21);
                 }
-                std::vector<uint32_t> words((size_t)cs.wpr + 2);   // words[m + 1] = voxels 32 m .. 32 m + 31
+                std::vector<uint32_t> words((size_t)words32 + 2);   // words[m + 1] = voxels 32 m .. 32 m + 31
                 int count = cs.base;                                // fluid index of the next fluid voxel
                 for (int r = 0; r < cs.ny * cs.nz; ++r) {
                     std::fill(words.begin(), words.end(), 0u);
                     const int* row = index_of[k].data() + (int64_t)r * cs.nx;
                     for (int x = 0; x < cs.nx; ++x)
                         if (row[x] >= 0) words[(size_t)(x >> 5) + 1] |= 1u << (x & 31);
+                    if (L.tiled) {   // windows of 32 voxels, one every 16 (lbms_step_tile.cuh)
+                        for (int w = 0; w < cs.wpr; ++w) {
+                            const uint64_t two = (w & 1) ? ((uint64_t)words[(w >> 1) + 2] << 32) | words[(w >> 1) + 1]
+                                                         : ((uint64_t)words[(w >> 1) + 1] << 32) | words[w >> 1];
+                            const uint32_t win = (uint32_t)(two >> ((w & 1) ? 8 : 24));
+                            const int before = kTile + count - __builtin_popcount(win & 0xFFu);
+                            tab16[(size_t)cs.tab + (size_t)r * cs.wpr + w] = make_uint2(win, (uint32_t)before);
+                            count += __builtin_popcount((win >> 8) & 0xFFFFu);
+                        }
+                        continue;
+                    }
                     for (int w = 0; w < cs.wpr; ++w) {
                         const uint64_t win = (uint64_t)(words[w] >> 16) | ((uint64_t)words[w + 1] << 16) |
                                              ((uint64_t)(words[w + 2] & 0xFFFFu) << 48);
@@ -1076,16 +1098,17 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
                 if (count != cs.base + cs.nf) return bail(fail(c, LBMS_EINVAL, "case %d: row table count mismatch", k));
             }
             L.b.cell_code = static_cast<uint32_t*>(dev_alloc(c, (size_t)L.S * sizeof(uint32_t)));
-            L.b.rowtab = static_cast<uint4*>(dev_alloc(c, (size_t)std::max<int64_t>(entries, 1) * sizeof(uint4)));
+            L.b.rowtab = static_cast<uint4*>(dev_alloc(c, (size_t)std::max<int64_t>(entries, 1) * (L.tiled ? sizeof(uint2) : sizeof(uint4))));
             if (!L.b.cell_code || !L.b.rowtab) return bail(fail(c, LBMS_ENOMEM, "row-bitmask tables"));
             e = cudaMemcpyAsync(L.b.cell_code, code.data(), code.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
                                 c->stream);
             if (e == cudaSuccess && entries)
-                e = cudaMemcpyAsync(L.b.rowtab, tab.data(), tab.size() * sizeof(uint4), cudaMemcpyHostToDevice,
+                e = cudaMemcpyAsync(L.b.rowtab, L.tiled ? (const void*)tab16.data() : tab.data(),
+                                    (size_t)entries * (L.tiled ? sizeof(uint2) : sizeof(uint4)), cudaMemcpyHostToDevice,
                                     c->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             if (e != cudaSuccess) return bail(cuda_fail(c, e, "upload of the row-bitmask tables"));
-            c->h2d += code.size() * sizeof(uint32_t) + tab.size() * sizeof(uint4);
+            c->h2d += code.size() * sizeof(uint32_t) + tab.size() * sizeof(uint4) + tab16.size() * sizeof(uint2);
         }
     }
     std::vector<int> rows;
@@ -1377,6 +1400,13 @@ lbms_status lbms_get_info(const lbms_ctx* c, lbms_info* info) {
     info->h2d_bytes = c->h2d;
     info->d2h_bytes = c->d2h;
     info->n_cases = (int)c->cases.size();
+    if (c->L.tiled) {
+        info->tile_cells = kTile;
+        info->tile_min_blocks = tile_min_blocks(c->dim, c->opt.precision);
+        info->neighbour_bits = c->L.b.rowtab ? 1 : 32;
+        info->threads_per_cell = 1;
+        return LBMS_OK;
+    }
     info->tile_cells = kVariantCells[c->L.variant];
     info->tile_min_blocks = kVariantMinBlocks[c->L.variant];
     info->neighbour_bits = kVariantNb[c->L.variant] == kNbOffset16 ? 16 : (kVariantNb[c->L.variant] == kNbRowMask ? 1 : 32);

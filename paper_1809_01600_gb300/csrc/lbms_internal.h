@@ -27,6 +27,26 @@ constexpr int kVariantNb[kStepVariants] = {kNbIndex32,  kNbIndex32, kNbIndex32, 
                                            kNbOffset16, kNbIndex32, kNbIndex32, kNbRowMask,  kNbRowMask};
 constexpr int kVariantPerCell[kStepVariants] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
 
+// The default step (lbms_step_tile.cuh): cells per tile of its population
+// layout and per block, the variant whose block -> case table it shares, how
+// many cells per SM ahead of a block it prefetches, and the blocks per SM its
+// registers are budgeted for.  Measured on the 256x128x128 anode (1.69 M fluid
+// cells, us per step), blocks per SM 5 / 6 / 8 / 9 / 10 / 12: FP32 151 / 151 /
+// 143 / 153 / 140 / 191, FP16 127 / 127 / 112 / 119 / 118 / 151, FP64 2231 /
+// 2253 / 2297 / 2306 / 2306 / 2308; 2-D FP32 (1.22 M cells) 59 up to 10, 56.5
+// at 12.  Prefetch none / 16 / 24 / 48 thousand cells ahead: FP32 155 / 144 /
+// 143 / 145, FP16 122 / 113 / 112 / 113.
+constexpr int kTile = 64;
+constexpr int kTileBlkCase = 2;
+constexpr int kTilePrefetch = 160;      // 24,320 cells on 152 SMs
+constexpr int tile_min_blocks(int dim, int precision) {
+    return dim == 2 ? (precision == 1 ? 12 : 8) : (precision == 0 ? 5 : (precision == 1 ? 10 : 8));
+}
+// Below this many cells a launch does not fill the GPU (5 blocks of 64 cells
+// on each of 152 SMs) and the autotuned variants are the faster step: 26 k
+// cells in FP32 take 4.6 us against 5.5.
+constexpr int kTileMinCells = 48640;
+
 // Limits of the per-cell coordinate word of kNbRowMask (x | y << 11 | z << 21).
 constexpr int kRowMaskMaxNx = 2048, kRowMaskMaxNy = 1024, kRowMaskMaxNz = 2048;
 
@@ -37,7 +57,8 @@ struct DevBuffers {
     int* nbr = nullptr;                // [S][nb_width]
     int16_t* nbr16 = nullptr;          // [S][nb16_width] offsets, when they all fit (else null)
     uint32_t* cell_code = nullptr;     // [S] x | y << 11 | z << 21 of each fluid cell (kNbRowMask; else null)
-    uint4* rowtab = nullptr;           // per case [rows][words]: 64-bit fluid window + index (kNbRowMask)
+    uint4* rowtab = nullptr;           // per case [rows][words]: 64-bit fluid window + index (kNbRowMask); with
+                                       // Launch::tiled uint2 windows of 32 voxels (lbms_step_tile.cuh)
     int* rows = nullptr;               // [3][total rows]: x = 0, x = 1, x = nx-1 cell of each row (-1 if solid)
     int2* case_rows = nullptr;         // [cases]: first row, row count
     void* cases = nullptr;             // [cases] CaseBC<XS> (inlet values, outlet flux, range)
@@ -66,6 +87,7 @@ struct Launch {
     int n_segs = 0;
     int nblk[kStepVariants] = {};
     int variant = 0;                   // chosen step-kernel tile shape
+    bool tiled = false;                // the step of lbms_step_tile.cuh and its population layout, instead of a variant
     int cur = 0;                       // lattice holding the latest post-collision state
     DevBuffers b;
     double D12 = 1, D13 = 1, D23 = 1;  // lattice binary diffusivities
@@ -99,6 +121,8 @@ cudaError_t launch_step(const Launch& L, cudaStream_t st);
 cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st);
 // the same with the grad_forward / outlet_extrap options compiled in
 cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream_t st);
+// the default step (lbms_step_tile.cuh); needs L.tiled
+cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st);
 cudaError_t launch_fields(const Launch& L, cudaStream_t st);
 cudaError_t launch_case_residuals(const Launch& L, int update, cudaStream_t st);

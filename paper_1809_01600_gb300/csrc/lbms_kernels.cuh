@@ -30,6 +30,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "lbms_internal.h"
 #include "lbms_lattice.cuh"
 
 namespace lbms {
@@ -214,6 +215,7 @@ struct Xv<double> {
     // value of a neighbour as used by the exchange terms and the gradient
     __device__ __forceinline__ static T nb(const double* xb, int64_t S, int s, int j) { return xb[s * S + j]; }
     __device__ __forceinline__ T exch(T n) const { return n - v; }          // neighbour minus own
+    __device__ __forceinline__ T exch_base() const { return v; }            // what exch subtracts
     __device__ __forceinline__ T minus(const Xv& b) const { return v - b.v; }  // full precision
     __device__ __forceinline__ T value() const { return v; }
     __device__ __forceinline__ double to_double() const { return v; }
@@ -235,6 +237,7 @@ struct Xv<float> {
     __device__ __forceinline__ static T nb(const float* xb, int64_t S, int s, int j) { return xb[s * S + j]; }
     // hi_n - hi is exact for neighbouring values and antisymmetric between two cells
     __device__ __forceinline__ T exch(T n) const { return n - hi; }
+    __device__ __forceinline__ T exch_base() const { return hi; }
     __device__ __forceinline__ T minus(const Xv& b) const { return (hi - b.hi) + (lo - b.lo); }
     __device__ __forceinline__ T value() const { return hi + lo; }
     __device__ __forceinline__ double to_double() const { return (double)hi + (double)lo; }
@@ -777,11 +780,19 @@ __global__ void fields_kernel(const XS* __restrict__ xcur, const XS* __restrict_
     }
 }
 
+// Element of population (s, k) of cell i: rows of stride S, or the tiled
+// layout of lbms_step_tile.cuh.
+template <class L>
+__device__ __forceinline__ int64_t pop_index(bool tiled, int64_t S, int s, int k, int i) {
+    return tiled ? (int64_t)(i / kTile) * (3 * kTile * L::Q) + (s * L::Q + k) * kTile + i % kTile
+                 : (int64_t)(s * L::Q + k) * S + i;
+}
+
 // Equilibrium start (Eq. 29, f = w X) of cells [first, first + count): h = 0;
 // the second X copy and the residual snapshot take X (already in x0).
 template <class L, typename XS, typename P>
 __global__ void init_kernel(P* __restrict__ h, const XS* __restrict__ x0, XS* __restrict__ x1,
-                            double* __restrict__ snap, int64_t S, int first, int count) {
+                            double* __restrict__ snap, int64_t S, int first, int count, bool tiled) {
     using T = typename Xv<XS>::T;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= count) return;
@@ -792,7 +803,7 @@ __global__ void init_kernel(P* __restrict__ h, const XS* __restrict__ x0, XS* __
         v.store(x1, S, s, i);
         snap[s * S + i] = v.to_double();
 #pragma unroll
-        for (int k = 0; k < L::Q; ++k) h[(int64_t)(s * L::Q + k) * S + i] = Pop<T, P>::quant(T(0));
+        for (int k = 0; k < L::Q; ++k) h[pop_index<L>(tiled, S, s, k, i)] = Pop<T, P>::quant(T(0));
     }
 }
 
@@ -939,7 +950,7 @@ __global__ void seg_finalize_kernel(const double* __restrict__ partials, const i
 // w X + h of the last step; out[3..5] = sum of X over the outlet column.
 template <class L, typename XS, typename P>
 __global__ void __launch_bounds__(kSegThreads) case_boundary_kernel(
-    const P* __restrict__ h, const XS* __restrict__ X, const int* __restrict__ nbr, int64_t S,
+    const P* __restrict__ h, bool tiled, const XS* __restrict__ X, const int* __restrict__ nbr, int64_t S,
     const int* __restrict__ row_x0, const int* __restrict__ row_x1, const int* __restrict__ row_out,
     const int2* __restrict__ case_rows, double* __restrict__ out) {
     using T = typename Xv<XS>::T;
@@ -963,14 +974,14 @@ __global__ void __launch_bounds__(kSegThreads) case_boundary_kernel(
 #pragma unroll
                     for (int s = 0; s < 3; ++s)
                         acc[s] += w * Xv<XS>::own(X, S, s, i0).to_double() +
-                                  (double)Pop<T, P>::load(h + (int64_t)(s * Q + k) * S + i0);
+                                  (double)Pop<T, P>::load(h + pop_index<L>(tiled, S, s, k, i0));
                 }
             } else if (ex == -1 && i1 >= 0) {
                 if (nbr[(int64_t)i1 * nb_width<L>() + opp<L>(k) - 1] >= 0) {
 #pragma unroll
                     for (int s = 0; s < 3; ++s)
                         acc[s] -= w * Xv<XS>::own(X, S, s, i1).to_double() +
-                                  (double)Pop<T, P>::load(h + (int64_t)(s * Q + k) * S + i1);
+                                  (double)Pop<T, P>::load(h + pop_index<L>(tiled, S, s, k, i1));
                 }
             }
         }

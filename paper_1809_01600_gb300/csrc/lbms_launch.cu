@@ -48,7 +48,8 @@ cudaError_t init_t(const Launch& L, int first, int count, cudaStream_t st) {
     const int grid = (count + kBlock - 1) / kBlock;
     init_kernel<Lat, XS, P><<<grid, kBlock, 0, st>>>(static_cast<P*>(L.b.f[L.cur]),
                                                      static_cast<const XS*>(L.b.X[L.cur]),
-                                                     static_cast<XS*>(L.b.X[L.cur ^ 1]), L.b.snap, L.S, first, count);
+                                                     static_cast<XS*>(L.b.X[L.cur ^ 1]), L.b.snap, L.S, first, count,
+                                                     L.tiled);
     return cudaGetLastError();
 }
 
@@ -96,7 +97,7 @@ template <class Lat, typename XS, typename P>
 cudaError_t boundary_t(const Launch& L, cudaStream_t st) {
     // per-case sums land in case_out[n_cases * 10 + c * 6 + v]
     case_boundary_kernel<Lat, XS, P><<<L.n_cases, kSegThreads, 0, st>>>(
-        static_cast<const P*>(L.b.f[L.cur]), static_cast<const XS*>(L.b.X[L.cur]), L.b.nbr, L.S, L.b.rows,
+        static_cast<const P*>(L.b.f[L.cur]), L.tiled, static_cast<const XS*>(L.b.X[L.cur]), L.b.nbr, L.S, L.b.rows,
         L.b.rows + L.total_rows, L.b.rows + 2 * L.total_rows, L.b.case_rows,
         L.b.case_out + (int64_t)L.n_cases * 10);
     return cudaGetLastError();
@@ -133,7 +134,9 @@ cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st) {
     if (L.grad_forward || L.outlet_extrap) return launch_step_variant_literal(L, variant, st);
     LBMS_STEP_DISPATCH(false);
 }
-cudaError_t launch_step(const Launch& L, cudaStream_t st) { return launch_step_variant(L, L.variant, st); }
+cudaError_t launch_step(const Launch& L, cudaStream_t st) {
+    return L.tiled ? launch_step_tile(L, st) : launch_step_variant(L, L.variant, st);
+}
 
 cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st) {
     LBMS_DISPATCH(init_t, L, first, count, st);
