@@ -132,7 +132,7 @@ void lbms_net_destroy(lbms_net *net);
  * added voxels solid (mask 0).  max_voxels bounds the voxels of one batch
  * (B volumes; one volume for lbms_unet_warm_start), up to
  * LBMS_UNET_MAX_VOXELS.  Activation buffers are allocated for the largest
- * batch met, about 3.4 kB per voxel of it (8 volumes of 96^3: 27 GB).
+ * batch met, about 1.2 kB per voxel of it (8 volumes of 96^3: 8.4 GB).
  * width 4..32 (28 gives 1.05M parameters); weights He-uniform from a
  * counter-based generator keyed by seed, head and biases zero. */
 typedef struct lbms_unet lbms_unet;

@@ -156,32 +156,75 @@ bool umma_gemm_supported(const void* A, int lda, const void* B, int ldb, int M, 
 cudaError_t umma_gemm_tn(const void* A, int lda, const void* B, int ldb, float* P, int M, int N, int K, int S,
                          unsigned int* err, cudaStream_t st);
 
-// Tap table of the 3-D U-Net's convolutions on the tcgen05 kernel: per tap
-// t = 9 (dz + 1) + 3 (dy + 1) + (dx + 1) a row offset in the zero-halo layout
-// of the activations.  umma_conv_gemm: P[r][n] = sum_t sum_c x[r + off[t]][c]
-// W[n][t C + c] over rows r of x [rows][C] (C = 64 per_tap), W [N][27 C].
-// umma_wgrad_gemm: P[z][t C + c][n] = sum_{r in chunk z}
-// xT[t % 3][c][r + off[t]] dzT[n][r] with xT[j] [C][rows], dzT [N][rows]
-// (per_tap = C, a multiple of 64; N a multiple of 64; each off a multiple of
-// 8).  Both read zeros outside their operands' extents.
-struct ConvTaps {
-    int per_tap = 1;
-    int off[27] = {};
+// Products of the 3-D U-Net (lbms_conv.cu).  Activations are BF16 rows
+// [row][C] of a zero-halo layout: volumes of X x Y x Z voxels in Xp x Yp x Zp
+// rows each, R rows in all.
+struct RowLayout {
+    int X = 0, Y = 0, Z = 0, Xp = 1, Yp = 1, Zp = 1;
+    long long R = 0;
 };
-// Optional epilogue of umma_conv_gemm: instead of FP32 P, out[r][n] =
-// BF16(relu(P[r][n] + bias[n])) on the interior rows of the zero-halo layout
-// (volumes of X x Y x Z voxels in Xp x Yp x Zp rows, R rows in all) and 0 on
-// every other row.
+
+// What becomes of the product's FP32 accumulators acc[r][n] (kept in TMEM):
+enum ConvOut {
+    kOutRelu,       // out[r][n] = BF16(relu(acc + bias[n])) on interior rows, 0 elsewhere; with cat, the
+                    //   first w columns also to cat[r][cat_off + n], and 0 to all of cat[r] elsewhere
+    kOutReluBack,   // out[r][n] = BF16(act[r][n] > 0 ? acc : 0), gb[n] += the column sums (before rounding)
+    kOutStore,      // P[r][n] = acc
+    kOutSplit,      // gradient of a concatenation of two w-wide halves, interior rows: columns [0, w) as BF16 to
+                    //   G[parent][t Cg + n] of the coarser layout (t = 4 dz + 2 dy + dx) and their sums to gb[n];
+                    //   columns [w, 2 w) to P[r][n - w] (stride Cg), which is 0 on other rows
+    kOutUp,         // transposed 2x2x2 convolution: column t Cg + n of an interior row, plus bias[n], to the row's
+                    //   child t of the finer layout, cat[child][n] (n < w)
+    kOutHead        // Y = acc + bias (3 columns): Y[r][4] if given; against T [r][4] = (targets, mask), if given,
+                    //   out[r][n] = BF16(2 inv_n (Y - T) mask) (0 for n >= 3), its column sums into gb and
+                    //   inv_n sum((Y - T)^2 mask^2) into loss
+};
 struct ConvEpilogue {
     const float* bias = nullptr;
     void* out = nullptr;          // BF16 [rows][N]
-    int X = 0, Y = 0, Z = 0, Xp = 0, Yp = 0, Zp = 0;
-    long long R = 0;
+    const void* act = nullptr;    // BF16 [rows][N]
+    void* cat = nullptr;          // BF16 [rows][cat_ld]
+    int cat_ld = 0, cat_off = 0, w = 0;
+    void* G = nullptr;            // BF16 [coarse rows][8 Cg]
+    int Cg = 0;
+    float* P = nullptr;
+    float* gb = nullptr;
+    const float* T = nullptr;
+    float* Y = nullptr;
+    double* loss = nullptr;
+    float inv_n = 0.0f;
+    RowLayout g;                  // the product's rows
+    RowLayout other;              // kOutSplit: the coarser layout; kOutUp: the finer one
 };
-cudaError_t umma_conv_gemm(const void* x, int rows, int C, const void* W, int N, const ConvTaps& taps, float* P,
-                           unsigned int* err, cudaStream_t st, const ConvEpilogue* ep = nullptr);
-cudaError_t umma_wgrad_gemm(const void* dzT, int N, const void* const xT[3], int C, int rows, int S,
-                            const ConvTaps& taps, float* P, unsigned int* err, cudaStream_t st);
+
+// acc[r][n] = sum_t sum_c x[r + off[t]][c] W[n][t C + c] over x [rows][C]
+// (zeros outside) and W [N][taps C]: a 3x3x3 convolution or its input
+// gradient (taps = 27; the three offsets of a (dz, dy) row consecutive) or a
+// plain product (taps = 1, off[0] = 0).  *err is raised if a wait in the
+// kernel timed out.  cudaErrorInvalidValue for shapes that are not built.
+struct ConvJob {
+    const void* x = nullptr;
+    const void* W = nullptr;
+    int rows = 0, C = 0, N = 0, taps = 27;
+    int off[27] = {};
+    ConvOut kind = kOutRelu;
+    ConvEpilogue ep;
+};
+cudaError_t conv_init();
+cudaError_t umma_conv(const ConvJob& j, unsigned int* err, cudaStream_t st);
+
+// P[z][t C + c][n] = sum over the rows r of chunk z of x[r + off[t]][c]
+// dz[r][n] (taps = 27, off[3 g + d] = off[3 g] + d), or P[z][c][n] with
+// taps = 1; x [rows][C], dz [rows][N], S chunks of rows / S (a multiple of 64)
+// rows each.
+struct WgradJob {
+    const void* x = nullptr;
+    const void* dz = nullptr;
+    int rows = 0, C = 0, N = 0, S = 1, taps = 27;
+    int off[27] = {};
+    float* P = nullptr;
+};
+cudaError_t umma_wgrad(const WgradJob& j, unsigned int* err, cudaStream_t st);
 
 // Read-only view of one case of a handle (for the warm-start network).
 struct CaseView {

@@ -3,31 +3,29 @@
 // tcgen05 kernels of lbms_umma.cu.  Included at the end of lbms_net.cu, whose
 // feature builder, split-K sum, Adam and weight-cast kernels it shares.
 //
-// Layout.  Activations are channels-last BF16 rows [row][C] (C a multiple
-// of 64, the real channels first, zeros after).  Each volume of X x Y x Z
-// voxels is stored with a zero halo of one voxel per side, in Xp x Yp x Zp
-// rows (Xp = X + 2 rounded up to a multiple of 8, Yp = Y + 2, Zp = Z + 2),
-// volumes one after the other; the row count is padded to a multiple of 64 S
-// (S chunks of the reductions over rows).  The neighbour of a voxel at tap
-// (dz, dy, dx) is then off = (dz Yp + dy) Xp + dx rows away, so a 3x3x3
-// convolution is an implicit GEMM on the tensor cores: the A tile of each
-// tap is the activation matrix read at a shifted row (umma_conv_kernel,
-// whose epilogue also adds the bias, applies ReLU and the zero halo and
-// stores BF16).  Its input gradient is the same with the flipped weights
-// and negated offsets, its weight gradient a product over rows against
-// three shifted transposed copies of the input (load mode 2 of
-// umma_gemm_kernel).  Every kernel that writes an activation writes all its
-// rows, zeros outside the volumes, so the halo reads as zero padding
-// whatever batch used the buffers before; an input gradient is masked the
-// same way where its reader needs it (unet_backward says which).  The
-// 2x2x2 transposed convolution of the decoder is one product whose 8 C
-// columns go to the 8 children of each voxel; max pooling keeps the index
-// of the first maximum.
+// Layout.  Activations are channels-last BF16 rows [row][C] (C = 32, 64 or
+// 128 at the three levels, the smallest that holds the real channels; the
+// real channels first, zeros after).  Each volume of X x Y x Z voxels is
+// stored with a zero halo of one voxel per side, in Xp x Yp x Zp rows (Xp =
+// X + 2 rounded up to a multiple of 8, Yp = Y + 2, Zp = Z + 2), volumes one
+// after the other; the row count is padded to a multiple of 64 S (S chunks of
+// the reductions over rows).  The neighbour of a voxel at tap (dz, dy, dx) is
+// then off = (dz Yp + dy) Xp + dx rows away, so a 3x3x3 convolution is an
+// implicit GEMM on the tensor cores (lbms_conv.cu).  What follows a product
+// is done on its accumulators: bias, ReLU, zero halo and the copy into the
+// concatenation's buffer (forward); the ReLU mask of the next layer down, its
+// BF16 gradient and the bias-gradient sums (backward); the split of a
+// concatenation's gradient; the transposed convolution's scatter to the 8
+// children of a voxel; the head's loss.  Weight gradients are products over
+// rows that read both operands as they lie in memory.  Every kernel that
+// writes an activation or a gradient writes all its rows, zeros outside the
+// volumes, so the halo reads as zero padding whatever batch used the buffers
+// before (the gathered gradients G are cleared when the layout changes).
 namespace {
 
-constexpr int kUInC = 64;      // stored input channels: the 16 feature columns, the fluid mask, zeros
+constexpr int kUInC = 32;      // stored input channels: the 16 feature columns, the fluid mask, zeros
 constexpr int kUInReal = 17;
-constexpr int kUOutC = 64;     // stored output channels of the 1x1 head (3 used)
+constexpr int kUOutC = 32;     // stored output channels of the 1x1 head (3 used)
 constexpr int kULayers = 13;
 
 // Layout of one resolution level of a batch (all row counts below 2^31).
@@ -61,199 +59,126 @@ __device__ __forceinline__ int64_t voxel_row(const Geo& g, int b, int x, int y, 
 __device__ __forceinline__ int64_t warp_id() { return ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
 __device__ __forceinline__ int64_t warp_count() { return ((int64_t)gridDim.x * blockDim.x) >> 5; }
 
-// dst[r][c] = P[r][c] on interior rows, 0 elsewhere (FP32 gradients).
-__global__ void mask_rows_kernel(const float* __restrict__ P, Geo g, int C, float* __restrict__ dst) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp_id(); r < g.Rp; r += warp_count()) {
-        int x, y, z, b;
-        const bool in = row_voxel(g, r, x, y, z, b);
-        for (int c = lane; c < C; c += 32) dst[r * C + c] = in ? P[r * C + c] : 0.0f;
-    }
-}
-
 // 2x2x2 max pooling from level `hi` to level `lo` (C channels): every row
 // of lo, the maximum of the 8 children and the child (dz 4 + dy 2 + dx) of
-// the first maximum on interior rows, 0 elsewhere.
-__global__ void pool_rows_kernel(const bf16* __restrict__ x, Geo hi, Geo lo, int C, bf16* __restrict__ y,
-                                 uint8_t* __restrict__ arg) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp_id(); r < lo.Rp; r += warp_count()) {
+// the first maximum on interior rows, 0 elsewhere.  A thread takes 8 channels
+// of a row (16-byte loads).
+__global__ void __launch_bounds__(256) pool_rows_kernel(const bf16* __restrict__ x, Geo hi, Geo lo, int C,
+                                                        bf16* __restrict__ y, uint8_t* __restrict__ arg) {
+    const int per = C / 8;
+    const int64_t n = lo.Rp * per;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = e / per;
+        const int c = (int)(e - r * per) * 8;
         int xl, yl, zl, b;
         const bool in = row_voxel(lo, r, xl, yl, zl, b);
-        const int64_t c0 = in ? voxel_row(hi, b, 2 * xl, 2 * yl, 2 * zl) : 0;
-        for (int c = lane; c < C; c += 32) {
-            float best = 0.0f;
-            int bi = 0;
-            if (in) {
-                best = -3.0e38f;
-                for (int t = 0; t < 8; ++t) {
-                    const int64_t w = c0 + ((int64_t)(t >> 2) * hi.Yp + ((t >> 1) & 1)) * hi.Xp + (t & 1);
-                    const float v = __bfloat162float(x[w * C + c]);
-                    if (v > best) {
-                        best = v;
-                        bi = t;
+        __align__(16) bf16 best[8];
+        __align__(8) uint8_t at[8];
+        for (int q = 0; q < 8; ++q) {
+            best[q] = __float2bfloat16_rn(0.0f);
+            at[q] = 0;
+        }
+        if (in) {
+            const int64_t c0 = voxel_row(hi, b, 2 * xl, 2 * yl, 2 * zl);
+            float m[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int64_t w = c0 + ((int64_t)(t >> 2) * hi.Yp + ((t >> 1) & 1)) * hi.Xp + (t & 1);
+                __align__(16) bf16 v[8];
+                *reinterpret_cast<uint4*>(v) = __ldg(reinterpret_cast<const uint4*>(x + w * C + c));
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float f = __bfloat162float(v[q]);
+                    if (t == 0 || f > m[q]) {
+                        m[q] = f;
+                        best[q] = v[q];
+                        at[q] = (uint8_t)t;
                     }
                 }
             }
-            y[r * C + c] = __float2bfloat16_rn(best);
-            arg[r * C + c] = (uint8_t)bi;
         }
+        *reinterpret_cast<uint4*>(y + r * C + c) = *reinterpret_cast<const uint4*>(best);
+        *reinterpret_cast<uint2*>(arg + r * C + c) = *reinterpret_cast<const uint2*>(at);
     }
 }
 
-// Gradient of the pooling: dx[r][c] += dp[parent][c] on the interior rows
-// of hi that hold their parent's maximum.
-__global__ void pool_back_rows_kernel(const float* __restrict__ dp, const uint8_t* __restrict__ arg, Geo hi, Geo lo,
-                                      int C, float* __restrict__ dx) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp_id(); r < hi.R; r += warp_count()) {
-        int x, y, z, b;
-        if (!row_voxel(hi, r, x, y, z, b)) continue;
-        const int64_t p = voxel_row(lo, b, x >> 1, y >> 1, z >> 1);
-        const int t = (z & 1) * 4 + (y & 1) * 2 + (x & 1);
-        for (int c = lane; c < C; c += 32)
-            if (arg[p * C + c] == t) dx[r * C + c] += dp[p * C + c];
-    }
-}
-
-// Transposed 2x2x2 convolution, stride 2: every row of hi, y[r][c] =
-// P[parent][t C + c] + b[c] with t the row's child index, on interior rows;
-// 0 elsewhere.
-__global__ void up_rows_kernel(const float* __restrict__ P, const float* __restrict__ bias, Geo lo, Geo hi, int C,
-                               bf16* __restrict__ y) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp_id(); r < hi.Rp; r += warp_count()) {
-        int x, yy, z, b;
-        const bool in = row_voxel(hi, r, x, yy, z, b);
-        const int64_t p = in ? voxel_row(lo, b, x >> 1, yy >> 1, z >> 1) : 0;
-        const int t = in ? (z & 1) * 4 + (yy & 1) * 2 + (x & 1) : 0;
-        for (int c = lane; c < C; c += 32)
-            y[r * C + c] = __float2bfloat16_rn(in ? P[p * 8 * C + t * C + c] + bias[c] : 0.0f);
-    }
-}
-
-// Gradient of up_rows_kernel: every row of lo, G[r][t C + c] = dy[child t][c]
-// (BF16) on interior rows, 0 elsewhere.
-__global__ void upgather_rows_kernel(const float* __restrict__ dy, Geo lo, Geo hi, int C, bf16* __restrict__ G) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = warp_id(); r < lo.Rp; r += warp_count()) {
-        int xl, yl, zl, b;
-        const bool in = row_voxel(lo, r, xl, yl, zl, b);
-        const int64_t c0 = in ? voxel_row(hi, b, 2 * xl, 2 * yl, 2 * zl) : 0;
-        for (int e = lane; e < 8 * C; e += 32) {
-            float g = 0.0f;
-            if (in) {
-                const int t = e / C, c = e - t * C;
-                g = dy[(c0 + ((int64_t)(t >> 2) * hi.Yp + ((t >> 1) & 1)) * hi.Xp + (t & 1)) * C + c];
-            }
-            G[r * 8 * C + e] = __float2bfloat16_rn(g);
-        }
-    }
-}
-
-// out[r] = (a[r][0:na], b[r][0:nb], zeros) with Co stored channels, R rows.
-__global__ void concat_kernel(const bf16* __restrict__ a, int Ca, int na, const bf16* __restrict__ bsrc, int Cb, int nb,
-                              int64_t R, int Co, bf16* __restrict__ out) {
-    const int64_t n = R * Co;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / Co;
-        const int c = (int)(e % Co);
-        out[e] = c < na ? a[r * Ca + c] : c < na + nb ? bsrc[r * Cb + (c - na)] : __float2bfloat16_rn(0.0f);
-    }
-}
-
-// The gradient of concat_kernel: da[r][c] = d[r][c] (c < na, else 0) and
-// db[r][c] = d[r][na + c] (c < nb, else 0), with d stored Cd wide.
-__global__ void split_kernel(const float* __restrict__ d, int Cd, int na, int nb, int Ca, int Cb, int64_t R,
-                             float* __restrict__ da, float* __restrict__ db) {
-    const int Cm = Ca > Cb ? Ca : Cb;
-    const int64_t n = R * Cm;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / Cm;
-        const int c = (int)(e % Cm);
-        if (c < Ca) da[r * Ca + c] = c < na ? d[r * Cd + c] : 0.0f;
-        if (c < Cb) db[r * Cb + c] = c < nb ? d[r * Cd + na + c] : 0.0f;
-    }
-}
-
-// Column sums of a FP32 [R][C] added into acc (R a multiple of 32).
-__global__ void colsum_kernel(const float* __restrict__ d, int64_t R, int C, float* __restrict__ acc) {
-    const int64_t r0 = (int64_t)blockIdx.x * 32;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float s = 0.0f;
-        for (int64_t r = r0; r < r0 + 32; ++r) s += d[r * C + c];
-        atomicAdd(&acc[c], s);
-    }
-}
-
-// ncopy transposed copies of in [R][C]: out[j][c][r] = in[r + j + shift0][c]
-// (0 where that row is outside [0, R)); R and C multiples of 64.  A block of
-// 256 threads reads 64 + ncopy - 1 rows x 64 channels once (16-byte loads)
-// and writes the 64 x 64 tiles of every copy (16-byte stores, 8 threads per
-// 128-byte output row).  The shared tile's rows are 33 words apart, so the
-// 8 rows a warp reads at once fall in 2 ways of the banks.
-__global__ void __launch_bounds__(256) transpose_copies_kernel(const bf16* __restrict__ in, bf16* __restrict__ out,
-                                                               int64_t R, int C, int ncopy, int shift0) {
-    __shared__ __align__(16) bf16 tile[66][66];
-    const int64_t r0 = (int64_t)blockIdx.x * 64;
-    const int c0 = blockIdx.y * 64;
-    const int nrows = 64 + ncopy - 1;
-    for (int e = threadIdx.x; e < nrows * 8; e += 256) {
-        const int i = e >> 3, q = (e & 7) * 8;
-        const int64_t rs = r0 + i + shift0;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (rs >= 0 && rs < R) v = *reinterpret_cast<const uint4*>(in + rs * C + c0 + q);
-        uint32_t* d = reinterpret_cast<uint32_t*>(&tile[i][q]);
-        d[0] = v.x;
-        d[1] = v.y;
-        d[2] = v.z;
-        d[3] = v.w;
-    }
-    __syncthreads();
-    for (int j = 0; j < ncopy; ++j) {
-        bf16* o = out + (size_t)j * C * R;
-        for (int e = threadIdx.x; e < 64 * 8; e += 256) {
-            const int c = e >> 3, q = (e & 7) * 8;
-            __align__(16) bf16 v[8];
+// The gradient through a pooling, a skip connection and the ReLU below both:
+// dz[r][c] = BF16(act > 0 ? skip[r][c] + (dp of the parent where r holds its
+// maximum) : 0) on every row of hi (act is 0 outside the volumes), and the
+// column sums of the unrounded values added into gb.  C is 32 or 64; a thread
+// takes 8 channels of a row.  Bound by memory: 9 C bytes a row read (skip
+// FP32, act, arg of the parent) and 2 C written.
+__global__ void __launch_bounds__(256) pool_relu_back_kernel(const float* __restrict__ dp, const uint8_t* __restrict__ arg,
+                                                             const float* __restrict__ skip,
+                                                             const bf16* __restrict__ act, Geo hi, Geo lo, int C,
+                                                             bf16* __restrict__ dz, float* __restrict__ gb) {
+    __shared__ float part[256 * 8];
+    const int per = C / 8;
+    const int c = (threadIdx.x % per) * 8;
+    float sum[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = tile[q + k + j][c];
-            *reinterpret_cast<uint4*>(o + (int64_t)(c0 + c) * R + r0 + q) = *reinterpret_cast<const uint4*>(v);
+    for (int q = 0; q < 8; ++q) sum[q] = 0.0f;
+    const int rows = 256 / per;
+    for (int64_t r = (int64_t)blockIdx.x * rows + threadIdx.x / per; r < hi.Rp; r += (int64_t)gridDim.x * rows) {
+        const uint4 av = __ldg(reinterpret_cast<const uint4*>(act + r * C + c));
+        __align__(16) bf16 o[8];
+        if (av.x | av.y | av.z | av.w) {
+            __align__(16) bf16 a[8];
+            *reinterpret_cast<uint4*>(a) = av;
+            float v[8];
+            *reinterpret_cast<float4*>(v) = __ldg(reinterpret_cast<const float4*>(skip + r * C + c));
+            *reinterpret_cast<float4*>(v + 4) = __ldg(reinterpret_cast<const float4*>(skip + r * C + c + 4));
+            int x, y, z, b;
+            if (row_voxel(hi, r, x, y, z, b)) {
+                const int64_t p = voxel_row(lo, b, x >> 1, y >> 1, z >> 1);
+                const int t = (z & 1) * 4 + (y & 1) * 2 + (x & 1);
+                __align__(8) uint8_t at[8];
+                *reinterpret_cast<uint2*>(at) = __ldg(reinterpret_cast<const uint2*>(arg + p * C + c));
+                float d[8];
+                *reinterpret_cast<float4*>(d) = __ldg(reinterpret_cast<const float4*>(dp + p * C + c));
+                *reinterpret_cast<float4*>(d + 4) = __ldg(reinterpret_cast<const float4*>(dp + p * C + c + 4));
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (at[q] == t) v[q] += d[q];
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float w = __bfloat162float(a[q]) > 0.0f ? v[q] : 0.0f;
+                o[q] = __float2bfloat16_rn(w);
+                sum[q] += w;
+            }
+        } else {
+            *reinterpret_cast<uint4*>(o) = make_uint4(0u, 0u, 0u, 0u);
         }
+        *reinterpret_cast<uint4*>(dz + r * C + c) = *reinterpret_cast<const uint4*>(o);
     }
-}
-
-// dZ = dA * (act > 0) as BF16 [R][C] (C 64 or 128) and the column sums of
-// dZ added into gb; a block of 256 threads per 64 rows.
-__global__ void __launch_bounds__(256) relu_back_rows_kernel(const float* __restrict__ dA, const bf16* __restrict__ act,
-                                                             int64_t R, int C, bf16* __restrict__ dZ,
-                                                             float* __restrict__ gb) {
-    __shared__ float part[256];
-    const int64_t r0 = (int64_t)blockIdx.x * 64;
-    const int c = threadIdx.x % C, g = threadIdx.x / C, ng = 256 / C;
-    float s = 0.0f;
-    for (int64_t r = r0 + g; r < r0 + 64 && r < R; r += ng) {
-        const int64_t e = r * C + c;
-        const float v = __bfloat162float(act[e]) > 0.0f ? dA[e] : 0.0f;
-        dZ[e] = __float2bfloat16_rn(v);
-        s += v;
-    }
-    part[threadIdx.x] = s;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) part[threadIdx.x * 8 + q] = sum[q];
     __syncthreads();
-    if (threadIdx.x < C) {
+    if (threadIdx.x < C) {   // column threadIdx.x: threads of channel group threadIdx.x / 8
         float t = 0.0f;
-        for (int k = 0; k < ng; ++k) t += part[k * C + threadIdx.x];
+        for (int g = threadIdx.x / 8; g < 256; g += per) t += part[g * 8 + threadIdx.x % 8];
         atomicAdd(&gb[threadIdx.x], t);
     }
 }
 
-// G[o][i] = sum_z P[z][i][o] (split-K partials of a transposed product).
+// G[o][i] = sum_z P[z][i][o] (split-K partials of a transposed product), in
+// the order of z; threads walk P's order, 8 chunks in flight.
 __global__ void splitk_sum_t_kernel(const float* __restrict__ P, int S, int I, int O, float* __restrict__ G) {
     const int64_t n = (int64_t)O * I;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int o = (int)(e / I), i = (int)(e % I);
         float acc = 0.0f;
-        for (int z = 0; z < S; ++z) acc += P[(int64_t)z * n + (int64_t)i * O + o];
-        G[e] = acc;
+        int z = 0;
+        for (; z + 8 <= S; z += 8) {
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = __ldg(P + (int64_t)(z + q) * n + e);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc += v[q];
+        }
+        for (; z < S; ++z) acc += __ldg(P + (int64_t)z * n + e);
+        const int i = (int)(e / O), o = (int)(e % O);
+        G[(int64_t)o * I + i] = acc;
     }
 }
 
@@ -318,46 +243,6 @@ __global__ void unet_inputs_kernel(const bf16* __restrict__ rows, const int64_t*
     }
 }
 
-// Masked mean-square error of the head's output Y = P + b (3 used columns)
-// against T [r][4] = (3 targets, fluid mask) over R rows (a multiple of 64),
-// one block of 256 threads per 64 rows: dP (BF16, zero in the padded
-// columns), the head's bias gradient and the loss, with inv_n = 1 / (3 x
-// fluid voxels); Y[r][c] (c < 3) is kept for predictions.
-__global__ void unet_loss_kernel(const float* __restrict__ P, const float* __restrict__ b, const float* __restrict__ T,
-                                 int64_t R, float inv_n, bf16* __restrict__ dP, float* __restrict__ gb,
-                                 double* __restrict__ loss, float* __restrict__ Y) {
-    __shared__ float colsum[3];
-    __shared__ double lsum[256];
-    if (threadIdx.x < 3) colsum[threadIdx.x] = 0.0f;
-    __syncthreads();
-    double l = 0.0;
-    const int64_t r0 = (int64_t)blockIdx.x * 64;
-    for (int e = threadIdx.x; e < 64 * kUOutC; e += 256) {
-        const int64_t r = r0 + e / kUOutC;
-        const int c = e % kUOutC;
-        float g = 0.0f;
-        if (r < R && c < 3) {
-            const float y = P[r * kUOutC + c] + b[c];
-            if (Y) Y[r * 4 + c] = y;
-            if (T) {
-                const float d = (y - T[r * 4 + c]) * T[r * 4 + 3];
-                l += (double)d * d;
-                g = 2.0f * inv_n * d;
-                atomicAdd(&colsum[c], g);
-            }
-        }
-        if (r < R && dP) dP[r * kUOutC + c] = __float2bfloat16_rn(g);
-    }
-    lsum[threadIdx.x] = l;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) lsum[threadIdx.x] += lsum[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (T && threadIdx.x == 0) atomicAdd(loss, lsum[0] * (double)inv_n);
-    if (T && threadIdx.x < 3) atomicAdd(&gb[threadIdx.x], colsum[threadIdx.x]);
-}
-
 // The prediction of one case from the head's output Y [r][4] at its row
 // row[j]: X_s = profile_s(x) + Y[row][s] / 100, clamped at 1e-6 and
 // renormalised; out [3][nf] FP64.  Xp: the padded x extent (x = row mod Xp - 1).
@@ -396,13 +281,17 @@ struct lbms_unet {
     int64_t vcap = 0;            // interior voxels of one batch at most
     // activations and scratch, sized for the largest batch layout so far (grown on demand)
     int64_t cap[3] = {0, 0, 0};  // rows per level the buffers hold
-    bf16 *x0 = nullptr, *e1a = nullptr, *e1 = nullptr, *u1 = nullptr, *c1 = nullptr, *d1a = nullptr, *d1 = nullptr;
-    bf16 *p1 = nullptr, *e2a = nullptr, *e2 = nullptr, *u2 = nullptr, *c2 = nullptr, *d2a = nullptr, *d2 = nullptr;
+    bf16 *x0 = nullptr, *e1a = nullptr, *e1 = nullptr, *c1 = nullptr, *d1a = nullptr, *d1 = nullptr;
+    bf16 *p1 = nullptr, *e2a = nullptr, *e2 = nullptr, *c2 = nullptr, *d2a = nullptr, *d2 = nullptr;
     bf16 *p2 = nullptr, *e3a = nullptr, *e3 = nullptr;
     uint8_t *arg1 = nullptr, *arg2 = nullptr;
-    bf16 *dz = nullptr, *dzT = nullptr, *G = nullptr, *aT = nullptr, *xT = nullptr;
-    float *P = nullptr, *fa = nullptr, *fb = nullptr, *fc = nullptr, *fd = nullptr, *Y = nullptr, *T = nullptr;
-    size_t P_floats = 0, g_elems = 0, xT_elems = 0, f_floats = 0;
+    bf16 *za[3] = {nullptr, nullptr, nullptr}, *zb[3] = {nullptr, nullptr, nullptr};   // pre-activation gradients per level
+    bf16 *G1 = nullptr, *G2 = nullptr;            // transposed convolutions' output gradients, gathered by parent
+    float *skip0 = nullptr, *skip1 = nullptr;     // skip connections' gradients
+    float *dp1 = nullptr, *dp2 = nullptr;         // pooled activations' gradients
+    float *P = nullptr, *Y = nullptr, *T = nullptr;
+    size_t P_floats = 0;
+    int last[4] = {0, 0, 0, 0};  // B, X, Y, Z of the layout the buffers held last
     std::vector<void*> bufs;     // the grown buffers
     double* loss = nullptr;
     unsigned int* gemm_err = nullptr;
@@ -514,11 +403,7 @@ lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
     for (int l = 0; l < 3; ++l) u->cap[l] = 0;
     const size_t c0 = c[0], c1 = c[1], c2 = c[2];
     const size_t s0 = splits_for(c0), s1 = splits_for(c1), s2 = splits_for(c2);
-    u->g_elems = std::max({c0 * 64, c1 * 512, c2 * 512});
-    u->xT_elems = 3 * std::max({c0 * 64, c1 * 128, c2 * 128});
-    u->f_floats = std::max({c0 * 64, c1 * 128, c2 * 128});
-    u->P_floats = std::max({c0 * 64, c1 * 512, c2 * 512, s0 * 64 * 1728, s1 * 64 * 3456, s2 * 128 * 3456,
-                            s1 * 512 * 64, s2 * 512 * 128, s0 * 64 * 64});
+    u->P_floats = std::max({s0 * 64 * 864, s1 * 128 * 1728, s2 * 128 * 3456, s1 * 256 * 64, s2 * 512 * 128});
     bool ok = true;
     auto get = [&](size_t bytes) {
         void* p = nullptr;
@@ -531,37 +416,38 @@ lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
         return p;
     };
     auto act = [&](size_t rows, int C) { return static_cast<bf16*>(get(rows * C * sizeof(bf16))); };
+    auto f32 = [&](size_t count) { return static_cast<float*>(get(count * sizeof(float))); };
     u->x0 = act(c0, kUInC);
-    u->e1a = act(c0, 64);
-    u->e1 = act(c0, 64);
-    u->u1 = act(c0, 64);
+    u->e1a = act(c0, 32);
+    u->e1 = act(c0, 32);
     u->c1 = act(c0, 64);
-    u->d1a = act(c0, 64);
-    u->d1 = act(c0, 64);
-    u->p1 = act(c1, 64);
+    u->d1a = act(c0, 32);
+    u->d1 = act(c0, 32);
+    u->p1 = act(c1, 32);
     u->e2a = act(c1, 64);
     u->e2 = act(c1, 64);
-    u->u2 = act(c1, 64);
     u->c2 = act(c1, 128);
     u->d2a = act(c1, 64);
     u->d2 = act(c1, 64);
     u->p2 = act(c2, 64);
     u->e3a = act(c2, 128);
     u->e3 = act(c2, 128);
-    u->arg1 = static_cast<uint8_t*>(get(c1 * 64));
+    u->arg1 = static_cast<uint8_t*>(get(c1 * 32));
     u->arg2 = static_cast<uint8_t*>(get(c2 * 64));
-    u->dz = static_cast<bf16*>(get(u->g_elems * sizeof(bf16)));
-    u->dzT = static_cast<bf16*>(get(u->g_elems * sizeof(bf16)));
-    u->G = static_cast<bf16*>(get(u->g_elems * sizeof(bf16)));
-    u->aT = static_cast<bf16*>(get(u->g_elems * sizeof(bf16)));
-    u->xT = static_cast<bf16*>(get(u->xT_elems * sizeof(bf16)));
-    u->P = static_cast<float*>(get(u->P_floats * sizeof(float)));
-    u->fa = static_cast<float*>(get(u->f_floats * sizeof(float)));
-    u->fb = static_cast<float*>(get(u->f_floats * sizeof(float)));
-    u->fc = static_cast<float*>(get(u->f_floats * sizeof(float)));
-    u->fd = static_cast<float*>(get(u->f_floats * sizeof(float)));
-    u->Y = static_cast<float*>(get(c0 * 4 * sizeof(float)));
-    u->T = static_cast<float*>(get(c0 * 4 * sizeof(float)));
+    for (int l = 0; l < 3; ++l) {
+        u->za[l] = act(l == 0 ? c0 : l == 1 ? c1 : c2, 32 << l);
+        u->zb[l] = act(l == 0 ? c0 : l == 1 ? c1 : c2, 32 << l);
+    }
+    u->G1 = act(c1, 256);
+    u->G2 = act(c2, 512);
+    u->skip0 = f32(c0 * 32);
+    u->skip1 = f32(c1 * 64);
+    u->dp1 = f32(c1 * 32);
+    u->dp2 = f32(c2 * 64);
+    u->P = f32(u->P_floats);
+    u->Y = f32(c0 * 4);
+    u->T = f32(c0 * 4);
+    for (int& d : u->last) d = 0;
     if (!ok) {
         for (void* p : u->bufs) cudaFree(p);
         u->bufs.clear();
@@ -574,214 +460,230 @@ lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
 // Blocks of 256 threads for one warp per row over R rows (grid-stride beyond 152 x 16 blocks).
 int warp_grid(int64_t R) { return (int)std::max<int64_t>(1, std::min<int64_t>((R + 7) / 8, 152 * 16)); }
 
-// Tap table of a 3x3x3 convolution on layout g: row offsets sign * off(t).
-lbms::ConvTaps conv_taps(const Geo& g, int per_tap, int sign) {
-    lbms::ConvTaps t;
-    t.per_tap = per_tap;
+lbms::RowLayout layout_of(const Geo& g) {
+    lbms::RowLayout l;
+    l.X = g.X;
+    l.Y = g.Y;
+    l.Z = g.Z;
+    l.Xp = g.Xp;
+    l.Yp = g.Yp;
+    l.Zp = g.Zp;
+    l.R = g.R;
+    return l;
+}
+
+// Row offsets of the 27 taps on layout g, times sign.
+void set_taps(const Geo& g, int sign, int (&off)[27]) {
     for (int k = 0; k < 27; ++k) {
         const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-        t.off[k] = sign * ((dz * g.Yp + dy) * g.Xp + dx);
+        off[k] = sign * ((dz * g.Yp + dy) * g.Xp + dx);
     }
-    return t;
 }
 
-// Tap table of the weight gradient: the shift (dz Yp + dy) Xp of the copy dx + 1.
-lbms::ConvTaps wgrad_taps(const Geo& g, int C) {
-    lbms::ConvTaps t;
-    t.per_tap = C;
-    for (int k = 0; k < 27; ++k) {
-        const int dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-        t.off[k] = (dz * g.Yp + dy) * g.Xp;
-    }
-    return t;
+// A product over the rows of g: x [Rp][C] with the layer's weights W [N][taps C].
+lbms::ConvJob conv_job(const Geo& g, const bf16* x, int C, const bf16* W, int N, int taps, int sign,
+                       lbms::ConvOut kind) {
+    lbms::ConvJob j;
+    j.x = x;
+    j.W = W;
+    j.rows = (int)g.Rp;
+    j.C = C;
+    j.N = N;
+    j.taps = taps;
+    if (taps == 27) set_taps(g, sign, j.off);
+    j.kind = kind;
+    j.ep.g = layout_of(g);
+    return j;
 }
 
-// P[z] = A . B^T on the tcgen05 tensor cores (lbms_umma.cu), plain operands.
-lbms_status ugemm(lbms_unet* u, const bf16* A, int64_t lda, const bf16* B, int64_t ldb, int64_t M, int N, int64_t K,
-                  int S) {
-    if ((size_t)S * M * N > u->P_floats || M > INT32_MAX || K > INT32_MAX || lda > INT32_MAX || ldb > INT32_MAX ||
-        !lbms::umma_gemm_supported(A, (int)lda, B, (int)ldb, (int)M, N, (int)K, S))
-        return ufail(u, LBMS_EINVAL, "U-Net product %lld x %d x %lld (split %d) not supported", (long long)M, N,
-                     (long long)K, S);
-    UCK(lbms::umma_gemm_tn(A, (int)lda, B, (int)ldb, u->P, (int)M, N, (int)K, S, u->gemm_err, 0), "tensor-core gemm");
+lbms_status run_conv(lbms_unet* u, const lbms::ConvJob& j, const char* what) {
+    UCK(lbms::umma_conv(j, u->gemm_err, 0), what);
     ++u->tcgen05_calls;
-    return LBMS_OK;
-}
-
-// ncopy transposed copies out[j][c][r] = in[r + j + shift0][c] over R rows (zero outside).
-lbms_status transpose_rows(lbms_unet* u, const bf16* in, bf16* out, int64_t R, int C, int ncopy, int shift0,
-                           size_t cap) {
-    if ((size_t)ncopy * R * C > cap || R % 64 || C % 64)
-        return ufail(u, LBMS_EINVAL, "U-Net transpose %lld x %d not supported", (long long)R, C);
-    transpose_copies_kernel<<<dim3((unsigned)(R / 64), C / 64), 256>>>(in, out, R, C, ncopy, shift0);
-    UCK(cudaGetLastError(), "transpose");
-    return LBMS_OK;
-}
-
-lbms_status mask_rows(lbms_unet* u, const Geo& g, int C, float* dst) {
-    if ((size_t)g.Rp * C > u->f_floats) return ufail(u, LBMS_EINVAL, "U-Net gradient %lld x %d too large",
-                                                      (long long)g.Rp, C);
-    mask_rows_kernel<<<warp_grid(g.Rp), 256>>>(u->P, g, C, dst);
-    UCK(cudaGetLastError(), "gradient rows");
     return LBMS_OK;
 }
 
 // ------------------------------------------------------ layer passes
-// relu(conv3(x) + b) -> out (kind 3: implicit GEMM), or the 1x1 head's product (left in P, out unused)
-lbms_status conv_fwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const Geo& g, bf16* out) {
-    if (l.kind == 3) {
-        // bias, ReLU, the zero halo and the BF16 store happen in the GEMM's epilogue
-        const lbms::ConvTaps tp = conv_taps(g, l.ci_s / 64, 1);
-        lbms::ConvEpilogue ep;
-        ep.bias = l.b;
-        ep.out = out;
-        ep.X = g.X;
-        ep.Y = g.Y;
-        ep.Z = g.Z;
-        ep.Xp = g.Xp;
-        ep.Yp = g.Yp;
-        ep.Zp = g.Zp;
-        ep.R = g.R;
-        if (!out) return ufail(u, LBMS_EINVAL, "U-Net convolution without an output");
-        UCK(lbms::umma_conv_gemm(x, (int)g.Rp, l.ci_s, l.Wb, l.co_s, tp, u->P, u->gemm_err, 0, &ep), "convolution");
-        ++u->tcgen05_calls;
-        return LBMS_OK;
-    }
-    return ugemm(u, x, l.ci_s, l.Wb, l.K, g.Rp, l.rows, l.K, 1);   // the 1x1 head: P [Rp][64]
+// relu(conv3(x) + b) -> out; with cat, the first w columns also to cat[r][off ...] (stride ld)
+lbms_status conv_fwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const Geo& g, bf16* out,
+                     bf16* cat = nullptr, int ld = 0, int off = 0, int w = 0) {
+    lbms::ConvJob j = conv_job(g, x, l.ci_s, l.Wb, l.co_s, 27, 1, lbms::kOutRelu);
+    j.ep.bias = l.b;
+    j.ep.out = out;
+    j.ep.cat = cat;
+    j.ep.cat_ld = ld;
+    j.ep.cat_off = off;
+    j.ep.w = w;
+    return run_conv(u, j, "convolution");
 }
 
-// transposed 2x2x2 convolution of x [lo.Rp][ci_s] -> y [hi.Rp][co_s]
-lbms_status up_fwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const Geo& lo, const Geo& hi, bf16* y) {
-    UST(ugemm(u, x, l.ci_s, l.Wb, l.K, lo.Rp, l.rows, l.K, 1));
-    up_rows_kernel<<<warp_grid(hi.Rp), 256>>>(u->P, l.b, lo, hi, l.co_s, y);
-    UCK(cudaGetLastError(), "up convolution");
+// transposed 2x2x2 convolution of x [lo.Rp][ci_s] into the first w columns of cat [hi.Rp][2 co_s]
+lbms_status up_fwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const Geo& lo, const Geo& hi, bf16* cat) {
+    lbms::ConvJob j = conv_job(lo, x, l.ci_s, l.Wb, l.rows, 1, 1, lbms::kOutUp);
+    j.ep.bias = l.b;
+    j.ep.cat = cat;
+    j.ep.cat_ld = 2 * l.co_s;
+    j.ep.Cg = l.co_s;
+    j.ep.w = l.co;
+    j.ep.other = layout_of(hi);
+    return run_conv(u, j, "up convolution");
+}
+
+// Weight gradient from the pre-activation gradient dz (kind 3: dz [Rp][co_s]
+// against the taps of x [Rp][ci_s]; kinds 1, 2: of [rows] = dz's or G's columns)
+lbms_status layer_wgrad(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const bf16* dz, const Geo& g) {
+    if ((size_t)g.S * l.rows * l.K > u->P_floats) return ufail(u, LBMS_EINVAL, "U-Net weight gradient too large");
+    lbms::WgradJob j;
+    j.rows = (int)g.Rp;
+    j.S = g.S;
+    j.P = u->P;
+    const int64_t n = (int64_t)l.rows * l.K;
+    if (l.kind == 3) {   // P [S][27 ci_s][co_s]
+        j.x = x;
+        j.C = l.ci_s;
+        j.dz = dz;
+        j.N = l.co_s;
+        set_taps(g, 1, j.off);
+    } else {             // P [S][rows][K]
+        j.x = dz;
+        j.C = l.rows;
+        j.dz = x;
+        j.N = l.K;
+        j.taps = 1;
+    }
+    UCK(lbms::umma_wgrad(j, u->gemm_err, 0), "weight gradient");
+    ++u->tcgen05_calls;
+    if (l.kind == 3)
+        splitk_sum_t_kernel<<<grid_for(n), 256>>>(u->P, g.S, l.K, l.co_s, l.g);
+    else
+        splitk_sum_kernel<<<grid_for(n), 256>>>(u->P, g.S, n, l.g);
+    UCK(cudaGetLastError(), "split-k sum");
     return LBMS_OK;
 }
 
-// Backward pass of a 3x3x3 convolution + ReLU from dA (the gradient of its
-// output a; it may be u->P): weight and bias gradients and, with dx, the
-// input gradient [Rp][ci_s]: masked to zero outside the volumes into dx, or
-// left unmasked in u->P when dx is u->P (for a ReLU backward or a pooling
-// gradient next, which read only what the zero halo of their activations
-// lets through).
-lbms_status conv_bwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const bf16* a, const float* dA,
-                     const Geo& g, float* dx) {
-    relu_back_rows_kernel<<<(unsigned)(g.Rp / 64), 256>>>(dA, a, g.Rp, l.co_s, u->dz, l.gb);
-    UCK(cudaGetLastError(), "relu backward");
-    UST(transpose_rows(u, u->dz, u->dzT, g.Rp, l.co_s, 1, 0, u->g_elems));
-    UST(transpose_rows(u, x, u->xT, g.Rp, l.ci_s, 3, -1, u->xT_elems));
-    const void* xT[3];
-    for (int j = 0; j < 3; ++j) xT[j] = u->xT + (size_t)j * l.ci_s * g.Rp;
-    if ((size_t)g.S * l.co_s * l.K > u->P_floats) return ufail(u, LBMS_EINVAL, "U-Net weight gradient too large");
-    const lbms::ConvTaps tw = wgrad_taps(g, l.ci_s);
-    UCK(lbms::umma_wgrad_gemm(u->dzT, l.co_s, xT, l.ci_s, (int)g.Rp, g.S, tw, u->P, u->gemm_err, 0),
-        "weight gradient");
-    ++u->tcgen05_calls;
-    splitk_sum_t_kernel<<<grid_for((int64_t)l.co_s * l.K), 256>>>(u->P, g.S, l.K, l.co_s, l.g);
-    UCK(cudaGetLastError(), "split-k sum");
-    if (!dx) return LBMS_OK;
-    if ((size_t)g.Rp * l.ci_s > u->P_floats) return ufail(u, LBMS_EINVAL, "U-Net input gradient too large");
-    const lbms::ConvTaps tn = conv_taps(g, l.co_s / 64, -1);
-    UCK(lbms::umma_conv_gemm(u->dz, (int)g.Rp, l.co_s, l.Wt, l.ci_s, tn, u->P, u->gemm_err, 0), "input gradient");
-    ++u->tcgen05_calls;
-    return dx == u->P ? LBMS_OK : mask_rows(u, g, l.ci_s, dx);
+// The gradient of a layer's input through the ReLU of the layer `prev` that
+// made it (activation act): prev's pre-activation gradient into out, its bias
+// gradient into prev.gb.
+lbms_status dgrad_relu(lbms_unet* u, const lbms_unet::Layer& l, const bf16* dz, const Geo& g, const bf16* act,
+                       const lbms_unet::Layer& prev, bf16* out) {
+    const bool conv = l.kind == 3;
+    lbms::ConvJob j = conv_job(g, dz, conv ? l.co_s : l.rows, l.Wt, l.ci_s, conv ? 27 : 1, -1, lbms::kOutReluBack);
+    j.ep.act = act;
+    j.ep.out = out;
+    j.ep.gb = prev.gb;
+    return run_conv(u, j, "input gradient");
 }
 
-// Backward pass of the transposed convolution from dy [hi.Rp][co_s]: weight
-// and bias gradients and the gradient of its input [lo.Rp][ci_s].
-lbms_status up_bwd(lbms_unet* u, const lbms_unet::Layer& l, const bf16* x, const float* dy, const Geo& lo,
-                   const Geo& hi, float* dx) {
-    colsum_kernel<<<(unsigned)(hi.Rp / 32), 128>>>(dy, hi.Rp, l.co_s, l.gb);
-    UCK(cudaGetLastError(), "bias gradient");
-    if ((size_t)lo.Rp * l.rows > u->g_elems) return ufail(u, LBMS_EINVAL, "U-Net gather too large");
-    upgather_rows_kernel<<<warp_grid(lo.Rp), 256>>>(dy, lo, hi, l.co_s, u->G);
-    UCK(cudaGetLastError(), "up gather");
-    UST(transpose_rows(u, u->G, u->dzT, lo.Rp, l.rows, 1, 0, u->g_elems));
-    UST(transpose_rows(u, x, u->aT, lo.Rp, l.ci_s, 1, 0, u->g_elems));
-    UST(ugemm(u, u->dzT, lo.Rp, u->aT, lo.Rp, l.rows, l.ci_s, lo.Rp, lo.S));
-    splitk_sum_kernel<<<grid_for((int64_t)l.rows * l.K), 256>>>(u->P, lo.S, (int64_t)l.rows * l.K, l.g);
-    UCK(cudaGetLastError(), "split-k sum");
-    UST(ugemm(u, u->G, l.rows, l.Wt, l.rows, lo.Rp, l.ci_s, l.rows, 1));
-    return dx == u->P ? LBMS_OK : mask_rows(u, lo, l.ci_s, dx);
+// The gradient of a concatenation (up-sampled half, skip half) read by l: the
+// first gathered into G for the transposed convolution `up`, the second into
+// skip.
+lbms_status dgrad_split(lbms_unet* u, const lbms_unet::Layer& l, const bf16* dz, const Geo& g, const Geo& lo,
+                        const lbms_unet::Layer& up, bf16* G, float* skip) {
+    lbms::ConvJob j = conv_job(g, dz, l.co_s, l.Wt, l.ci_s, 27, -1, lbms::kOutSplit);
+    j.ep.G = G;
+    j.ep.Cg = up.co_s;
+    j.ep.w = up.co;
+    j.ep.gb = up.gb;
+    j.ep.P = skip;
+    j.ep.other = layout_of(lo);
+    return run_conv(u, j, "input gradient");
+}
+
+// The gradient of a pooled activation, FP32 [Rp][ci_s].
+lbms_status dgrad_store(lbms_unet* u, const lbms_unet::Layer& l, const bf16* dz, const Geo& g, float* out) {
+    lbms::ConvJob j = conv_job(g, dz, l.co_s, l.Wt, l.ci_s, 27, -1, lbms::kOutStore);
+    j.ep.P = out;
+    return run_conv(u, j, "input gradient");
 }
 
 // ------------------------------------------------------ network passes
-// Forward pass of a batch already in u->x0 (layout v.g[0]); the head's
-// product (without its bias) is left in u->P [Rp][64].
-lbms_status unet_forward(lbms_unet* u, const Levels& v) {
+// Forward pass of a batch already in u->x0 (layout v.g[0]).  With `train`,
+// against u->T: the loss, the head's output gradient (za[0]) and its bias
+// gradient; otherwise the head's output in u->Y [Rp][4].
+lbms_status unet_forward(lbms_unet* u, const Levels& v, bool train, float inv_n) {
     const Geo &g0 = v.g[0], &g1 = v.g[1], &g2 = v.g[2];
     const int w = u->width;
     auto& L = u->L;
+    if (u->last[0] != g0.B || u->last[1] != g0.X || u->last[2] != g0.Y || u->last[3] != g0.Z) {
+        UCK(cudaMemsetAsync(u->G1, 0, (size_t)u->cap[1] * 256 * sizeof(bf16), 0), "clear gradients");
+        UCK(cudaMemsetAsync(u->G2, 0, (size_t)u->cap[2] * 512 * sizeof(bf16), 0), "clear gradients");
+        u->last[0] = g0.B;
+        u->last[1] = g0.X;
+        u->last[2] = g0.Y;
+        u->last[3] = g0.Z;
+    }
     UST(conv_fwd(u, L[0], u->x0, g0, u->e1a));
-    UST(conv_fwd(u, L[1], u->e1a, g0, u->e1));
-    pool_rows_kernel<<<warp_grid(g1.Rp), 256>>>(u->e1, g0, g1, 64, u->p1, u->arg1);
+    UST(conv_fwd(u, L[1], u->e1a, g0, u->e1, u->c1, 64, w, w));
+    pool_rows_kernel<<<grid_for(g1.Rp * 4), 256>>>(u->e1, g0, g1, 32, u->p1, u->arg1);
     UCK(cudaGetLastError(), "pool");
     UST(conv_fwd(u, L[2], u->p1, g1, u->e2a));
-    UST(conv_fwd(u, L[3], u->e2a, g1, u->e2));
-    pool_rows_kernel<<<warp_grid(g2.Rp), 256>>>(u->e2, g1, g2, 64, u->p2, u->arg2);
+    UST(conv_fwd(u, L[3], u->e2a, g1, u->e2, u->c2, 128, 2 * w, 2 * w));
+    pool_rows_kernel<<<grid_for(g2.Rp * 8), 256>>>(u->e2, g1, g2, 64, u->p2, u->arg2);
     UCK(cudaGetLastError(), "pool");
     UST(conv_fwd(u, L[4], u->p2, g2, u->e3a));
     UST(conv_fwd(u, L[5], u->e3a, g2, u->e3));
-    UST(up_fwd(u, L[6], u->e3, g2, g1, u->u2));
-    concat_kernel<<<grid_for(g1.Rp * 128), 256>>>(u->u2, 64, 2 * w, u->e2, 64, 2 * w, g1.Rp, 128, u->c2);
-    UCK(cudaGetLastError(), "concat");
+    UST(up_fwd(u, L[6], u->e3, g2, g1, u->c2));
     UST(conv_fwd(u, L[7], u->c2, g1, u->d2a));
     UST(conv_fwd(u, L[8], u->d2a, g1, u->d2));
-    UST(up_fwd(u, L[9], u->d2, g1, g0, u->u1));
-    concat_kernel<<<grid_for(g0.Rp * 64), 256>>>(u->u1, 64, w, u->e1, 64, w, g0.Rp, 64, u->c1);
-    UCK(cudaGetLastError(), "concat");
+    UST(up_fwd(u, L[9], u->d2, g1, g0, u->c1));
     UST(conv_fwd(u, L[10], u->c1, g0, u->d1a));
     UST(conv_fwd(u, L[11], u->d1a, g0, u->d1));
-    return conv_fwd(u, L[12], u->d1, g0, nullptr);
+    const lbms_unet::Layer& h = L[12];
+    lbms::ConvJob j = conv_job(g0, u->d1, h.ci_s, h.Wb, h.rows, 1, 1, lbms::kOutHead);
+    j.ep.bias = h.b;
+    if (train) {
+        UCK(cudaMemsetAsync(u->loss, 0, sizeof(double), 0), "loss");
+        for (auto& l : L) UCK(cudaMemsetAsync(l.gb, 0, l.co_s * sizeof(float), 0), "bias gradients");
+        j.ep.T = u->T;
+        j.ep.inv_n = inv_n;
+        j.ep.out = u->za[0];
+        j.ep.gb = h.gb;
+        j.ep.loss = u->loss;
+    } else {
+        j.ep.Y = u->Y;
+    }
+    return run_conv(u, j, "head");
 }
 
-// Loss against u->T (targets and mask) and the backward pass through every
-// layer after unet_forward; gradients in each layer's g / gb.
-lbms_status unet_backward(lbms_unet* u, const Levels& v, float inv_n) {
+// The backward pass through every layer after unet_forward(train); gradients
+// in each layer's g / gb.
+lbms_status unet_backward(lbms_unet* u, const Levels& v) {
     const Geo &g0 = v.g[0], &g1 = v.g[1], &g2 = v.g[2];
-    const int w = u->width;
     auto& L = u->L;
-    UCK(cudaMemsetAsync(u->loss, 0, sizeof(double), 0), "loss");
-    for (auto& l : L) UCK(cudaMemsetAsync(l.gb, 0, l.co_s * sizeof(float), 0), "bias gradients");
-    // head: dP, its weight gradient dP^T . d1 and the gradient of d1
-    const lbms_unet::Layer& h = L[12];
-    unet_loss_kernel<<<(unsigned)(g0.Rp / 64), 256>>>(u->P, h.b, u->T, g0.Rp, inv_n, u->dz, h.gb, u->loss, u->Y);
-    UCK(cudaGetLastError(), "loss");
-    UST(transpose_rows(u, u->dz, u->dzT, g0.Rp, kUOutC, 1, 0, u->g_elems));
-    UST(transpose_rows(u, u->d1, u->aT, g0.Rp, h.ci_s, 1, 0, u->g_elems));
-    UST(ugemm(u, u->dzT, g0.Rp, u->aT, g0.Rp, h.rows, h.ci_s, g0.Rp, g0.S));
-    splitk_sum_kernel<<<grid_for((int64_t)h.rows * h.K), 256>>>(u->P, g0.S, (int64_t)h.rows * h.K, h.g);
-    UCK(cudaGetLastError(), "split-k sum");
-    UST(ugemm(u, u->dz, kUOutC, h.Wt, h.rows, g0.Rp, h.ci_s, h.rows, 1));
-    // Input gradients stay in P (unmasked) when a ReLU backward or a pooling
-    // gradient reads them next; the two that feed a concatenation's split
-    // are masked into fa / fb (the split's halves reach bias column sums).
-    float* P = u->P;
+    bf16 **za = u->za, **zb = u->zb;
+    UST(layer_wgrad(u, L[12], u->d1, za[0], g0));
+    UST(dgrad_relu(u, L[12], za[0], g0, u->d1, L[11], zb[0]));
     // decoder, level 0
-    UST(conv_bwd(u, L[11], u->d1a, u->d1, P, g0, P));
-    UST(conv_bwd(u, L[10], u->c1, u->d1a, P, g0, u->fa));
-    split_kernel<<<grid_for(g0.Rp * 64), 256>>>(u->fa, 64, w, w, 64, 64, g0.Rp, u->fb, u->fc);
-    UCK(cudaGetLastError(), "split");
-    UST(up_bwd(u, L[9], u->d2, u->fb, g1, g0, P));
+    UST(layer_wgrad(u, L[11], u->d1a, zb[0], g0));
+    UST(dgrad_relu(u, L[11], zb[0], g0, u->d1a, L[10], za[0]));
+    UST(layer_wgrad(u, L[10], u->c1, za[0], g0));
+    UST(dgrad_split(u, L[10], za[0], g0, g1, L[9], u->G1, u->skip0));
+    UST(layer_wgrad(u, L[9], u->d2, u->G1, g1));
+    UST(dgrad_relu(u, L[9], u->G1, g1, u->d2, L[8], za[1]));
     // decoder, level 1
-    UST(conv_bwd(u, L[8], u->d2a, u->d2, P, g1, P));
-    UST(conv_bwd(u, L[7], u->c2, u->d2a, P, g1, u->fb));
-    split_kernel<<<grid_for(g1.Rp * 64), 256>>>(u->fb, 128, 2 * w, 2 * w, 64, 64, g1.Rp, u->fa, u->fd);
-    UCK(cudaGetLastError(), "split");
-    UST(up_bwd(u, L[6], u->e3, u->fa, g2, g1, P));
+    UST(layer_wgrad(u, L[8], u->d2a, za[1], g1));
+    UST(dgrad_relu(u, L[8], za[1], g1, u->d2a, L[7], zb[1]));
+    UST(layer_wgrad(u, L[7], u->c2, zb[1], g1));
+    UST(dgrad_split(u, L[7], zb[1], g1, g2, L[6], u->G2, u->skip1));
+    UST(layer_wgrad(u, L[6], u->e3, u->G2, g2));
+    UST(dgrad_relu(u, L[6], u->G2, g2, u->e3, L[5], za[2]));
     // bottom, level 2
-    UST(conv_bwd(u, L[5], u->e3a, u->e3, P, g2, P));
-    UST(conv_bwd(u, L[4], u->p2, u->e3a, P, g2, P));
-    pool_back_rows_kernel<<<warp_grid(g1.R), 256>>>(P, u->arg2, g1, g2, 64, u->fd);
-    UCK(cudaGetLastError(), "pool backward");
+    UST(layer_wgrad(u, L[5], u->e3a, za[2], g2));
+    UST(dgrad_relu(u, L[5], za[2], g2, u->e3a, L[4], zb[2]));
+    UST(layer_wgrad(u, L[4], u->p2, zb[2], g2));
+    UST(dgrad_store(u, L[4], zb[2], g2, u->dp2));
     // encoder, level 1
-    UST(conv_bwd(u, L[3], u->e2a, u->e2, u->fd, g1, P));
-    UST(conv_bwd(u, L[2], u->p1, u->e2a, P, g1, P));
-    pool_back_rows_kernel<<<warp_grid(g0.R), 256>>>(P, u->arg1, g0, g1, 64, u->fc);
+    pool_relu_back_kernel<<<152 * 4, 256>>>(u->dp2, u->arg2, u->skip1, u->e2, g1, g2, 64, za[1], L[3].gb);
     UCK(cudaGetLastError(), "pool backward");
+    UST(layer_wgrad(u, L[3], u->e2a, za[1], g1));
+    UST(dgrad_relu(u, L[3], za[1], g1, u->e2a, L[2], zb[1]));
+    UST(layer_wgrad(u, L[2], u->p1, zb[1], g1));
+    UST(dgrad_store(u, L[2], zb[1], g1, u->dp1));
     // encoder, level 0
-    UST(conv_bwd(u, L[1], u->e1a, u->e1, u->fc, g0, P));
-    return conv_bwd(u, L[0], u->x0, u->e1a, P, g0, nullptr);
+    pool_relu_back_kernel<<<152 * 4, 256>>>(u->dp1, u->arg1, u->skip0, u->e1, g0, g1, 32, za[0], L[1].gb);
+    UCK(cudaGetLastError(), "pool backward");
+    UST(layer_wgrad(u, L[1], u->e1a, za[0], g0));
+    UST(dgrad_relu(u, L[1], za[0], g0, u->e1a, L[0], zb[0]));
+    return layer_wgrad(u, L[0], u->x0, zb[0], g0);
 }
 
 // The BF16 copies of one layer's weights from its FP32 master copy.
@@ -883,13 +785,13 @@ lbms_status lbms_unet_create(int width, int64_t max_voxels, uint64_t seed, lbms_
     u->vcap = max_voxels;
     const int w = width;
     // kind, output level, real / stored input channels, real / stored output channels
-    const int spec[kULayers][6] = {{3, 0, kUInReal, kUInC, w, 64}, {3, 0, w, 64, w, 64},
-                                   {3, 1, w, 64, 2 * w, 64},       {3, 1, 2 * w, 64, 2 * w, 64},
+    const int spec[kULayers][6] = {{3, 0, kUInReal, kUInC, w, 32}, {3, 0, w, 32, w, 32},
+                                   {3, 1, w, 32, 2 * w, 64},       {3, 1, 2 * w, 64, 2 * w, 64},
                                    {3, 2, 2 * w, 64, 4 * w, 128},  {3, 2, 4 * w, 128, 4 * w, 128},
                                    {2, 1, 4 * w, 128, 2 * w, 64},  {3, 1, 4 * w, 128, 2 * w, 64},
-                                   {3, 1, 2 * w, 64, 2 * w, 64},   {2, 0, 2 * w, 64, w, 64},
-                                   {3, 0, 2 * w, 64, w, 64},       {3, 0, w, 64, w, 64},
-                                   {1, 0, w, 64, 3, kUOutC}};
+                                   {3, 1, 2 * w, 64, 2 * w, 64},   {2, 0, 2 * w, 64, w, 32},
+                                   {3, 0, 2 * w, 64, w, 32},       {3, 0, w, 32, w, 32},
+                                   {1, 0, w, 32, 3, kUOutC}};
     for (int i = 0; i < kULayers; ++i) {
         auto& l = u->L[i];
         l.kind = spec[i][0];
@@ -1111,8 +1013,8 @@ lbms_status lbms_unet_train(lbms_unet* u, int iters, int max_batch, double lr, d
         UCK(cudaMemsetAsync(u->T + g0.R * 4, 0, (g0.Rp - g0.R) * 4 * sizeof(float), 0), "batch");
         const double cw = 0.5 * (1.0 + std::cos(3.14159265358979323846 * (double)it / std::max(1, iters)));
         const double lr_it = lr / 20.0 + (lr - lr / 20.0) * cw;
-        UST(unet_forward(u, lv));
-        UST(unet_backward(u, lv, (float)(1.0 / (3.0 * (double)std::max<int64_t>(nfl, 1)))));
+        UST(unet_forward(u, lv, true, (float)(1.0 / (3.0 * (double)std::max<int64_t>(nfl, 1)))));
+        UST(unet_backward(u, lv));
         UST(unet_adam(u, lr_it));
         if (it >= iters - 10) {
             double l = 0.0;
@@ -1149,10 +1051,7 @@ lbms_status lbms_unet_warm_start(lbms_unet* u, lbms_ctx* ctx, int k, double* Xou
     UCK(cudaMemset(u->x0, 0, (size_t)g0.Rp * kUInC * sizeof(bf16)), "inputs");
     unet_inputs_kernel<<<grid_for((int64_t)v.nf * kUInC), 256>>>(F.rows, prow, v.nf, u->x0);
     UCK(cudaGetLastError(), "inputs");
-    UST(unet_forward(u, lv));
-    unet_loss_kernel<<<(unsigned)(g0.Rp / 64), 256>>>(u->P, u->L[kULayers - 1].b, nullptr, g0.Rp, 0.0f, nullptr,
-                                                      nullptr, nullptr, u->Y);
-    UCK(cudaGetLastError(), "head");
+    UST(unet_forward(u, lv, false, 0.0f));
     unet_post_kernel<<<(v.nf + 255) / 256, 256>>>(u->Y, prow, v.nf, g0.Xp, F.xtab, dX);
     UCK(cudaGetLastError(), "prediction");
     std::vector<double> c((size_t)3 * v.nf);
@@ -1214,11 +1113,8 @@ lbms_status lbms_unet_forward(lbms_unet* u, const float* x, int B, int X, int Y,
     if (!u || !y) return LBMS_EINVAL;
     Levels lv;
     UST(upload_batch(u, x, nullptr, B, X, Y, Z, &lv, nullptr));
-    UST(unet_forward(u, lv));
+    UST(unet_forward(u, lv, false, 0.0f));
     const Geo& g0 = lv.g[0];
-    unet_loss_kernel<<<(unsigned)(g0.Rp / 64), 256>>>(u->P, u->L[kULayers - 1].b, nullptr, g0.Rp, 0.0f, nullptr,
-                                                      nullptr, nullptr, u->Y);
-    UCK(cudaGetLastError(), "head");
     std::vector<float> h((size_t)g0.R * 4);
     UCK(cudaMemcpy(h.data(), u->Y, h.size() * sizeof(float), cudaMemcpyDeviceToHost), "read output");
     UST(unet_check_gemm(u));
@@ -1240,8 +1136,8 @@ lbms_status lbms_unet_train_batch(lbms_unet* u, const float* x, const float* t, 
     double nf = 0.0;
     Levels lv;
     UST(upload_batch(u, x, t, B, X, Y, Z, &lv, &nf));
-    UST(unet_forward(u, lv));
-    UST(unet_backward(u, lv, (float)(1.0 / (3.0 * std::max(nf, 1.0)))));
+    UST(unet_forward(u, lv, true, (float)(1.0 / (3.0 * std::max(nf, 1.0)))));
+    UST(unet_backward(u, lv));
     if (lr > 0.0) UST(unet_adam(u, lr));
     if (loss) UCK(cudaMemcpy(loss, u->loss, sizeof(double), cudaMemcpyDeviceToHost), "read loss");
     UCK(cudaDeviceSynchronize(), "train batch");
