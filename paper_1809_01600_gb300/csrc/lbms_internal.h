@@ -75,6 +75,7 @@ struct DevBuffers {
     double* rre_coef = nullptr;        // [cases][order] coefficients of the differences (lazy)
     double* case_out = nullptr;        // [cases][10] residual sums, then [cases][6] boundary sums
     void* fields = nullptr;            // [3 + 3 dim][S] of tau and u (lazy), FP64 or FP32
+    double* dense = nullptr;           // X on the dense grid of the largest case (lazy)
 };
 
 struct Launch {
@@ -111,6 +112,14 @@ struct CaseHostBC {
     int tab;            // first row-table entry of the case
 };
 
+// First touch of freshly mapped host memory by the CPU: a device copy into
+// untouched 64 KB pages takes a fault of some 25 us for each.
+inline void touch_pages(double* p, int64_t n) {
+    volatile double* v = p;
+    for (int64_t i = 0; i < n; i += 512) v[i] = 0.0;
+    if (n > 0) v[n - 1] = 0.0;
+}
+
 size_t pop_size(int precision);    // bytes per stored population
 size_t x_size(int precision);      // bytes per stored mole fraction
 size_t field_size(int precision);  // bytes per tau / u value of the fields kernel
@@ -125,6 +134,15 @@ cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st);
 cudaError_t launch_fields(const Launch& L, cudaStream_t st);
+// X of species s, s + 1, ... (`count` of them) of a case's cells [base, base + nf)
+// on its dense grid of N cells, dense[species - s][N] (coordinates from
+// cell_code; solid voxels are not written), and back
+cudaError_t launch_to_dense(const Launch& L, int base, int nf, int nx, int ny, int64_t N, int s, int count,
+                            double* dense, cudaStream_t st);
+cudaError_t launch_from_dense(const Launch& L, int base, int nf, int nx, int ny, int64_t N, int s, int count,
+                              const double* dense, cudaStream_t st);
+// X of a case's cells from [3][nf] values
+cudaError_t launch_put_x(const Launch& L, int base, int nf, const double* values, cudaStream_t st);
 cudaError_t launch_case_residuals(const Launch& L, int update, cudaStream_t st);
 cudaError_t launch_case_boundary(const Launch& L, cudaStream_t st);
 // per-case sums of (X - E)^2 etc. into case_out[c * 10 + v], E unchanged
@@ -232,6 +250,7 @@ struct CaseView {
     int64_t N;                    // cells of the dense grid
     int nf;                       // fluid cells
     const int64_t* fluid_cell;    // dense index of each fluid cell (host)
+    const uint32_t* cell_code;    // their coordinates x | y << 11 | z << 21 (device), or null
     double x_in[3];
     double current;               // A/cm2
     bool periodic_x;
@@ -243,5 +262,9 @@ bool case_view(const lbms_ctx* c, int k, CaseView* v);
 // data, prof[s * nx + x]; false if it goes negative (or the box is periodic
 // in x).
 bool case_profile_1d(const lbms_ctx* c, int k, std::vector<double>& prof);
+
+// Restarts case k from X [3][nf] in device memory (f = w X), as
+// lbms_batch_set_fields does from a host field; the values must be complete.
+int case_restart_device(lbms_ctx* c, int k, const double* X);
 
 }  // namespace lbms

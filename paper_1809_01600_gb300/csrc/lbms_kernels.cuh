@@ -807,6 +807,37 @@ __global__ void init_kernel(P* __restrict__ h, const XS* __restrict__ x0, XS* __
     }
 }
 
+// Dense grid index of a fluid cell from its coordinate word.
+__device__ __forceinline__ int64_t dense_index(uint32_t code, int nx, int ny) {
+    return ((int64_t)(code >> 21) * ny + ((code >> 11) & 1023u)) * nx + (code & 2047u);
+}
+
+template <typename XS>
+__global__ void to_dense_kernel(const XS* __restrict__ X, int64_t S, const uint32_t* __restrict__ code, int base, int nf,
+                                int nx, int ny, int64_t N, int s, int count, double* __restrict__ dense) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    const int64_t e = dense_index(__ldg(code + base + j), nx, ny);
+    for (int q = 0; q < count; ++q) dense[q * N + e] = Xv<XS>::own(X, S, s + q, base + j).to_double();
+}
+
+template <typename XS>
+__global__ void from_dense_kernel(XS* __restrict__ X, int64_t S, const uint32_t* __restrict__ code, int base, int nf,
+                                  int nx, int ny, int64_t N, int s, int count, const double* __restrict__ dense) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    const int64_t e = dense_index(__ldg(code + base + j), nx, ny);
+    for (int q = 0; q < count; ++q) store_x<XS>(X, S, s + q, base + j, dense[q * N + e]);
+}
+
+template <typename XS>
+__global__ void put_x_kernel(XS* __restrict__ X, int64_t S, int base, int nf, const double* __restrict__ v) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) store_x<XS>(X, S, s, base + j, v[(int64_t)s * nf + j]);
+}
+
 // -------------------------------------------------------------------------
 // Deterministic FP64 block reduction: warp shuffles, one partial per block,
 // and the last block to finish sums the partials in a fixed order.

@@ -144,6 +144,39 @@ cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st) 
 cudaError_t launch_fields(const Launch& L, cudaStream_t st) { LBMS_DISPATCH(fields_t, L, st); }
 cudaError_t launch_case_boundary(const Launch& L, cudaStream_t st) { LBMS_DISPATCH(boundary_t, L, st); }
 
+cudaError_t launch_to_dense(const Launch& L, int base, int nf, int nx, int ny, int64_t N, int s, int count,
+                            double* dense, cudaStream_t st) {
+    const int grid = (nf + kBlock - 1) / kBlock;
+    if (L.precision == 0)
+        to_dense_kernel<double><<<grid, kBlock, 0, st>>>(static_cast<const double*>(L.b.X[L.cur]), L.S, L.b.cell_code,
+                                                         base, nf, nx, ny, N, s, count, dense);
+    else
+        to_dense_kernel<float><<<grid, kBlock, 0, st>>>(static_cast<const float*>(L.b.X[L.cur]), L.S, L.b.cell_code,
+                                                        base, nf, nx, ny, N, s, count, dense);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_from_dense(const Launch& L, int base, int nf, int nx, int ny, int64_t N, int s, int count,
+                              const double* dense, cudaStream_t st) {
+    const int grid = (nf + kBlock - 1) / kBlock;
+    if (L.precision == 0)
+        from_dense_kernel<double><<<grid, kBlock, 0, st>>>(static_cast<double*>(L.b.X[L.cur]), L.S, L.b.cell_code, base,
+                                                           nf, nx, ny, N, s, count, dense);
+    else
+        from_dense_kernel<float><<<grid, kBlock, 0, st>>>(static_cast<float*>(L.b.X[L.cur]), L.S, L.b.cell_code, base,
+                                                          nf, nx, ny, N, s, count, dense);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_put_x(const Launch& L, int base, int nf, const double* values, cudaStream_t st) {
+    const int grid = (nf + kBlock - 1) / kBlock;
+    if (L.precision == 0)
+        put_x_kernel<double><<<grid, kBlock, 0, st>>>(static_cast<double*>(L.b.X[L.cur]), L.S, base, nf, values);
+    else
+        put_x_kernel<float><<<grid, kBlock, 0, st>>>(static_cast<float*>(L.b.X[L.cur]), L.S, base, nf, values);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_case_extrap_norms(const Launch& L, cudaStream_t st) {
     return L.precision == 0 ? extrap_norms_t<double>(L, st) : extrap_norms_t<float>(L, st);
 }

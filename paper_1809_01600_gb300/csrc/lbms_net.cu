@@ -19,6 +19,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lbms.h"
@@ -280,42 +281,99 @@ __global__ void sample_kernel(const bf16* __restrict__ feat, const float* __rest
 }
 
 // ------------------------------------------------------------- features
-// Sum of `in` over a window of half-width h along one axis of the dense
-// grid [nz][ny][nx]: clamped at the ends of x, periodic in y and z.  With
-// count != NULL the window sizes are accumulated too (x only).
-__global__ void box_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int nz, int axis,
-                           int h, const float* __restrict__ cnt_in, float* __restrict__ cnt_out) {
-    const int64_t N = (int64_t)nx * ny * nz;
+// Dense index of every fluid cell from its coordinate word.
+__global__ void cell_index_kernel(const uint32_t* __restrict__ code, int nf, int nx, int ny,
+                                  int64_t* __restrict__ cell) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    const uint32_t c = code[j];
+    cell[j] = ((int64_t)(c >> 21) * ny + ((c >> 11) & 1023u)) * nx + (c & 2047u);
+}
+
+// Fluid mask on the dense grid (cleared before) and fluid cells per x-plane.
+__global__ void mask_kernel(const int64_t* __restrict__ cell, int nf, int nx, uint8_t* __restrict__ mask,
+                            int* __restrict__ plane) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    mask[cell[j]] = 1;
+    atomicAdd(&plane[cell[j] % nx], 1);
+}
+
+// Fluid voxels in the windows of half-width 1, 3 and 7 around each voxel, one
+// axis after the other (x clamped, y and z periodic).  The counts are whole
+// numbers: at most 15, then 225, then 3375.
+struct Windows {
+    uint8_t* v[3];
+};
+__device__ constexpr int half_width(int q) { return q == 0 ? 1 : (q == 1 ? 3 : 7); }
+
+__global__ void window_x_kernel(const uint8_t* __restrict__ mask, int64_t N, int nx, Windows out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
         const int x = (int)(e % nx);
-        const int y = (int)((e / nx) % ny);
-        const int z = (int)(e / ((int64_t)nx * ny));
-        float s = 0.0f, c = 0.0f;
-        for (int d = -h; d <= h; ++d) {
-            int64_t j;
-            if (axis == 0) {
-                const int xx = x + d;
-                if (xx < 0 || xx >= nx) continue;
-                j = e + d;
-            } else if (axis == 1) {
-                const int yy = ((y + d) % ny + ny) % ny;
-                j = e + (int64_t)(yy - y) * nx;
-            } else {
-                const int zz = ((z + d) % nz + nz) % nz;
-                j = e + (int64_t)(zz - z) * nx * ny;
-            }
-            s += in[j];
-            if (cnt_in) c += cnt_in[j];
+        int s[3] = {0, 0, 0};
+#pragma unroll
+        for (int d = -7; d <= 7; ++d) {
+            const int v = x + d >= 0 && x + d < nx ? mask[e + d] : 0;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (d >= -half_width(q) && d <= half_width(q)) s[q] += v;
         }
-        out[e] = s;
-        if (cnt_out) cnt_out[e] = c;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) out.v[q][e] = (uint8_t)s[q];
     }
 }
 
-// w[e] = w[e] / cnt[e]: window sum to fluid fraction.
-__global__ void divide_kernel(float* __restrict__ w, const float* __restrict__ cnt, int64_t N) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x)
-        w[e] = cnt[e] > 0.0f ? w[e] / cnt[e] : 0.0f;
+__device__ __forceinline__ int wrap(int a, int n) {   // a in [-7, n + 7)
+    if (n >= 7) return a < 0 ? a + n : (a >= n ? a - n : a);
+    a %= n;
+    return a < 0 ? a + n : a;
+}
+
+__global__ void window_y_kernel(Windows in, int64_t N, int nx, int ny, Windows out) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
+        const int y = (int)((e / nx) % ny);
+        int s[3] = {0, 0, 0};
+#pragma unroll
+        for (int d = -7; d <= 7; ++d) {
+            const int64_t j = e + (int64_t)(wrap(y + d, ny) - y) * nx;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (d >= -half_width(q) && d <= half_width(q)) s[q] += in.v[q][j];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) out.v[q][e] = (uint8_t)s[q];
+    }
+}
+
+// The last axis, and the counts over the windows' sizes: w[q][e].
+__global__ void window_z_kernel(Windows in, int64_t N, int nx, int ny, int nz, float* __restrict__ w) {
+    const int64_t plane = (int64_t)nx * ny;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < N; e += (int64_t)gridDim.x * blockDim.x) {
+        const int x = (int)(e % nx), z = (int)(e / plane);
+        int s[3] = {0, 0, 0};
+#pragma unroll
+        for (int d = -7; d <= 7; ++d) {
+            if (nz == 1 && d != 0) continue;
+            const int64_t j = e + (int64_t)(wrap(z + d, nz) - z) * plane;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                if (d >= -half_width(q) && d <= half_width(q)) s[q] += in.v[q][j];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int h = half_width(q), t = 2 * h + 1;
+            const int wide = min(x + h, nx - 1) - max(x - h, 0) + 1;
+            w[q * N + e] = (float)s[q] / (float)(wide * t * (nz > 1 ? t : 1));
+        }
+    }
+}
+
+// dense[s][cell[j]] = v[s][j] (dense cleared before).
+__global__ void scatter_kernel(const double* __restrict__ v, const int64_t* __restrict__ cell, int nf, int64_t N,
+                               double* __restrict__ dense) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    for (int s = 0; s < 3; ++s) dense[s * N + cell[j]] = v[(int64_t)s * nf + j];
 }
 
 // Feature row of fluid cell j (dense index cell[j]), one thread per column:
@@ -399,6 +457,8 @@ struct lbms_net {
     int gemm_kind = LBMS_NET_GEMM_AUTO;
     int64_t tcgen05_calls = 0, mma_sync_calls = 0;
     std::vector<void*> allocs;
+    char* room = nullptr;                   // working memory of the case at hand, kept and grown on demand
+    size_t room_bytes = 0;
     std::string err;
 };
 
@@ -552,24 +612,17 @@ lbms_status backward_step(lbms_net* n, int R, double lr, double* loss) {
 }
 
 // Feature rows (device, [rows_pad][kF], zero padded) and the per-x table of
-// one case; rows_pad = nf rounded up to 64.
+// one case, with room for a prediction; rows_pad = nf rounded up to 64.  All
+// of it lies in the net's working memory, valid until its next case.
 struct CaseFeatures {
     bf16* rows = nullptr;
     float* xtab = nullptr;
-    int64_t* cell = nullptr;
+    int64_t* cell = nullptr;         // dense index of each fluid cell
+    int64_t* row = nullptr;          // [nf], for the caller
+    double* pred = nullptr;          // [3][nf], for the caller
+    double* dense = nullptr;         // [3][N], for the caller
     int nf = 0, nx = 0, rows_pad = 0;
     std::vector<double> prof;
-    std::vector<void*> tmp;
-    ~CaseFeatures() {
-        for (void* p : tmp) cudaFree(p);
-    }
-    template <typename T>
-    T* alloc(size_t count) {   // failures are recorded as null (see nalloc)
-        void* p = nullptr;
-        if (cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) p = nullptr;
-        tmp.push_back(p);
-        return static_cast<T*>(p);
-    }
 };
 
 lbms_status case_features(lbms_net* n, lbms_ctx* ctx, int k, CaseFeatures& F) {
@@ -584,13 +637,62 @@ lbms_status case_features(lbms_net* n, lbms_ctx* ctx, int k, CaseFeatures& F) {
     F.nf = v.nf;
     F.nx = nx;
     F.rows_pad = (v.nf + 63) / 64 * 64;
-    // host: dense fluid mask, per-x table (profile, x / (nx - 1), plane
-    // porosity, normalised cumulative resistance, inverse porosity)
-    std::vector<float> mask(N, 0.0f);
-    for (int j = 0; j < v.nf; ++j) mask[v.fluid_cell[j]] = 1.0f;
+    uint8_t *mask = nullptr, *b[6] = {};
+    float* w = nullptr;
+    int* plane = nullptr;
+    auto lay_out = [&](char* p) {
+        auto take = [&](auto*& ptr, size_t count) {
+            ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(p);
+            p += (count * sizeof(*ptr) + 255) / 256 * 256;
+        };
+        take(F.rows, (size_t)F.rows_pad * kF);
+        take(F.cell, v.nf);
+        take(F.row, v.nf);
+        take(F.pred, (size_t)3 * v.nf);
+        take(F.dense, (size_t)3 * N);
+        take(F.xtab, (size_t)nx * 8);
+        take(w, (size_t)3 * N);
+        take(plane, nx);
+        take(mask, N);
+        for (auto& q : b) take(q, N);
+        return p;
+    };
+    const size_t need = (size_t)(lay_out(nullptr) - (char*)nullptr);
+    if (need > n->room_bytes) {
+        NCK(cudaDeviceSynchronize(), "feature buffers");
+        cudaFree(n->room);
+        n->room = nullptr;
+        n->room_bytes = 0;
+        if (cudaMalloc(&n->room, need) != cudaSuccess) {
+            n->room = nullptr;
+            cudaGetLastError();
+            return nfail(n, LBMS_ENOMEM, "feature buffers");
+        }
+        n->room_bytes = need;
+    }
+    lay_out(n->room);
+    const int gc = (v.nf + 255) / 256, g = grid_for(N);
+    if (v.cell_code) {
+        cell_index_kernel<<<gc, 256>>>(v.cell_code, v.nf, nx, ny, F.cell);
+        NCK(cudaGetLastError(), "cells");
+    } else {
+        NCK(cudaMemcpy(F.cell, v.fluid_cell, v.nf * sizeof(int64_t), cudaMemcpyHostToDevice), "cells");
+    }
+    NCK(cudaMemsetAsync(mask, 0, N, 0), "mask");
+    NCK(cudaMemsetAsync(plane, 0, nx * sizeof(int), 0), "mask");
+    mask_kernel<<<gc, 256>>>(F.cell, v.nf, nx, mask, plane);
+    NCK(cudaGetLastError(), "mask");
+    const Windows wx{{b[0], b[1], b[2]}}, wy{{b[3], b[4], b[5]}};
+    window_x_kernel<<<g, 256>>>(mask, N, nx, wx);
+    window_y_kernel<<<g, 256>>>(wx, N, nx, ny, wy);
+    window_z_kernel<<<g, 256>>>(wy, N, nx, ny, nz, w);
+    NCK(cudaGetLastError(), "box filter");
+    // host: per-x table (profile, x / (nx - 1), plane porosity, normalised
+    // cumulative resistance, inverse porosity)
+    std::vector<int> count(nx);
+    NCK(cudaMemcpy(count.data(), plane, nx * sizeof(int), cudaMemcpyDeviceToHost), "plane porosity");
     std::vector<double> phi(nx, 0.0);
-    for (int64_t e = 0; e < N; ++e) phi[e % nx] += mask[e];
-    for (int x = 0; x < nx; ++x) phi[x] = std::max(phi[x] / ((double)ny * nz), 1.0 / ((double)ny * nz));
+    for (int x = 0; x < nx; ++x) phi[x] = std::max(count[x] / ((double)ny * nz), 1.0 / ((double)ny * nz));
     std::vector<double> res(nx, 0.0);
     for (int x = 1; x < nx; ++x) res[x] = res[x - 1] + 0.5 * (1.0 / phi[x - 1] + 1.0 / phi[x]);
     std::vector<float> xtab((size_t)nx * 8, 0.0f);
@@ -601,39 +703,30 @@ lbms_status case_features(lbms_net* n, lbms_ctx* ctx, int k, CaseFeatures& F) {
         xtab[(size_t)x * 8 + 5] = (float)(res[nx - 1] > 0 ? res[x] / res[nx - 1] : 0.0);
         xtab[(size_t)x * 8 + 6] = (float)(0.25 / phi[x]);
     }
-    float* dmask = F.alloc<float>(N);
-    float* ones = F.alloc<float>(N);
-    float* t0 = F.alloc<float>(N);
-    float* t1 = F.alloc<float>(N);
-    float* c0 = F.alloc<float>(N);
-    float* c1 = F.alloc<float>(N);
-    float* w[3] = {F.alloc<float>(N), F.alloc<float>(N), F.alloc<float>(N)};
-    float* cnt[3] = {F.alloc<float>(N), F.alloc<float>(N), F.alloc<float>(N)};
-    F.xtab = F.alloc<float>(xtab.size());
-    F.cell = F.alloc<int64_t>(v.nf);
-    F.rows = F.alloc<bf16>((size_t)F.rows_pad * kF);
-    for (void* p : F.tmp)
-        if (!p) return nfail(n, LBMS_ENOMEM, "feature buffers");
-    NCK(cudaMemcpy(dmask, mask.data(), N * sizeof(float), cudaMemcpyHostToDevice), "mask");
-    std::vector<float> one(N, 1.0f);
-    NCK(cudaMemcpy(ones, one.data(), N * sizeof(float), cudaMemcpyHostToDevice), "ones");
     NCK(cudaMemcpy(F.xtab, xtab.data(), xtab.size() * sizeof(float), cudaMemcpyHostToDevice), "x table");
-    NCK(cudaMemcpy(F.cell, v.fluid_cell, v.nf * sizeof(int64_t), cudaMemcpyHostToDevice), "cells");
-    NCK(cudaMemset(F.rows, 0, (size_t)F.rows_pad * kF * sizeof(bf16)), "rows");
-    const int hw[3] = {1, 3, 7};
-    const int g = grid_for(N);
-    for (int q = 0; q < 3; ++q) {
-        // window sums of the mask and of the window sizes (x clamped)
-        box_kernel<<<g, 256>>>(dmask, t0, nx, ny, nz, 0, hw[q], ones, c0);
-        box_kernel<<<g, 256>>>(t0, t1, nx, ny, nz, 1, hw[q], c0, c1);
-        box_kernel<<<g, 256>>>(t1, w[q], nx, ny, nz, 2, nz > 1 ? hw[q] : 0, c1, cnt[q]);
-        NCK(cudaGetLastError(), "box filter");
-    }
-    for (int q = 0; q < 3; ++q) divide_kernel<<<g, 256>>>(w[q], cnt[q], N);
+    NCK(cudaMemsetAsync(F.rows + (size_t)v.nf * kF, 0, (size_t)(F.rows_pad - v.nf) * kF * sizeof(bf16), 0), "rows");
     const dim3 blk(kF, 4);
-    assemble_kernel<<<(v.nf + 3) / 4, blk>>>(F.cell, v.nf, nx, F.xtab, w[0], w[1], w[2], (float)v.current,
+    assemble_kernel<<<(v.nf + 3) / 4, blk>>>(F.cell, v.nf, nx, F.xtab, w, w + N, w + 2 * N, (float)v.current,
                                              (float)v.x_in[0], (float)v.x_in[1], (float)v.x_in[2], F.rows);
     NCK(cudaGetLastError(), "features");
+    return LBMS_OK;
+}
+
+// The prediction F.pred becomes case k's state and, with Xout, the caller's
+// dense field.
+lbms_status take_prediction(lbms_net* n, lbms_ctx* ctx, int k, const CaseFeatures& F, double* Xout) {
+    lbms::CaseView v;
+    lbms::case_view(ctx, k, &v);
+    if (Xout) {
+        NCK(cudaMemsetAsync(F.dense, 0, (size_t)3 * v.N * sizeof(double), 0), "prediction");
+        scatter_kernel<<<(F.nf + 255) / 256, 256>>>(F.pred, F.cell, F.nf, v.N, F.dense);
+        NCK(cudaGetLastError(), "prediction");
+        lbms::touch_pages(Xout, 3 * v.N);
+        NCK(cudaMemcpy(Xout, F.dense, (size_t)3 * v.N * sizeof(double), cudaMemcpyDeviceToHost), "read prediction");
+    }
+    NCK(cudaStreamSynchronize(0), "prediction");   // the handle may work on another stream
+    const lbms_status st = (lbms_status)lbms::case_restart_device(ctx, k, F.pred);
+    if (st != LBMS_OK) return nfail(n, st, "restarting case %d: %s", k, lbms_last_error(ctx));
     return LBMS_OK;
 }
 
@@ -750,6 +843,7 @@ lbms_status lbms_net_create(int width, int depth, uint64_t seed, lbms_net** out)
 void lbms_net_destroy(lbms_net* n) {
     if (!n) return;
     for (void* p : n->allocs) cudaFree(p);
+    cudaFree(n->room);
     cudaFree(n->feat);
     cudaFree(n->targ);
     delete n;
@@ -929,8 +1023,6 @@ lbms_status lbms_net_warm_start(lbms_net* n, lbms_ctx* ctx, int k, double* Xout)
     if (st != LBMS_OK) return st;
     lbms::CaseView v;
     lbms::case_view(ctx, k, &v);
-    double* dX = F.alloc<double>((size_t)3 * v.nf);
-    if (!dX) return nfail(n, LBMS_ENOMEM, "prediction buffer");
     for (int j0 = 0; j0 < F.rows_pad; j0 += kMaxRows) {
         const int rows = std::min(kMaxRows, F.rows_pad - j0);
         NCK(cudaMemcpy(n->act[0], F.rows + (size_t)j0 * kF, (size_t)rows * kF * sizeof(bf16),
@@ -938,18 +1030,10 @@ lbms_status lbms_net_warm_start(lbms_net* n, lbms_ctx* ctx, int k, double* Xout)
             "rows");
         st = forward(n, rows, false);
         if (st != LBMS_OK) return st;
-        predict_post_kernel<<<(rows + 255) / 256, 256>>>(n->Y, F.cell, j0, rows, v.nf, v.nx, F.xtab, dX);
+        predict_post_kernel<<<(rows + 255) / 256, 256>>>(n->Y, F.cell, j0, rows, v.nf, v.nx, F.xtab, F.pred);
         NCK(cudaGetLastError(), "prediction");
     }
-    std::vector<double> c((size_t)3 * v.nf);
-    NCK(cudaMemcpy(c.data(), dX, c.size() * sizeof(double), cudaMemcpyDeviceToHost), "read prediction");
-    std::vector<double> X((size_t)3 * v.N, 0.0);
-    for (int s = 0; s < 3; ++s)
-        for (int j = 0; j < v.nf; ++j) X[(size_t)s * v.N + v.fluid_cell[j]] = c[(size_t)s * v.nf + j];
-    st = lbms_batch_set_fields(ctx, k, X.data());
-    if (st != LBMS_OK) return nfail(n, st, "restarting case %d: %s", k, lbms_last_error(ctx));
-    if (Xout) std::copy(X.begin(), X.end(), Xout);
-    return LBMS_OK;
+    return take_prediction(n, ctx, k, F, Xout);
 }
 
 }  // extern "C"

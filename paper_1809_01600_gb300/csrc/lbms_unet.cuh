@@ -243,6 +243,16 @@ __global__ void unet_inputs_kernel(const bf16* __restrict__ rows, const int64_t*
     }
 }
 
+// Row of every fluid cell of a case (dense index cell[j]) in the layout of
+// its volume.
+__global__ void cell_row_kernel(const int64_t* __restrict__ cell, int nf, int nx, int ny, Geo g,
+                                int64_t* __restrict__ row) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nf) return;
+    const int64_t e = cell[j];
+    row[j] = voxel_row(g, 0, (int)(e % nx), (int)((e / nx) % ny), (int)(e / ((int64_t)nx * ny)));
+}
+
 // The prediction of one case from the head's output Y [r][4] at its row
 // row[j]: X_s = profile_s(x) + Y[row][s] / 100, clamped at 1e-6 and
 // renormalised; out [3][nf] FP64.  Xp: the padded x extent (x = row mod Xp - 1).
@@ -294,6 +304,7 @@ struct lbms_unet {
     int last[4] = {0, 0, 0, 0};  // B, X, Y, Z of the layout the buffers held last
     std::vector<void*> bufs;     // the grown buffers
     double* loss = nullptr;
+    float* flat = nullptr;       // parameters or gradients in the caller's order
     unsigned int* gemm_err = nullptr;
     struct Sample {
         int X = 0, Y = 0, Z = 0;                // interior extents (multiples of 4)
@@ -306,7 +317,7 @@ struct lbms_unet {
     uint64_t seed = 0;
     std::vector<void*> allocs;   // weights and the small fixed buffers
     std::string msg;
-    lbms_net feat;               // error messages of the shared feature builder (holds no device memory)
+    lbms_net feat;               // error messages and working memory of the shared feature builder
 };
 
 namespace {
@@ -720,15 +731,19 @@ lbms_status unet_check_gemm(lbms_unet* u) {
     return ufail(u, LBMS_ECUDA, "tensor-core GEMM: an mbarrier wait timed out (flag %u)", f);
 }
 
+int64_t layer_weights(const lbms_unet::Layer& l) {
+    return (int64_t)l.co * l.ci * (l.kind == 3 ? 27 : l.kind == 2 ? 8 : 1);
+}
+
 int64_t unet_params(const lbms_unet* u) {
     int64_t s = 0;
-    for (const auto& l : u->L) s += (int64_t)l.co * l.ci * (l.kind == 3 ? 27 : l.kind == 2 ? 8 : 1) + l.co;
+    for (const auto& l : u->L) s += layer_weights(l) + l.co;
     return s;
 }
 
 // Flat index in W of the real weight number e of a layer, in PyTorch's
 // order: Conv3d [co][ci][kz][ky][kx], ConvTranspose3d [ci][co][kz][ky][kx].
-size_t weight_slot(const lbms_unet::Layer& l, int64_t e) {
+__host__ __device__ size_t weight_slot(const lbms_unet::Layer& l, int64_t e) {
     if (l.kind == 3) {
         const int tap = (int)(e % 27), ci = (int)((e / 27) % l.ci), co = (int)(e / (27 * (int64_t)l.ci));
         return (size_t)co * l.K + (size_t)tap * l.ci_s + ci;
@@ -739,6 +754,19 @@ size_t weight_slot(const lbms_unet::Layer& l, int64_t e) {
     }
     const int ci = (int)(e % l.ci), co = (int)(e / l.ci);
     return (size_t)co * l.K + ci;
+}
+
+// The n real weights and then the biases of a layer between its storage
+// (W, b) and a flat array in PyTorch's order: flat <- storage, or back.
+__global__ void layer_flat_kernel(const __grid_constant__ lbms_unet::Layer l, float* __restrict__ W,
+                                  float* __restrict__ b, int64_t n, float* __restrict__ flat, bool back) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n + l.co; e += (int64_t)gridDim.x * blockDim.x) {
+        float* p = e < n ? W + weight_slot(l, e) : b + (e - n);
+        if (back)
+            *p = flat[e];
+        else
+            flat[e] = *p;
+    }
 }
 
 // A case on the network's grid: interior extents rounded up to multiples
@@ -767,6 +795,7 @@ void lbms_unet_destroy(lbms_unet* u) {
     cudaDeviceSynchronize();
     for (void* p : u->allocs) cudaFree(p);
     for (void* p : u->bufs) cudaFree(p);
+    cudaFree(u->feat.room);
     for (auto& s : u->samples) {
         cudaFree(s.in);
         cudaFree(s.tg);
@@ -815,6 +844,7 @@ lbms_status lbms_unet_create(int width, int64_t max_voxels, uint64_t seed, lbms_
         l.Wt = ualloc<bf16>(u, l.kind == 3 ? (size_t)l.ci_s * 27 * l.co_s : nw);
     }
     u->loss = ualloc<double>(u, 1);
+    u->flat = ualloc<float>(u, unet_params(u));
     u->gemm_err = ualloc<unsigned int>(u, 1);
     bool ok = true;
     for (void* p : u->allocs) ok = ok && p;
@@ -896,8 +926,7 @@ lbms_status lbms_unet_add_sample(lbms_unet* u, lbms_ctx* ctx, int k) {
     s.Z = cv.g.Z;
     s.rows = R;
     s.nfluid = v.nf;
-    int64_t* prow = F.alloc<int64_t>(v.nf);
-    if (!prow) return ufail(u, LBMS_ENOMEM, "cell rows");
+    int64_t* prow = F.row;
     if (cudaMalloc(&s.in, (size_t)R * kUInC * sizeof(bf16)) != cudaSuccess) return ufail(u, LBMS_ENOMEM, "sample");
     if (cudaMalloc(&s.tg, (size_t)R * 4 * sizeof(float)) != cudaSuccess) {
         cudaFree(s.in);
@@ -1036,34 +1065,23 @@ lbms_status lbms_unet_warm_start(lbms_unet* u, lbms_ctx* ctx, int k, double* Xou
     if (st != LBMS_OK) return ufail(u, st, "%s", u->feat.err.c_str());
     lbms::CaseView v;
     lbms::case_view(ctx, k, &v);
-    CaseVolume cv;
-    case_volume(v, cv);
-    const Levels lv = levels_of(1, cv.g.X, cv.g.Y, cv.g.Z);
-    if (cv.g.V > u->vcap || !levels_fit(lv))
-        return ufail(u, LBMS_EINVAL, "case %d needs %lld voxels, the network was made for %lld", k, (long long)cv.g.V,
+    const Levels lv = levels_of(1, (v.nx + 3) / 4 * 4, (v.ny + 3) / 4 * 4, (v.nz + 3) / 4 * 4);
+    const Geo& g0 = lv.g[0];
+    if (g0.V > u->vcap || !levels_fit(lv))
+        return ufail(u, LBMS_EINVAL, "case %d needs %lld voxels, the network was made for %lld", k, (long long)g0.V,
                      (long long)u->vcap);
     UST(ensure_buffers(u, lv));
-    int64_t* prow = F.alloc<int64_t>(v.nf);
-    double* dX = F.alloc<double>((size_t)3 * v.nf);
-    if (!prow || !dX) return ufail(u, LBMS_ENOMEM, "prediction buffers");
-    const Geo& g0 = lv.g[0];
-    UCK(cudaMemcpy(prow, cv.row.data(), v.nf * sizeof(int64_t), cudaMemcpyHostToDevice), "cells");
-    UCK(cudaMemset(u->x0, 0, (size_t)g0.Rp * kUInC * sizeof(bf16)), "inputs");
-    unet_inputs_kernel<<<grid_for((int64_t)v.nf * kUInC), 256>>>(F.rows, prow, v.nf, u->x0);
+    cell_row_kernel<<<(v.nf + 255) / 256, 256>>>(F.cell, v.nf, v.nx, v.ny, g0, F.row);
+    UCK(cudaGetLastError(), "cells");
+    UCK(cudaMemsetAsync(u->x0, 0, (size_t)g0.Rp * kUInC * sizeof(bf16), 0), "inputs");
+    unet_inputs_kernel<<<grid_for((int64_t)v.nf * kUInC), 256>>>(F.rows, F.row, v.nf, u->x0);
     UCK(cudaGetLastError(), "inputs");
     UST(unet_forward(u, lv, false, 0.0f));
-    unet_post_kernel<<<(v.nf + 255) / 256, 256>>>(u->Y, prow, v.nf, g0.Xp, F.xtab, dX);
+    unet_post_kernel<<<(v.nf + 255) / 256, 256>>>(u->Y, F.row, v.nf, g0.Xp, F.xtab, F.pred);
     UCK(cudaGetLastError(), "prediction");
-    std::vector<double> c((size_t)3 * v.nf);
-    UCK(cudaMemcpy(c.data(), dX, c.size() * sizeof(double), cudaMemcpyDeviceToHost), "read prediction");
     UST(unet_check_gemm(u));
-    std::vector<double> X((size_t)3 * v.N, 0.0);
-    for (int s = 0; s < 3; ++s)
-        for (int j = 0; j < v.nf; ++j) X[(size_t)s * v.N + v.fluid_cell[j]] = c[(size_t)s * v.nf + j];
-    st = lbms_batch_set_fields(ctx, k, X.data());
-    if (st != LBMS_OK) return ufail(u, st, "restarting case %d: %s", k, lbms_last_error(ctx));
-    if (Xout) std::copy(X.begin(), X.end(), Xout);
-    return LBMS_OK;
+    st = take_prediction(&u->feat, ctx, k, F, Xout);
+    return st == LBMS_OK ? st : ufail(u, st, "%s", u->feat.err.c_str());
 }
 
 }  // extern "C"
@@ -1151,16 +1169,12 @@ lbms_status lbms_unet_get(const lbms_unet* cu, int what, float* buf, int64_t cou
         return ufail(u, LBMS_EINVAL, "buffer holds %lld floats, need %lld", (long long)count, (long long)unet_params(u));
     int64_t off = 0;
     for (const auto& l : u->L) {
-        const size_t nw = (size_t)l.rows * l.K;
-        std::vector<float> W(nw), b(l.co_s);
-        UCK(cudaMemcpy(W.data(), what ? l.g : l.W, nw * sizeof(float), cudaMemcpyDeviceToHost), "get");
-        UCK(cudaMemcpy(b.data(), what ? l.gb : l.b, l.co_s * sizeof(float), cudaMemcpyDeviceToHost), "get");
-        const int64_t n = (int64_t)l.co * l.ci * (l.kind == 3 ? 27 : l.kind == 2 ? 8 : 1);
-        for (int64_t e = 0; e < n; ++e) buf[off + e] = W[weight_slot(l, e)];
-        off += n;
-        for (int c = 0; c < l.co; ++c) buf[off + c] = b[c];
-        off += l.co;
+        const int64_t n = layer_weights(l);
+        layer_flat_kernel<<<grid_for(n + l.co), 256>>>(l, what ? l.g : l.W, what ? l.gb : l.b, n, u->flat + off, false);
+        off += n + l.co;
     }
+    UCK(cudaGetLastError(), "get");
+    UCK(cudaMemcpy(buf, u->flat, (size_t)off * sizeof(float), cudaMemcpyDeviceToHost), "get");
     return LBMS_OK;
 }
 
@@ -1168,17 +1182,15 @@ lbms_status lbms_unet_set(lbms_unet* u, const float* buf, int64_t count) {
     if (!u || !buf) return LBMS_EINVAL;
     if (count < unet_params(u))
         return ufail(u, LBMS_EINVAL, "buffer holds %lld floats, need %lld", (long long)count, (long long)unet_params(u));
+    UCK(cudaMemcpy(u->flat, buf, (size_t)unet_params(u) * sizeof(float), cudaMemcpyHostToDevice), "set");
     int64_t off = 0;
     for (const auto& l : u->L) {
-        const size_t nw = (size_t)l.rows * l.K;
-        std::vector<float> W(nw, 0.0f), b(l.co_s, 0.0f);
-        const int64_t n = (int64_t)l.co * l.ci * (l.kind == 3 ? 27 : l.kind == 2 ? 8 : 1);
-        for (int64_t e = 0; e < n; ++e) W[weight_slot(l, e)] = buf[off + e];
-        off += n;
-        for (int c = 0; c < l.co; ++c) b[c] = buf[off + c];
-        off += l.co;
-        UCK(cudaMemcpy(l.W, W.data(), nw * sizeof(float), cudaMemcpyHostToDevice), "set");
-        UCK(cudaMemcpy(l.b, b.data(), l.co_s * sizeof(float), cudaMemcpyHostToDevice), "set");
+        const int64_t n = layer_weights(l);
+        UCK(cudaMemsetAsync(l.W, 0, (size_t)l.rows * l.K * sizeof(float), 0), "set");
+        UCK(cudaMemsetAsync(l.b, 0, l.co_s * sizeof(float), 0), "set");
+        layer_flat_kernel<<<grid_for(n + l.co), 256>>>(l, l.W, l.b, n, u->flat + off, true);
+        UCK(cudaGetLastError(), "set");
+        off += n + l.co;
         UST(cast_layer(u, l));
     }
     UCK(cudaDeviceSynchronize(), "set");
