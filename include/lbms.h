@@ -116,8 +116,8 @@ typedef struct {
  *             (per case, FP64), which removes up to M - 1 decay modes at once;
  *             a case whose snapshot differences do not shrink is left alone.
  *             Holds (M + 1) x 3 x cells doubles of snapshots [1]
- *  step_variant  0: handles of at least 48,640 cells with the default
- *             outlet_bc and grad_stencil take the tiled per-cell step; for
+ *  step_variant  0: handles with the default
+ *             outlet_bc and grad_stencil take a step chosen by size; for
  *             others the autotuner picks the step kernel's tile, thread
  *             mapping (a thread per cell and species, or per cell) and
  *             neighbour lookup by timing; k in 1..10 forces variant k - 1

@@ -259,7 +259,7 @@ size_t x_word(int precision) { return precision == LBMS_FP64 ? sizeof(double) : 
 // swapping, so the state is unchanged; the X copy of cur ^ 1 is restored.
 lbms_status autotune(lbms_ctx* c) {
     Launch& L = c->L;
-    if (L.tiled) {   // chosen by rule at create
+    if (L.tiled || L.small) {   // chosen by rule at create
         c->tuned = true;
         return LBMS_OK;
     }
@@ -454,6 +454,13 @@ lbms_status set_case_bc(lbms_ctx* c, int k, const double* x_inlet, double curren
 }
 
 lbms_status launch_steps(lbms_ctx* c, int64_t n) {
+    while (n > 0 && c->L.small && c->L.small != kSmall) {   // a block per case: many steps a launch
+        const int m = (int)std::min<int64_t>(n, kBlockSteps);
+        CK(launch_steps_block(c->L, m, c->stream), "step kernel");
+        c->L.cur ^= m & 1;
+        c->steps += m;
+        n -= m;
+    }
     while (n > 0) {
         if (n >= kGraphSteps) {
             const int par = c->L.cur;
@@ -966,10 +973,19 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
     L.drift = c->opt.coupling == LBMS_COUPLING_MS ? 1 : 0;
     L.grad_forward = c->opt.grad_stencil == LBMS_GRAD_FORWARD ? 1 : 0;
     L.outlet_extrap = c->opt.outlet_bc == LBMS_OUTLET_EXTRAPOLATED ? 1 : 0;
-    // the default step: the paper's default readings, element offsets of all
-    // populations in 32 bits, enough cells to fill the GPU
-    L.tiled = c->opt.step_variant == 0 && !L.grad_forward && !L.outlet_extrap && L.ncells >= kTileMinCells &&
-              3 * (int64_t)c->Q * (L.S + kTile) < (int64_t)1 << 32;
+    int dev = 0;
+    if (cudaError_t de = cudaGetDevice(&dev); de != cudaSuccess) return bail(cuda_fail(c, de, "cudaGetDevice"));
+    int smc = 0;
+    if (cudaDeviceGetAttribute(&smc, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && smc > 0) L.sm_count = smc;
+    // the steps chosen by rule, for the paper's default readings: the small
+    // handles' while the cells do not fill the GPU, else the tiled step (whose
+    // element offsets of all populations need 32 bits)
+    if (c->opt.step_variant == 0 && !L.grad_forward && !L.outlet_extrap) {
+        int max_nf = 0;
+        for (const auto& cs : c->cases) max_nf = std::max(max_nf, cs.nf);
+        L.small = choose_small(L, max_nf);
+        L.tiled = !L.small && 3 * (int64_t)c->Q * (L.S + kTile) < (int64_t)1 << 32;
+    }
 
     // reduction segments and block -> case tables
     std::vector<int2> segs, case_segs(n_cases), case_rows(n_cases);
@@ -997,12 +1013,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
         }
     }
 
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaGetDevice"));
-    int smc = 0;
-    if (cudaDeviceGetAttribute(&smc, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && smc > 0) L.sm_count = smc;
-    e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
+    cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "create capture stream"));
     e = cudaMallocHost(&c->host_out, (size_t)n_cases * kCaseOutSlots * sizeof(double));
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "pinned readback buffer"));
@@ -1045,7 +1056,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
             max_nf = std::max<int64_t>(max_nf, cs.nf);
         }
         int16_t* nb16 =
-            L.tiled ? nullptr : static_cast<int16_t*>(dev_alloc(c, (size_t)nbw16 * L.S * sizeof(int16_t)));
+            L.windows16() ? nullptr : static_cast<int16_t*>(dev_alloc(c, (size_t)nbw16 * L.S * sizeof(int16_t)));
         int* d_index = static_cast<int*>(dev_alloc(c, (size_t)max_n * sizeof(int)));
         int64_t* d_cells = static_cast<int64_t*>(dev_alloc(c, (size_t)max_nf * sizeof(int64_t)));
         unsigned long long* d_counts = static_cast<unsigned long long*>(dev_alloc(c, 2 * sizeof(unsigned long long)));
@@ -1092,18 +1103,18 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
         for (const auto& cs : c->cases) {
             ok_rm = ok_rm && !cs.periodic_x && cs.nx <= kRowMaskMaxNx && cs.ny <= kRowMaskMaxNy &&
                     cs.nz <= kRowMaskMaxNz;
-            entries += (int64_t)cs.ny * cs.nz * (L.tiled ? (cs.nx + 15) / 16 : (cs.nx + 31) / 32);
+            entries += (int64_t)cs.ny * cs.nz * (L.windows16() ? (cs.nx + 15) / 16 : (cs.nx + 31) / 32);
         }
         ok_rm = ok_rm && entries < (int64_t)std::numeric_limits<int>::max();
         if (ok_rm) {
             std::vector<uint32_t> code((size_t)L.S, 0xFFFFFFFFu);
-            std::vector<uint4> tab(L.tiled ? 0 : (size_t)entries);
-            std::vector<uint2> tab16(L.tiled ? (size_t)entries : 0);
+            std::vector<uint4> tab(L.windows16() ? 0 : (size_t)entries);
+            std::vector<uint2> tab16(L.windows16() ? (size_t)entries : 0);
             int64_t next_tab = 0;
             for (int k = 0; k < n_cases; ++k) {
                 CaseHost& cs = c->cases[k];
                 const int words32 = (cs.nx + 31) / 32;
-                cs.wpr = L.tiled ? (cs.nx + 15) / 16 : words32;
+                cs.wpr = L.windows16() ? (cs.nx + 15) / 16 : words32;
                 cs.tab = (int)next_tab;
                 next_tab += (int64_t)cs.ny * cs.nz * cs.wpr;
                 for (int li = 0; li < cs.nf; ++li) {
@@ -1120,7 +1131,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
                     const int* row = index_of[k].data() + (int64_t)r * cs.nx;
                     for (int x = 0; x < cs.nx; ++x)
                         if (row[x] >= 0) words[(size_t)(x >> 5) + 1] |= 1u << (x & 31);
-                    if (L.tiled) {   // windows of 32 voxels, one every 16 (lbms_step_tile.cuh)
+                    if (L.windows16()) {   // windows of 32 voxels, one every 16 (lbms_step_tile.cuh)
                         for (int w = 0; w < cs.wpr; ++w) {
                             const uint64_t two = (w & 1) ? ((uint64_t)words[(w >> 1) + 2] << 32) | words[(w >> 1) + 1]
                                                          : ((uint64_t)words[(w >> 1) + 1] << 32) | words[w >> 1];
@@ -1145,13 +1156,13 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
                 if (count != cs.base + cs.nf) return bail(fail(c, LBMS_EINVAL, "case %d: row table count mismatch", k));
             }
             L.b.cell_code = static_cast<uint32_t*>(dev_alloc(c, (size_t)L.S * sizeof(uint32_t)));
-            L.b.rowtab = static_cast<uint4*>(dev_alloc(c, (size_t)std::max<int64_t>(entries, 1) * (L.tiled ? sizeof(uint2) : sizeof(uint4))));
+            L.b.rowtab = static_cast<uint4*>(dev_alloc(c, (size_t)std::max<int64_t>(entries, 1) * (L.windows16() ? sizeof(uint2) : sizeof(uint4))));
             if (!L.b.cell_code || !L.b.rowtab) return bail(fail(c, LBMS_ENOMEM, "row-bitmask tables"));
             e = cudaMemcpyAsync(L.b.cell_code, code.data(), code.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
                                 c->stream);
             if (e == cudaSuccess && entries)
-                e = cudaMemcpyAsync(L.b.rowtab, L.tiled ? (const void*)tab16.data() : tab.data(),
-                                    (size_t)entries * (L.tiled ? sizeof(uint2) : sizeof(uint4)), cudaMemcpyHostToDevice,
+                e = cudaMemcpyAsync(L.b.rowtab, L.windows16() ? (const void*)tab16.data() : tab.data(),
+                                    (size_t)entries * (L.windows16() ? sizeof(uint2) : sizeof(uint4)), cudaMemcpyHostToDevice,
                                     c->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             if (e != cudaSuccess) return bail(cuda_fail(c, e, "upload of the row-bitmask tables"));

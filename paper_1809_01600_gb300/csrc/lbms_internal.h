@@ -42,10 +42,15 @@ constexpr int kTilePrefetch = 160;      // 24,320 cells on 152 SMs
 constexpr int tile_min_blocks(int dim, int precision) {
     return dim == 2 ? (precision == 1 ? 12 : 8) : (precision == 0 ? 5 : (precision == 1 ? 10 : 8));
 }
-// Below this many cells a launch does not fill the GPU (5 blocks of 64 cells
-// on each of 152 SMs) and the autotuned variants are the faster step: 26 k
-// cells in FP32 take 4.6 us against 5.5.
-constexpr int kTileMinCells = 48640;
+// Below this many cells (4 blocks of 64 on each of 152 SMs) a launch does not
+// fill the GPU and the small handles' step is the faster: 37 k cells in FP32
+// take 4.0 us, 46 k with the tiled step 4.7 (26 k: 3.9 against 5.5).
+constexpr int kTileMinCells = 38913;
+
+// Steps of handles that do not fill the GPU (lbms_step_small.cuh): many steps
+// of a block per case of at most 64, 128 or 320 cells, or a launch a step.
+enum { kNotSmall = 0, kBlock64, kBlock128, kBlock320, kSmall };
+constexpr int kBlockSteps = 65536;   // steps of one launch at most
 
 // Limits of the per-cell coordinate word of kNbRowMask (x | y << 11 | z << 21).
 constexpr int kRowMaskMaxNx = 2048, kRowMaskMaxNy = 1024, kRowMaskMaxNz = 2048;
@@ -89,6 +94,8 @@ struct Launch {
     int nblk[kStepVariants] = {};
     int variant = 0;                   // chosen step-kernel tile shape
     bool tiled = false;                // the step of lbms_step_tile.cuh and its population layout, instead of a variant
+    int small = kNotSmall;             // which of the small handles' steps, instead of a variant
+    bool windows16() const { return tiled || small != kNotSmall; }   // the row table's form (no 16-bit table then)
     int cur = 0;                       // lattice holding the latest post-collision state
     DevBuffers b;
     double D12 = 1, D13 = 1, D23 = 1;  // lattice binary diffusivities
@@ -132,6 +139,12 @@ cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st);
 cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream_t st);
 // the default step (lbms_step_tile.cuh); needs L.tiled
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
+// the step for a handle whose largest case has max_nf cells, or kNotSmall;
+// L.ncells and sm_count are set
+int choose_small(const Launch& L, int max_nf);
+cudaError_t launch_step_small(const Launch& L, cudaStream_t st);
+// n <= kBlockSteps steps of a kBlock* handle; cur turns n & 1 times
+cudaError_t launch_steps_block(const Launch& L, int n, cudaStream_t st);
 cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st);
 cudaError_t launch_fields(const Launch& L, cudaStream_t st);
 // X of species s, s + 1, ... (`count` of them) of a case's cells [base, base + nf)

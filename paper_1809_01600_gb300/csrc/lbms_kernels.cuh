@@ -49,6 +49,7 @@ struct MsConst {
     int reacting[3];      // nu_i != 0 (Eq. 24 applies); 0: inert, mixture value
     T tau_min, tau_max;
     int drift;            // 1: drift velocity carries the Maxwell-Stefan flux tau does not
+    T it_min, it_max;     // 1 / tau_min, 1 / tau_max
     int grad_forward;     // 1: Eq. 35 literally (forward difference along x only)
     int outlet_extrap;    // 1: outlet as an extrapolated wet node (Eq. 37 reading), per-cell kernel only
 };
@@ -386,6 +387,86 @@ __device__ __forceinline__ void ms_relax(const T (&X)[3], const T (&gs)[DIM], co
     } else {
 #pragma unroll
         for (int d = 0; d < DIM; ++d) v[d] = T(0);
+    }
+}
+
+// What a collision needs of the coupling of species s: 1 / tau and the drift
+// velocity.  FP64: the quotients of ms_flux, ms_relax and 1 / tau through one
+// reciprocal of the product of their denominators (the FP64 pipe bounds the
+// FP64 steps, and a division costs it about ten operations).
+template <typename T, int DIM>
+__device__ __forceinline__ void ms_couple(const T (&X)[3], const T (&g)[3][DIM], const T (&gs)[DIM],
+                                          const MsConst<T>& c, int s, T& it, T (&v)[DIM]) {
+    T J[DIM], tau, xinv;
+    ms_flux<T, DIM>(X, g, c, s, J);
+    ms_relax<T, DIM>(X, gs, J, c, s, tau, v, xinv);
+    it = Arith<T>::div(T(1), tau);
+}
+template <int DIM>
+__device__ __forceinline__ void ms_couple(const double (&X)[3], const double (&g)[3][DIM], const double (&gs)[DIM],
+                                          const MsConst<double>& c, int s, double& it, double (&v)[DIM]) {
+    const double B11 = X[0] * c.i13 + X[1] * c.i12 + X[2] * c.i13;
+    const double B12 = -X[0] * (c.i12 - c.i13);
+    const double B21 = -X[1] * (c.i12 - c.i23);
+    const double B22 = X[1] * c.i23 + X[0] * c.i12 + X[2] * c.i23;
+    const double det0 = B11 * B22 - B12 * B21;
+    const double Xs = s == 0 ? X[0] : (s == 1 ? X[1] : X[2]);
+    double num = 1.0, den0;      // D_s = num / den
+    if (c.reacting[s]) {
+        den0 = c.a[s][0] * X[0] + c.a[s][1] * X[1] + c.a[s][2] * X[2];
+    } else {
+        num = (s == 0 ? X[1] + X[2] : (s == 1 ? X[0] + X[2] : X[0] + X[1])) + kMixDelta;
+        den0 = (s == 0 ? X[1] * c.i12 + X[2] * c.i13
+                       : (s == 1 ? X[0] * c.i12 + X[2] * c.i23 : X[0] * c.i13 + X[1] * c.i23)) +
+               kMixDelta * c.h[s];
+    }
+    const double d30 = s == 2 ? X[0] * c.i13 + X[1] * c.i23 : 1.0;
+    const bool det_ok = det0 > 0.0, den_ok = den0 > 0.0, d3_ok = d30 > 0.0;
+    const double det = det_ok ? det0 : 1.0, den = den_ok ? den0 : 1.0, d3 = d3_ok ? d30 : 1.0;
+    const double e2 = 3.0 * num + 0.5 * den;                // tau = e2 / den
+    const double xq = Xs * Xs + kEpsX * kEpsX;
+    const double p1 = det * den, p2 = e2 * xq, p1d = p1 * d3;
+    const double R = 1.0 / (p1d * p2);
+    const double Rp2 = R * p2, Rp1 = R * p1d;
+    const double idet = det_ok ? Rp2 * (den * d3) : 0.0;
+    const double xinv = Xs * (Rp1 * e2);
+    double Dt;
+    if (!den_ok || e2 > c.tau_max * den) {
+        it = c.it_max;
+        Dt = (c.tau_max - 0.5) * (1.0 / 3.0);
+    } else if (e2 < c.tau_min * den) {
+        it = c.it_min;
+        Dt = (c.tau_min - 0.5) * (1.0 / 3.0);
+    } else {
+        it = den * (Rp1 * xq);
+        Dt = num * (Rp2 * (det * d3));
+    }
+    if (!c.drift) {
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) v[a] = 0.0;
+        return;
+    }
+    double vn2 = 0.0;
+    const double id3 = d3_ok ? Rp2 * p1 : 0.0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        double J;
+        if (s == 0) {
+            J = -(B22 * g[0][a] - B12 * g[1][a]) * idet;
+        } else if (s == 1) {
+            J = -(B11 * g[1][a] - B21 * g[0][a]) * idet;
+        } else {
+            const double j1 = -(B22 * g[0][a] - B12 * g[1][a]) * idet;
+            const double j2 = -(B11 * g[1][a] - B21 * g[0][a]) * idet;
+            J = (-g[2][a] + X[2] * (j1 * c.i13 + j2 * c.i23)) * id3;
+        }
+        v[a] = (J + Dt * gs[a]) * xinv;
+        vn2 += v[a] * v[a];
+    }
+    if (vn2 > kVMax * kVMax) {
+        const double sc = kVMax * rsqrt(vn2);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) v[a] *= sc;
     }
 }
 

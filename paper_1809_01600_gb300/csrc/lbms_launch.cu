@@ -135,6 +135,7 @@ cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st) {
     LBMS_STEP_DISPATCH(false);
 }
 cudaError_t launch_step(const Launch& L, cudaStream_t st) {
+    if (L.small) return launch_step_small(L, st);
     return L.tiled ? launch_step_tile(L, st) : launch_step_variant(L, L.variant, st);
 }
 

@@ -32,6 +32,8 @@ MsConst<T> make_const(const Launch& L) {
     }
     c.tau_min = T(L.tau_min);
     c.tau_max = T(L.tau_max);
+    c.it_min = T(1.0 / L.tau_min);
+    c.it_max = T(1.0 / L.tau_max);
     c.drift = L.drift;
     c.grad_forward = L.grad_forward;
     c.outlet_extrap = L.outlet_extrap;
