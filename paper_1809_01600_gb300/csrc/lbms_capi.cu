@@ -509,11 +509,18 @@ lbms_status read_case_out(lbms_ctx* c, size_t offset, size_t n) {
     return LBMS_OK;
 }
 
+// Waits for the residual sums, which the kernel leaves in host_out itself.
+lbms_status wait_case_sums(lbms_ctx* c) {
+    CK(cudaStreamSynchronize(c->stream), "reduction");
+    c->d2h += (size_t)c->L.n_cases * 10 * sizeof(double);
+    return LBMS_OK;
+}
+
 // Per-case residuals (refreshing the snapshots); LBMS_EUNSTABLE on NaN/Inf.
 lbms_status case_residuals(lbms_ctx* c, int K, double* r) {
     const int n = c->L.n_cases;
     CK(launch_case_residuals(c->L, 1, c->stream), "residual kernels");
-    lbms_status st = read_case_out(c, 0, (size_t)n * 10);
+    lbms_status st = wait_case_sums(c);
     if (st != LBMS_OK) return st;
     bool bad = false;
     for (int k = 0; k < n; ++k) {
@@ -597,7 +604,7 @@ lbms_status extrap_begin(lbms_ctx* c, Extrapolator& ex) {
 lbms_status extrap_check(lbms_ctx* c, Extrapolator& ex) {
     const int n = c->L.n_cases;
     CK(launch_case_extrap_norms(c->L, c->stream), "extrapolation norms");
-    lbms_status st = read_case_out(c, 0, (size_t)n * 10);
+    lbms_status st = wait_case_sums(c);
     if (st != LBMS_OK) return st;
     for (int k = 0; k < n; ++k) {
         const double* o = c->host_out + (size_t)k * 10;
@@ -1039,8 +1046,10 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
     L.b.coef = static_cast<double*>(dev_alloc(c, (size_t)n_cases * sizeof(double)));
     L.b.partials = static_cast<double*>(dev_alloc(c, segs.size() * 10 * sizeof(double)));
     L.b.case_out = static_cast<double*>(dev_alloc(c, (size_t)n_cases * kCaseOutSlots * sizeof(double)));
+    L.b.case_out_host = c->host_out;
+    L.b.seg_done = static_cast<unsigned int*>(dev_alloc(c, (size_t)n_cases * sizeof(unsigned int)));
     bool ok = L.b.f[0] && L.b.f[1] && L.b.X[0] && L.b.X[1] && L.b.snap && L.b.nbr && L.b.rows && L.b.case_rows &&
-              L.b.cases && L.b.segs && L.b.case_segs && L.b.seg_case && L.b.coef && L.b.partials && L.b.case_out;
+              L.b.cases && L.b.segs && L.b.case_segs && L.b.seg_case && L.b.coef && L.b.partials && L.b.case_out && L.b.seg_done;
     for (int v = 0; v < kStepVariants; ++v) ok = ok && L.b.blk_case[v];
     if (!ok) return bail(fail(c, LBMS_ENOMEM, "device allocation of %zu bytes failed", 2 * fbytes + 2 * xbytes + sbytes));
 
@@ -1189,6 +1198,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMemsetAsync(L.b.X[k], 0, xbytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(L.b.snap, 0, sbytes, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(L.b.cases, 0, cbytes, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(L.b.seg_done, 0, (size_t)n_cases * sizeof(unsigned int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "upload of the neighbour table"));
     for (int k = 0; k < n_cases && st == LBMS_OK; ++k) st = upload_case_bc(c, k);
@@ -1436,7 +1446,7 @@ lbms_status lbms_boundary_flux(lbms_ctx* c, double* inlet_flux, double* totals) 
     }
     if (totals) {
         CK(launch_case_residuals(c->L, 0, c->stream), "sum kernels");
-        lbms_status st = read_case_out(c, 0, (size_t)c->L.n_cases * 10);
+        lbms_status st = wait_case_sums(c);
         if (st != LBMS_OK) return st;
         for (int s = 0; s < 3; ++s) totals[s] = c->host_out[6 + s];
     }

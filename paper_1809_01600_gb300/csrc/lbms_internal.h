@@ -79,6 +79,8 @@ struct DevBuffers {
     double* rre_out = nullptr;         // [cases][order (order + 1) / 2] Gram matrices (lazy)
     double* rre_coef = nullptr;        // [cases][order] coefficients of the differences (lazy)
     double* case_out = nullptr;        // [cases][10] residual sums, then [cases][6] boundary sums
+    double* case_out_host = nullptr;   // pinned: the residual sums again, written by the kernel
+    unsigned int* seg_done = nullptr;  // [cases] finished segments of the running reduction, 0 between reductions
     void* fields = nullptr;            // [3 + 3 dim][S] of tau and u (lazy), FP64 or FP32
     double* dense = nullptr;           // X on the dense grid of the largest case (lazy)
 };

@@ -990,37 +990,60 @@ __device__ __forceinline__ void reduce_to_out(double (&acc)[NV], double* __restr
 constexpr int kSegCells = 1024;
 constexpr int kSegThreads = 256;
 
+// Sums of v[0 .. N) over the warp by halving: in each of the five rounds a
+// lane keeps one half of its values and adds the other lane's, so N values
+// take about N + 4 additions instead of 5 N.  Lane with cnt = 1 holds value idx.
+template <int N, int O>
+__device__ __forceinline__ void warp_fold(double* v, int lane, int& idx, int& cnt) {
+    constexpr int H = (N + 1) / 2;
+    const bool up = lane & O;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const double lo = v[i], hi = i + H < N ? v[i + H] : 0.0;
+        const double send = up ? lo : hi;
+        v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    idx += up ? H : 0;
+    cnt = up ? max(cnt - H, 0) : min(cnt, H);
+    if constexpr (O > 1) warp_fold<H, O / 2>(v, lane, idx, cnt);
+}
+
+// Sums acc over the block's first `used` threads (the rest hold zeros) into
+// dst, thread v the v-th; all threads call.  The FP64 pipe bounds it: as 5 NV
+// shuffled additions a thread the ten sums of a residual took 3 us of an SM,
+// twice; halving them and skipping idle warps leaves a quarter.
 template <int NV>
-__device__ __forceinline__ void block_sum(double (&acc)[NV], double* __restrict__ dst) {
+__device__ __forceinline__ void block_sum(double (&acc)[NV], int used, double* __restrict__ dst) {
     __shared__ double sm[kSegThreads / 32][NV];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        double a = acc[v];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) sm[warp][v] = a;
+    const int warps = (min(used, kSegThreads) + 31) / 32;
+    if (warp < warps) {
+        int idx = 0, cnt = NV;
+        static_assert(NV <= 32, "a lane is left with one value at most");
+        warp_fold<NV, 16>(acc, lane, idx, cnt);
+        if (cnt) sm[warp][idx] = acc[0];
     }
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            double a = lane < kSegThreads / 32 ? sm[lane][v] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-            if (lane == 0) dst[v] = a;
-        }
+    if (threadIdx.x < NV) {
+        double a = 0.0;
+        for (int w = 0; w < warps; ++w) a += sm[w][threadIdx.x];
+        dst[threadIdx.x] = a;
     }
 }
 
-// Residual partials of one segment (NV = 10: sum (X - snap)^2, sum X^2,
-// sum X per species, count of non-finite X); the snapshot takes X when
-// update != 0.
+// Residual sums (NV = 10: sum (X - snap)^2, sum X^2, sum X per species, count
+// of non-finite X); the snapshot takes X when update != 0.  One block per
+// segment; the last block of a case to finish sums the case's partials in
+// order (as seg_finalize_kernel does) into out[case][10] and the host's copy,
+// so that a residual is one launch and no copy.  done[case] counts the
+// finished segments and returns to 0.
 template <typename XS>
-__global__ void __launch_bounds__(kSegThreads) seg_residual_kernel(const XS* __restrict__ X, double* __restrict__ snap,
-                                                                   int64_t S, const int2* __restrict__ segs, int update,
-                                                                   double* __restrict__ partials) {
+__global__ void __launch_bounds__(kSegThreads) seg_residual_kernel(
+    const XS* __restrict__ X, double* __restrict__ snap, int64_t S, const int2* __restrict__ segs,
+    const int* __restrict__ seg_case, const int2* __restrict__ case_segs, int update, double* partials,
+    unsigned int* __restrict__ done, double* out, double* host_out) {
+    __shared__ bool last;
     const int2 sg = segs[blockIdx.x];   // (first cell, cell count)
     double acc[10];
 #pragma unroll
@@ -1038,7 +1061,27 @@ __global__ void __launch_bounds__(kSegThreads) seg_residual_kernel(const XS* __r
             if (update) snap[s * S + i] = x;
         }
     }
-    block_sum<10>(acc, partials + (int64_t)blockIdx.x * 10);
+    block_sum<10>(acc, sg.y, partials + (int64_t)blockIdx.x * 10);
+    const int cs = seg_case[blockIdx.x];
+    const int2 r = case_segs[cs];
+    if (threadIdx.x < 10) __threadfence();   // the partials' writers
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&done[cs], 1u) + 1u == (unsigned int)r.y;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int v = 0; v < 10; ++v) acc[v] = 0.0;
+    for (int j = threadIdx.x; j < r.y; j += kSegThreads) {
+#pragma unroll
+        for (int v = 0; v < 10; ++v) acc[v] += __ldcg(partials + (int64_t)(r.x + j) * 10 + v);
+    }
+    block_sum<10>(acc, r.y, out + (int64_t)cs * 10);
+    if (threadIdx.x == 0) done[cs] = 0u;
+    if (threadIdx.x < 10) host_out[(int64_t)cs * 10 + threadIdx.x] = out[(int64_t)cs * 10 + threadIdx.x];
 }
 
 // Sums the partials of each case's segments [first, first + count) in order.
@@ -1053,7 +1096,7 @@ __global__ void seg_finalize_kernel(const double* __restrict__ partials, const i
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v] += partials[(int64_t)(r.x + j) * NV + v];
     }
-    block_sum<NV>(acc, out + (int64_t)blockIdx.x * NV);
+    block_sum<NV>(acc, r.y, out + (int64_t)blockIdx.x * NV);
 }
 
 // Boundary sums of each case (one block per case, rows [first, first + count)
@@ -1102,7 +1145,7 @@ __global__ void __launch_bounds__(kSegThreads) case_boundary_kernel(
             for (int s = 0; s < 3; ++s) acc[3 + s] += Xv<XS>::own(X, S, s, io).to_double();
         }
     }
-    block_sum<6>(acc, out + (int64_t)blockIdx.x * 6);
+    block_sum<6>(acc, rr.y, out + (int64_t)blockIdx.x * 6);
 }
 
 // Extrapolation of the slowest decay mode for segment blockIdx.x of case
@@ -1182,7 +1225,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_gram_kernel(const double* __r
                 for (int b = a; b < M; ++b) acc[v++] += u[a] * u[b];
         }
     }
-    block_sum<NV>(acc, partials + (int64_t)blockIdx.x * NV);
+    block_sum<NV>(acc, sg.y, partials + (int64_t)blockIdx.x * NV);
 }
 
 // X += sum_a c_a u_a with the case's coefficients coef[case * M + a], in both

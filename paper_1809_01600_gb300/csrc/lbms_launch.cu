@@ -64,24 +64,12 @@ cudaError_t fields_t(const Launch& L, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// sums against `ref` into case_out[c * 10 + v] and the host's copy of it
 template <typename XS>
-cudaError_t residual_t(const Launch& L, int update, cudaStream_t st) {
-    seg_residual_kernel<XS><<<L.n_segs, kSegThreads, 0, st>>>(static_cast<const XS*>(L.b.X[L.cur]), L.b.snap, L.S,
-                                                              L.b.segs, update, L.b.partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // per-case sums land in case_out[c * 10 + v]
-    seg_finalize_kernel<10><<<L.n_cases, kSegThreads, 0, st>>>(L.b.partials, L.b.case_segs, L.b.case_out);
-    return cudaGetLastError();
-}
-
-template <typename XS>
-cudaError_t extrap_norms_t(const Launch& L, cudaStream_t st) {
-    seg_residual_kernel<XS><<<L.n_segs, kSegThreads, 0, st>>>(static_cast<const XS*>(L.b.X[L.cur]), L.b.extrap, L.S,
-                                                              L.b.segs, 0, L.b.partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    seg_finalize_kernel<10><<<L.n_cases, kSegThreads, 0, st>>>(L.b.partials, L.b.case_segs, L.b.case_out);
+cudaError_t residual_t(const Launch& L, double* ref, int update, cudaStream_t st) {
+    seg_residual_kernel<XS><<<L.n_segs, kSegThreads, 0, st>>>(static_cast<const XS*>(L.b.X[L.cur]), ref, L.S, L.b.segs,
+                                                              L.b.seg_case, L.b.case_segs, update, L.b.partials,
+                                                              L.b.seg_done, L.b.case_out, L.b.case_out_host);
     return cudaGetLastError();
 }
 
@@ -179,7 +167,7 @@ cudaError_t launch_put_x(const Launch& L, int base, int nf, const double* values
 }
 
 cudaError_t launch_case_extrap_norms(const Launch& L, cudaStream_t st) {
-    return L.precision == 0 ? extrap_norms_t<double>(L, st) : extrap_norms_t<float>(L, st);
+    return L.precision == 0 ? residual_t<double>(L, L.b.extrap, 0, st) : residual_t<float>(L, L.b.extrap, 0, st);
 }
 
 cudaError_t launch_extrapolate(const Launch& L, cudaStream_t st) {
@@ -243,7 +231,7 @@ cudaError_t launch_rre_apply(const Launch& L, int order, cudaStream_t st) {
 }
 
 cudaError_t launch_case_residuals(const Launch& L, int update, cudaStream_t st) {
-    return L.precision == 0 ? residual_t<double>(L, update, st) : residual_t<float>(L, update, st);
+    return L.precision == 0 ? residual_t<double>(L, L.b.snap, update, st) : residual_t<float>(L, L.b.snap, update, st);
 }
 
 }  // namespace lbms
