@@ -1,6 +1,6 @@
-// The products of the 3-D U-Net on the tcgen05 tensor cores: convolutions,
-// input gradients and weight gradients, with what follows each product done
-// on its accumulators.
+// The products of the two networks on the tcgen05 tensor cores: convolutions
+// (the 3-D U-Net), plain products (the pointwise network), input gradients and
+// weight gradients, with what follows each product done on its accumulators.
 //
 // Activations are stored in a layout with a zero halo of one voxel per side,
 // so the neighbour of every interior voxel at tap t = (dz, dy, dx) lies a
@@ -260,7 +260,9 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
             const long long row = m0 + 32 * quarter + lane;
             const bool valid = row < rows;
             int x = 0, y = 0, z = 0, vb = 0;
-            const bool in = KIND != kOutReluBack && KIND != kOutStore && voxel_of(ep.g, row, x, y, z, vb);
+            const bool in = KIND == kOutRelu && NT == 1 ? valid   // a plain layer: every row
+                            : KIND != kOutReluBack && KIND != kOutStore && KIND != kOutHead &&
+                                  voxel_of(ep.g, row, x, y, z, vb);
             const uint32_t taddr = tmem + b * N + ((uint32_t)(32 * quarter) << 16);
             constexpr int kChunks = KIND == kOutHead ? 1 : N / 32;
 #pragma unroll
@@ -278,12 +280,12 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                     uint32_t wv[16];
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
-                        const float a0 = in ? fmaxf(__uint_as_float(u[c]) + __ldg(ep.bias + c0 + c), 0.0f) : 0.0f;
-                        const float a1 = in ? fmaxf(__uint_as_float(u[c + 1]) + __ldg(ep.bias + c0 + c + 1), 0.0f) : 0.0f;
+                        const float a0 = in ? fmaxf(__uint_as_float(u[c]) + __ldg(ep.bias + n0 + c0 + c), 0.0f) : 0.0f;
+                        const float a1 = in ? fmaxf(__uint_as_float(u[c + 1]) + __ldg(ep.bias + n0 + c0 + c + 1), 0.0f) : 0.0f;
                         wv[c / 2] = pack2(a0, a1);
                     }
                     if (valid) {
-                        uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * N + c0);
+                        uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * job.N + n0 + c0);
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
                             dst[q] = make_uint4(wv[4 * q], wv[4 * q + 1], wv[4 * q + 2], wv[4 * q + 3]);
@@ -308,8 +310,8 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                     }
                 } else if constexpr (KIND == kOutReluBack) {
                     float v[32];
-                    const uint4* act = reinterpret_cast<const uint4*>(static_cast<const bf16*>(ep.act) + row * N + c0);
-                    uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * N + c0);
+                    const uint4* act = reinterpret_cast<const uint4*>(static_cast<const bf16*>(ep.act) + row * job.N + n0 + c0);
+                    uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * job.N + n0 + c0);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const uint4 av = valid ? __ldg(act + q) : make_uint4(0u, 0u, 0u, 0u);
@@ -326,7 +328,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                         if (valid) dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                     const float sum = column_sum(v, lane);
-                    atomicAdd(&cs[c0 + lane], sum);
+                    atomicAdd(ntn == 1 ? &cs[c0 + lane] : &ep.gb[n0 + c0 + lane], sum);
                 } else if constexpr (KIND == kOutStore) {
                     if (valid) {
                         float4* dst = reinterpret_cast<float4*>(ep.P + row * N + c0);
@@ -410,13 +412,13 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                             for (int c = 0; c < 3; ++c) {
                                 const float d = (yv[c] - tv[c]) * t.w;
                                 loss += (double)d * d;
-                                gv[c] = 2.0f * ep.inv_n * d;
+                                gv[c] = ep.grad_scale * d;
                                 hs[c] += gv[c];
                             }
                             uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * N);
                             dst[0] = make_uint4(pack2(gv[0], gv[1]), pack2(gv[2], 0.0f), 0u, 0u);
 #pragma unroll
-                            for (int q = 1; q < 4; ++q) dst[q] = make_uint4(0u, 0u, 0u, 0u);
+                            for (int q = 1; q < N / 8; ++q) dst[q] = make_uint4(0u, 0u, 0u, 0u);
                         }
                     }
                 }
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
         if constexpr (KIND == kOutReluBack || KIND == kOutSplit) {
             asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
             const int e = (int)threadIdx.x - 64;
-            if (e < N && (KIND == kOutReluBack || e < ep.w)) atomicAdd(&ep.gb[e], cs[e]);
+            if (e < N && (KIND == kOutReluBack ? ntn == 1 : e < ep.w)) atomicAdd(&ep.gb[e], cs[e]);
         }
         if constexpr (KIND == kOutHead) {
             if (ep.T) {
@@ -436,7 +438,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                     for (int c = 0; c < 3; ++c) hs[c] += __shfl_down_sync(0xffffffffu, hs[c], o);
                 }
                 if (lane == 0) {
-                    atomicAdd(ep.loss, loss * (double)ep.inv_n);
+                    atomicAdd(ep.loss, loss * ep.loss_scale);
 #pragma unroll
                     for (int c = 0; c < 3; ++c) atomicAdd(&ep.gb[c], hs[c]);
                 }
@@ -482,7 +484,7 @@ struct WgradShape {
 template <int RBA, int NBA, int RBB, int NBB, int NT>
 __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ CUtensorMap mapA,
                                                        const __grid_constant__ CUtensorMap mapB, int chunk, int GR,
-                                                       int ST, unsigned int* __restrict__ err,
+                                                       int ST, uint32_t cols, unsigned int* __restrict__ err,
                                                        const __grid_constant__ WgradJob job) {
     using Sh = WgradShape<RBA, NBA, RBB, NBB, NT>;
     constexpr uint32_t idesc = umma_idesc(128, Sh::kN, true);
@@ -497,6 +499,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
     volatile uint32_t* failed = tmem_slot + 1;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int g0 = blockIdx.x * GR;
+    const int n0 = blockIdx.z * Sh::kN;
     const int r0 = blockIdx.y * chunk;
     const int nk = chunk / kWL;
 
@@ -509,7 +512,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
         *failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    if (warp == 0) tmem_alloc(tmem_slot, cols);
     fence_before();
     __syncthreads();
     fence_after();
@@ -535,7 +538,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
                                     (NT == 1 ? (g0 + g) * CA : 0) + c * (RBA / 2),
                                     NT == 1 ? r : r + job.off[3 * (g0 + g)], &full[s]);
                 for (int c = 0; c < NBB; ++c)
-                    tma_load_2d(sa + GR * NBA * Sh::kABlock + c * Sh::kBBlock, &mapB, c * (RBB / 2), r, &full[s]);
+                    tma_load_2d(sa + GR * NBA * Sh::kABlock + c * Sh::kBBlock, &mapB, n0 + c * (RBB / 2), r, &full[s]);
             }
             if (++s == ST) {
                 s = 0;
@@ -599,14 +602,14 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
                     const int d = m * Sh::kTpm + tb;
                     const bool keep = NT == 1 ? (g0 + g) * CA + l < job.C && tb == 0 : d < 3;
                     const long long prow = NT == 1 ? (long long)(g0 + g) * CA + c : (long long)(3 * (g0 + g) + d) * job.C + c;
-                    float4* dst = reinterpret_cast<float4*>(job.P + ((long long)blockIdx.y * K + prow) * Sh::kN);
+                    float4* dst = reinterpret_cast<float4*>(job.P + ((long long)blockIdx.y * K + prow) * job.N + n0);
                     const uint32_t taddr = tmem + g * Sh::kGroupCols + m * Sh::kN + ((uint32_t)(32 * quarter) << 16);
 #pragma unroll
                     for (int n = 0; n < Sh::kN; n += 32) {
                         uint32_t u[32];
                         tmem_ld32(taddr + n, u);
                         tmem_wait_ld();
-                        if (keep) {
+                        if (keep && n0 + n < job.N) {
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
                                 dst[n / 4 + q] = make_float4(__uint_as_float(u[4 * q]), __uint_as_float(u[4 * q + 1]),
@@ -618,7 +621,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 512);
+    if (warp == 0) tmem_dealloc(tmem, cols);
 }
 
 // ------------------------------------------------------------------ launch
@@ -657,10 +660,14 @@ struct WgradK {
         CUtensorMap ma, mb;
         if (!make_map(&ma, j.x, j.C, j.rows, j.C, RBA, kWRows) || !make_map(&mb, j.dz, j.N, j.rows, j.N, RBB, kWL))
             return cudaErrorInvalidValue;
-        const int st_n = Sh::stages(gr);
+        // two CTAs an SM for the plain products of the pointwise network, whose chunks are a few stages long
+        const int nk = j.rows / j.S / kWL;
+        const int st_n = NT == 1 && nk <= 16 ? std::min(3, Sh::stages(gr)) : Sh::stages(gr);
         const int smem = 1024 + st_n * Sh::stage(gr) + 512;
-        wgrad_kernel<RBA, NBA, RBB, NBB, NT>
-            <<<dim3(groups / gr, j.S), 192, smem, st>>>(ma, mb, j.rows / j.S, gr, st_n, err, j);
+        uint32_t cols = 32;
+        while ((int)cols < gr * Sh::kGroupCols) cols *= 2;
+        wgrad_kernel<RBA, NBA, RBB, NBB, NT><<<dim3(groups / gr, j.S, (j.N + Sh::kN - 1) / Sh::kN), 192, smem, st>>>(
+            ma, mb, j.rows / j.S, gr, st_n, cols, err, j);
         return cudaGetLastError();
     }
 };
@@ -671,7 +678,8 @@ struct WgradK {
     F(128, 32, 3, kOutRelu) F(64, 32, 3, kOutReluBack) F(64, 64, 3, kOutSplit) F(128, 64, 3, kOutReluBack) \
     F(128, 128, 3, kOutSplit) F(128, 128, 3, kOutReluBack) F(128, 64, 3, kOutStore)                       \
     F(128, 32, 3, kOutStore) F(128, 128, 1, kOutUp) F(128, 128, 1, kOutReluBack)                          \
-    F(128, 64, 1, kOutReluBack) F(64, 32, 1, kOutHead) F(64, 32, 1, kOutReluBack)
+    F(128, 64, 1, kOutReluBack) F(64, 32, 1, kOutHead) F(64, 32, 1, kOutReluBack)                         \
+    F(128, 64, 1, kOutRelu) F(128, 64, 1, kOutHead)
 #define LBMS_WGRAD_SHAPES(F)                                                                        \
     F(64, 1, 64, 1, 3) F(64, 1, 128, 1, 3) F(128, 1, 64, 1, 3) F(128, 1, 128, 1, 3) F(128, 1, 128, 2, 3) \
     F(128, 2, 128, 1, 3) F(128, 2, 128, 2, 3) F(64, 1, 64, 1, 1) F(128, 2, 128, 1, 1) F(128, 2, 128, 2, 1)
@@ -696,7 +704,7 @@ cudaError_t conv_init() {
 }
 
 cudaError_t umma_conv(const ConvJob& j, unsigned int* err, cudaStream_t st) {
-    cudaError_t e = umma_gemm_init();
+    cudaError_t e = umma_init();
     if (e != cudaSuccess) return e;
     if (j.rows < 1 || (j.C != 32 && (j.C < 64 || j.C % 64)) || !aligned16(j.x) || !aligned16(j.W) ||
         !aligned16(j.ep.out) || !aligned16(j.ep.act) || !aligned16(j.ep.cat) || !aligned16(j.ep.P) ||
@@ -708,7 +716,8 @@ cudaError_t umma_conv(const ConvJob& j, unsigned int* err, cudaStream_t st) {
             j.off[3 * g + 2] != j.off[3 * g] + 2 * dir)
             return cudaErrorInvalidValue;
     const int rb = j.C == 32 ? 64 : 128, nt = j.taps == 27 ? 3 : 1;
-    const int n = j.kind == kOutUp ? 128 : j.N;
+    // columns of a tile: all of them, or 64 (128 for the transposed convolutions) where N is larger
+    const int n = j.kind == kOutUp ? 128 : (j.N == 32 || (j.N == 128 && j.kind != kOutRelu) || nt == 3 ? j.N : 64);
     if (j.N % n || (nt == 3 && rb * n <= 4096 && j.C > 64)) return cudaErrorInvalidValue;
 #define LBMS_TRY(RB, N, NT, KIND) \
     if (rb == RB && n == N && nt == NT && j.kind == KIND) return ConvK<RB, N, NT, KIND>::launch(j, err, st);
@@ -718,7 +727,7 @@ cudaError_t umma_conv(const ConvJob& j, unsigned int* err, cudaStream_t st) {
 }
 
 cudaError_t umma_wgrad(const WgradJob& j, unsigned int* err, cudaStream_t st) {
-    cudaError_t e = umma_gemm_init();
+    cudaError_t e = umma_init();
     if (e != cudaSuccess) return e;
     if (j.rows < kWL || j.S < 1 || j.S > 65535 || j.rows % j.S || (j.rows / j.S) % kWL || !aligned16(j.x) ||
         !aligned16(j.dz) || !aligned16(j.P) || (j.taps != 27 && j.taps != 1))
@@ -726,9 +735,11 @@ cudaError_t umma_wgrad(const WgradJob& j, unsigned int* err, cudaStream_t st) {
     for (int g = 0; g < 9 && j.taps == 27; ++g)
         if (j.off[3 * g + 1] != j.off[3 * g] + 1 || j.off[3 * g + 2] != j.off[3 * g] + 2) return cudaErrorInvalidValue;
     const int nt = j.taps == 27 ? 3 : 1;
-    const int rba = j.C == 32 ? 64 : 128, nba = j.C == 32 || j.C == 64 ? 1 : 2;
-    const int rbb = j.N == 32 ? 64 : 128, nbb = j.N == 128 ? 2 : 1;
-    if (j.C % (rba / 2 * nba) || (j.N != 32 && j.N != 64 && j.N != 128) || (nt == 3 && j.C > 128))
+    // a plain product takes any multiple of 64 channels in tiles of 128 (those past C or N read as zero)
+    const int rba = j.C == 32 ? 64 : 128, nba = j.C == 32 || (j.C == 64 && nt == 3) ? 1 : 2;
+    const int rbb = j.N == 32 ? 64 : 128, nbb = j.N > 64 ? 2 : 1;
+    if ((j.C != 32 && j.C % 64) || (j.N != 32 && j.N % 64) || j.C < 32 || j.N < 32 ||
+        (nt == 3 && (j.C > 128 || j.N > 128 || j.C % (rba / 2 * nba) || j.N % (rbb / 2 * nbb))))
         return cudaErrorInvalidValue;
 #define LBMS_TRY(A, NA, B, NB, NT) \
     if (rba == A && nba == NA && rbb == B && nbb == NB && nt == NT) return WgradK<A, NA, B, NB, NT>::launch(j, err, st);

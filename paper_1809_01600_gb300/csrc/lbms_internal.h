@@ -179,18 +179,11 @@ cudaError_t launch_build_neighbours(int dim, const int64_t* fluid_cell, const in
                                     unsigned long long* counts, cudaStream_t st);
 cudaError_t launch_fill16(int16_t* p, int64_t n, int16_t v, cudaStream_t st);
 
-// BF16 "TN" matrix product of the warm-start network on the tcgen05 tensor
-// cores (lbms_umma.cu): P[z][M][N] = A[M][K chunk z] . B[N][K chunk z]^T,
-// FP32.  Needs N a multiple of 64, (K / S) a multiple of 64, 16-byte aligned
-// operands with row strides a multiple of 8 elements; M is free.  *err is
-// raised if a wait in the kernel timed out.
-cudaError_t umma_gemm_init();
-bool umma_gemm_supported(const void* A, int lda, const void* B, int ldb, int M, int N, int K, int S);
-cudaError_t umma_gemm_tn(const void* A, int lda, const void* B, int ldb, float* P, int M, int N, int K, int S,
-                         unsigned int* err, cudaStream_t st);
+// Readies the tcgen05 kernels (lbms_umma.cu); the error if the device or driver lacks what they need.
+cudaError_t umma_init();
 
-// Products of the 3-D U-Net (lbms_conv.cu).  Activations are BF16 rows
-// [row][C] of a zero-halo layout: volumes of X x Y x Z voxels in Xp x Yp x Zp
+// Products of the two networks (lbms_conv.cu).  The U-Net's activations are BF16
+// rows [row][C] of a zero-halo layout: volumes of X x Y x Z voxels in Xp x Yp x Zp
 // rows each, R rows in all.
 struct RowLayout {
     int X = 0, Y = 0, Z = 0, Xp = 1, Yp = 1, Zp = 1;
@@ -199,8 +192,8 @@ struct RowLayout {
 
 // What becomes of the product's FP32 accumulators acc[r][n] (kept in TMEM):
 enum ConvOut {
-    kOutRelu,       // out[r][n] = BF16(relu(acc + bias[n])) on interior rows, 0 elsewhere; with cat, the
-                    //   first w columns also to cat[r][cat_off + n], and 0 to all of cat[r] elsewhere
+    kOutRelu,       // out[r][n] = BF16(relu(acc + bias[n])) on interior rows (taps = 1: all rows), 0 elsewhere;
+                    //   with cat, the first w columns also to cat[r][cat_off + n], and 0 to all of cat[r] elsewhere
     kOutReluBack,   // out[r][n] = BF16(act[r][n] > 0 ? acc : 0), gb[n] += the column sums (before rounding)
     kOutStore,      // P[r][n] = acc
     kOutSplit,      // gradient of a concatenation of two w-wide halves, interior rows: columns [0, w) as BF16 to
@@ -209,8 +202,8 @@ enum ConvOut {
     kOutUp,         // transposed 2x2x2 convolution: column t Cg + n of an interior row, plus bias[n], to the row's
                     //   child t of the finer layout, cat[child][n] (n < w)
     kOutHead        // Y = acc + bias (3 columns): Y[r][4] if given; against T [r][4] = (targets, mask), if given,
-                    //   out[r][n] = BF16(2 inv_n (Y - T) mask) (0 for n >= 3), its column sums into gb and
-                    //   inv_n sum((Y - T)^2 mask^2) into loss
+                    //   out[r][n] = BF16(grad_scale (Y - T) mask) (0 for n >= 3), its column sums into gb and
+                    //   loss_scale sum((Y - T)^2 mask^2) into loss
 };
 struct ConvEpilogue {
     const float* bias = nullptr;
@@ -225,7 +218,8 @@ struct ConvEpilogue {
     const float* T = nullptr;
     float* Y = nullptr;
     double* loss = nullptr;
-    float inv_n = 0.0f;
+    float grad_scale = 0.0f;
+    double loss_scale = 0.0;
     RowLayout g;                  // the product's rows
     RowLayout other;              // kOutSplit: the coarser layout; kOutUp: the finer one
 };
@@ -234,7 +228,9 @@ struct ConvEpilogue {
 // (zeros outside) and W [N][taps C]: a 3x3x3 convolution or its input
 // gradient (taps = 27; the three offsets of a (dz, dy) row consecutive) or a
 // plain product (taps = 1, off[0] = 0).  *err is raised if a wait in the
-// kernel timed out.  cudaErrorInvalidValue for shapes that are not built.
+// kernel timed out.  cudaErrorInvalidValue for shapes that are not built; plain
+// products into kOutRelu, kOutReluBack and kOutHead take every C and N that are
+// multiples of 64 (kOutHead: N = 64).
 struct ConvJob {
     const void* x = nullptr;
     const void* W = nullptr;

@@ -1,14 +1,21 @@
 // Learned warm start (declared in include/lbms_net.h): feature rows of an
 // anode's fluid cells, a pointwise MLP with BF16 tensor-core matrix products
-// (mma.sync m16n8k16, FP32 accumulation), its backward pass and Adam.
+// and FP32 accumulation, its backward pass and Adam.
 //
-// Matrix products are all of one form, P = A . B^T with A [M][K] and B [N][K]
-// both K-contiguous BF16 ("TN"), M and N multiples of 64, K a multiple of 32
-// per split; the forward pass, the input gradients and the weight gradients
-// get that form by keeping transposed copies of the weights and of the
-// activations.  Every size is padded at allocation so that no tile crosses a
-// buffer's end: the kernels need no bounds checks, and the host checks the
-// divisibility before every launch.
+// The products run on the tcgen05 kernels of lbms_conv.cu.  At 8192 rows and
+// width 704 they are small (11 products of 8 GFLOP at most), so what bounds a
+// step is everything around them: bias, ReLU and its gradient, the loss and the
+// bias gradients are taken on a product's accumulators, the weight gradients
+// read both operands as they lie, and Adam is one launch.  A step with its
+// transfers and the gradients: 0.771 ms with a kernel for each of these, 0.376.
+//
+// The mma.sync kernel here (m16n8k16) is what remains when it is forced or
+// tcgen05 is missing: P = A . B^T with A [M][K] and B [N][K] both K-contiguous
+// BF16 ("TN"), M and N multiples of 64, K a multiple of 32 per split; the
+// weight gradients get that form from transposed copies of the activations.
+// Every size is padded at allocation so that no tile crosses a buffer's end:
+// the kernels need no bounds checks, and the host checks the divisibility
+// before every launch.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -17,6 +24,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -237,24 +245,40 @@ __global__ void splitk_sum_kernel(const float* __restrict__ P, int S, int64_t n,
     }
 }
 
-// Adam on the weights of one layer [O][I] (and the refresh of the BF16 copy
-// and its transpose), then on the biases [O].
-__global__ void adam_kernel(float* __restrict__ W, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ G, int64_t n, float lr, float c1, float c2, int O, int I,
-                            bf16* __restrict__ Wb, bf16* __restrict__ WbT) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const float gr = G[e];
-        const float mm = 0.9f * m[e] + 0.1f * gr;
-        const float vv = 0.999f * v[e] + 0.001f * gr * gr;
-        m[e] = mm;
-        v[e] = vv;
-        const float w = W[e] - lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
-        W[e] = w;
-        if (Wb) {
-            const int o = (int)(e / I), i = (int)(e % I);
+// One Adam step (betas 0.9 / 0.999, eps 1e-8) over all parameter arrays of a
+// network in one launch (blockIdx.y: the array), with the BF16 copies of the
+// weights: Wb as stored [O][I]; Wt its transpose [I][O], or for 3x3x3
+// convolutions (ci != 0, I = 27 ci) the flipped weights [ci][27 O].  Launched
+// per array this took 39 launches and 230 us of a U-Net step.
+struct AdamItem {
+    float *p, *m, *v;
+    const float* g;
+    int64_t n;
+    bf16 *Wb, *Wt;
+    int O, I, ci;
+};
+struct AdamList {
+    AdamItem it[26];
+};
+
+__global__ void adam_all_kernel(const __grid_constant__ AdamList list, float lr, float c1, float c2) {
+    const AdamItem& a = list.it[blockIdx.y];
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < a.n; e += (int64_t)gridDim.x * blockDim.x) {
+        const float gr = a.g[e];
+        const float mm = 0.9f * a.m[e] + 0.1f * gr;
+        const float vv = 0.999f * a.v[e] + 0.001f * gr * gr;
+        a.m[e] = mm;
+        a.v[e] = vv;
+        const float w = a.p[e] - lr * (mm * c1) / (sqrtf(vv * c2) + 1e-8f);
+        a.p[e] = w;
+        if (a.Wb) {
+            const int o = (int)(e / a.I), i = (int)(e % a.I);
             const bf16 wb = __float2bfloat16_rn(w);
-            Wb[e] = wb;
-            WbT[(int64_t)i * O + o] = wb;
+            a.Wb[e] = wb;
+            if (a.ci)
+                a.Wt[(int64_t)(i % a.ci) * 27 * a.O + (int64_t)(i / a.ci) * a.O + o] = wb;
+            else
+                a.Wt[(int64_t)i * a.O + o] = wb;
         }
     }
 }
@@ -416,7 +440,7 @@ __global__ void assemble_kernel(const int64_t* __restrict__ cell, int nf, int nx
 
 // X_s = profile_s(x) + Y[j][s] / 100, clamped at 1e-6 and renormalised;
 // out [3][nf] in FP64.
-__global__ void predict_post_kernel(const float* __restrict__ Y, const int64_t* __restrict__ cell, int j0, int rows,
+__global__ void predict_post_kernel(const float* __restrict__ Y, int ld, const int64_t* __restrict__ cell, int j0, int rows,
                                     int nf, int nx, const float* __restrict__ xtab, double* __restrict__ out) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = j0 + r;
@@ -424,7 +448,7 @@ __global__ void predict_post_kernel(const float* __restrict__ Y, const int64_t* 
     const int x = (int)(cell[j] % nx);
     double X[3], s = 0.0;
     for (int q = 0; q < 3; ++q) {
-        double v = (double)xtab[(int64_t)x * 8 + q] + (double)Y[(int64_t)r * kOutPad + q] / kTargetScale;
+        double v = (double)xtab[(int64_t)x * 8 + q] + (double)Y[(int64_t)r * ld + q] / kTargetScale;
         v = v < 1e-6 ? 1e-6 : v;
         X[q] = v;
         s += v;
@@ -445,8 +469,13 @@ struct lbms_net {
     bf16* dzT = nullptr;                    // [max width][kMaxRows]
     float* P = nullptr;                     // GEMM partials
     size_t P_floats = 0;
-    float* Y = nullptr;                     // [kMaxRows][kOutPad]
-    float* T = nullptr;                     // [kMaxRows][4]
+    float* Y = nullptr;                     // output rows, y_ld apart
+    int y_ld = kOutPad;
+    float* T = nullptr;                     // [kMaxRows][4]: targets, 1
+    float* zero = nullptr;                  // the loss and all bias gradients, cleared together
+    size_t zero_bytes = 0;
+    float* flat = nullptr;                  // parameters or gradients in the caller's order
+    std::mutex flat_use;
     double* loss = nullptr;
     bf16* feat = nullptr;                   // training rows [cap][kF]
     float* targ = nullptr;                  // [cap][4]
@@ -503,21 +532,12 @@ int64_t n_params(const lbms_net* n) {
     return s;
 }
 
-// P[z] = A . B^T with the checks the kernel relies on.
-// P = A . B^T on the fifth-generation tensor cores (tcgen05, lbms_umma.cu)
-// whenever the shape allows it; otherwise, or when forced, the mma.sync
-// kernel above.
+// P[z] = A . B^T on the mma.sync kernel, with the checks the kernel relies on.
 lbms_status gemm(lbms_net* n, const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, int S) {
     if ((size_t)S * M * N > n->P_floats)
         return nfail(n, LBMS_EINVAL, "internal GEMM shape %d x %d x %d (split %d) exceeds the partials", M, N, K, S);
-    if (n->gemm_kind != LBMS_NET_GEMM_MMA_SYNC && lbms::umma_gemm_supported(A, lda, B, ldb, M, N, K, S) &&
-        lbms::umma_gemm_init() == cudaSuccess) {
-        NCK(lbms::umma_gemm_tn(A, lda, B, ldb, n->P, M, N, K, S, n->gemm_err, 0), "tensor-core gemm");
-        ++n->tcgen05_calls;
-        return LBMS_OK;
-    }
     if (n->gemm_kind == LBMS_NET_GEMM_TCGEN05)
-        return nfail(n, LBMS_EINVAL, "GEMM %d x %d x %d (split %d) is not supported by the tcgen05 kernel", M, N, K, S);
+        return nfail(n, LBMS_ECUDA, "the tcgen05 kernels are unavailable: %s", cudaGetErrorString(lbms::umma_init()));
     if (M % kTM || N % kTN || K % (kTK * S) || lda % 8 || ldb % 8)
         return nfail(n, LBMS_EINVAL, "internal GEMM shape %d x %d x %d (split %d) not tileable", M, N, K, S);
     gemm_tn_kernel<<<dim3(N / kTN, M / kTM, S), 128>>>(A, lda, B, ldb, n->P, M, N, K / S);
@@ -541,10 +561,56 @@ lbms_status transpose(lbms_net* n, const bf16* in, bf16* out, int R, int C) {
     return LBMS_OK;
 }
 
-// Forward pass of R rows already in act[0]; with `train` the transposed
-// activations are kept for the weight gradients.  Output in n->Y.
+// Whether the passes run on the tensor-core kernels with the work after each
+// product on its accumulators (lbms_conv.cu), which take every shape of the
+// network; the mma.sync kernel, when forced, runs the passes below it one
+// kernel at a time.
+bool fused(const lbms_net* n) { return n->gemm_kind != LBMS_NET_GEMM_MMA_SYNC && lbms::umma_init() == cudaSuccess; }
+
+// A layer's product over R rows: x [R][C] . W [N][C]^T.
+lbms::ConvJob layer_job(const bf16* x, int R, int C, const bf16* W, int N, lbms::ConvOut kind) {
+    lbms::ConvJob j;
+    j.x = x;
+    j.W = W;
+    j.rows = R;
+    j.C = C;
+    j.N = N;
+    j.taps = 1;
+    j.kind = kind;
+    return j;
+}
+
+// Forward pass of R rows already in act[0].  With `train`, what the backward
+// pass needs is kept: fused, the output gradient (dz[0]), its bias gradient
+// and the loss against n->T; else the transposed activations.  Without it the
+// output is in n->Y, y_ld apart.
 lbms_status forward(lbms_net* n, int R, bool train) {
     lbms_status st;
+    if (train) NCK(cudaMemsetAsync(n->zero, 0, n->zero_bytes, 0), "loss and bias grads");
+    if (fused(n)) {
+        for (int l = 0; l < n->layers; ++l) {
+            const bool last = l == n->layers - 1;
+            lbms::ConvJob j = layer_job(n->act[l], R, n->in[l], n->Wb[l], n->out[l], last ? lbms::kOutHead : lbms::kOutRelu);
+            j.ep.bias = n->b[l];
+            if (!last) {
+                j.ep.out = n->act[l + 1];
+            } else if (train) {
+                j.ep.T = n->T;
+                j.ep.grad_scale = 2.0f / (float)(R * kOut);
+                j.ep.loss_scale = 1.0 / (double)(R * kOut);
+                j.ep.out = n->dz[0];
+                j.ep.gb = n->gb[l];
+                j.ep.loss = n->loss;
+            } else {
+                j.ep.Y = n->Y;
+                n->y_ld = 4;
+            }
+            NCK(lbms::umma_conv(j, n->gemm_err, 0), "layer");
+            ++n->tcgen05_calls;
+        }
+        return LBMS_OK;
+    }
+    n->y_ld = kOutPad;
     for (int l = 0; l < n->layers; ++l) {
         const bool last = l == n->layers - 1;
         if (train) {
@@ -562,14 +628,15 @@ lbms_status forward(lbms_net* n, int R, bool train) {
 }
 
 // Backward pass and (lr > 0) Adam step for the R rows of the last forward
-// pass with targets in n->T.  Gradients stay in gW / gb.
+// pass (train) with targets in n->T.  Gradients stay in gW / gb.
 lbms_status backward_step(lbms_net* n, int R, double lr, double* loss) {
     lbms_status st;
-    NCK(cudaMemset(n->loss, 0, sizeof(double)), "loss");
-    for (int l = 0; l < n->layers; ++l) NCK(cudaMemset(n->gb[l], 0, n->out[l] * sizeof(float)), "bias grads");
     const int L = n->layers;
-    loss_grad_kernel<<<R / 64, 256>>>(n->Y, n->T, R, n->dz[0], n->gb[L - 1], n->loss);
-    NCK(cudaGetLastError(), "loss");
+    const bool fast = fused(n);
+    if (!fast) {
+        loss_grad_kernel<<<R / 64, 256>>>(n->Y, n->T, R, n->dz[0], n->gb[L - 1], n->loss);
+        NCK(cudaGetLastError(), "loss");
+    }
     int cur = 0;
     // split of the R-long reduction of the weight gradients: chunks of >= 512
     // rows, a divisor of R / 64 so that every chunk is whole 64-row steps (the
@@ -579,18 +646,41 @@ lbms_status backward_step(lbms_net* n, int R, double lr, double* loss) {
     for (int l = L - 1; l >= 0; --l) {
         const int O = n->out[l], I = n->in[l];
         // weight gradient: dZ^T [O][R] . act^T [I][R]
-        st = transpose(n, n->dz[cur], n->dzT, R, O);
-        if (st != LBMS_OK) return st;
-        st = gemm(n, n->dzT, R, n->actT[l], R, O, I, R, S);
-        if (st != LBMS_OK) return st;
+        if (fast) {
+            lbms::WgradJob j;
+            j.x = n->dz[cur];
+            j.C = O;
+            j.dz = n->act[l];
+            j.N = I;
+            j.rows = R;
+            j.S = S;
+            j.taps = 1;
+            j.P = n->P;
+            NCK(lbms::umma_wgrad(j, n->gemm_err, 0), "weight gradient");
+            ++n->tcgen05_calls;
+        } else {
+            st = transpose(n, n->dz[cur], n->dzT, R, O);
+            if (st != LBMS_OK) return st;
+            st = gemm(n, n->dzT, R, n->actT[l], R, O, I, R, S);
+            if (st != LBMS_OK) return st;
+        }
         splitk_sum_kernel<<<grid_for((int64_t)O * I), 256>>>(n->P, S, (int64_t)O * I, n->gW[l]);
         NCK(cudaGetLastError(), "split-k sum");
         if (l > 0) {
             // input gradient: dZ [R][O] . W^T -> [R][I], then through the ReLU of layer l - 1
-            st = gemm(n, n->dz[cur], O, n->WbT[l], O, R, I, O, 1);
-            if (st != LBMS_OK) return st;
-            relu_back_kernel<<<R / 32, 256>>>(n->P, n->act[l], R, I, n->dz[cur ^ 1], n->gb[l - 1]);
-            NCK(cudaGetLastError(), "relu backward");
+            if (fast) {
+                lbms::ConvJob j = layer_job(n->dz[cur], R, O, n->WbT[l], I, lbms::kOutReluBack);
+                j.ep.act = n->act[l];
+                j.ep.out = n->dz[cur ^ 1];
+                j.ep.gb = n->gb[l - 1];
+                NCK(lbms::umma_conv(j, n->gemm_err, 0), "input gradient");
+                ++n->tcgen05_calls;
+            } else {
+                st = gemm(n, n->dz[cur], O, n->WbT[l], O, R, I, O, 1);
+                if (st != LBMS_OK) return st;
+                relu_back_kernel<<<R / 32, 256>>>(n->P, n->act[l], R, I, n->dz[cur ^ 1], n->gb[l - 1]);
+                NCK(cudaGetLastError(), "relu backward");
+            }
             cur ^= 1;
         }
     }
@@ -598,14 +688,14 @@ lbms_status backward_step(lbms_net* n, int R, double lr, double* loss) {
         ++n->step;
         const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)n->step)));
         const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)n->step)));
+        AdamList list = {};
         for (int l = 0; l < L; ++l) {
-            const int64_t nw = (int64_t)n->out[l] * n->in[l];
-            adam_kernel<<<grid_for(nw), 256>>>(n->W[l], n->mW[l], n->vW[l], n->gW[l], nw, (float)lr, c1, c2,
-                                               n->out[l], n->in[l], n->Wb[l], n->WbT[l]);
-            adam_kernel<<<grid_for(n->out[l]), 256>>>(n->b[l], n->mb[l], n->vb[l], n->gb[l], n->out[l], (float)lr,
-                                                      c1, c2, n->out[l], 1, nullptr, nullptr);
-            NCK(cudaGetLastError(), "adam");
+            const int O = n->out[l], I = n->in[l];
+            list.it[2 * l] = {n->W[l], n->mW[l], n->vW[l], n->gW[l], (int64_t)O * I, n->Wb[l], n->WbT[l], O, I, 0};
+            list.it[2 * l + 1] = {n->b[l], n->mb[l], n->vb[l], n->gb[l], O, nullptr, nullptr, O, 1, 0};
         }
+        adam_all_kernel<<<dim3(152, 2 * L), 256>>>(list, (float)lr, c1, c2);
+        NCK(cudaGetLastError(), "adam");
     }
     if (loss) NCK(cudaMemcpy(loss, n->loss, sizeof(double), cudaMemcpyDeviceToHost), "read loss");
     return LBMS_OK;
@@ -789,7 +879,6 @@ lbms_status lbms_net_create(int width, int depth, uint64_t seed, lbms_net** out)
         n->b.push_back(nalloc<float>(n, n->out[l]));
         n->mb.push_back(nalloc<float>(n, n->out[l]));
         n->vb.push_back(nalloc<float>(n, n->out[l]));
-        n->gb.push_back(nalloc<float>(n, n->out[l]));
         n->Wb.push_back(nalloc<bf16>(n, nw));
         n->WbT.push_back(nalloc<bf16>(n, nw));
         n->act.push_back(nalloc<bf16>(n, (size_t)kMaxRows * n->in[l]));
@@ -803,7 +892,13 @@ lbms_status lbms_net_create(int width, int depth, uint64_t seed, lbms_net** out)
     n->P_floats = pmax;
     n->Y = nalloc<float>(n, (size_t)kMaxRows * kOutPad);
     n->T = nalloc<float>(n, (size_t)kMaxRows * 4);
-    n->loss = nalloc<double>(n, 1);
+    size_t biases = 0;
+    for (int l = 0; l < n->layers; ++l) biases += n->out[l];
+    n->zero_bytes = sizeof(double) + biases * sizeof(float);
+    n->zero = nalloc<float>(n, 2 + biases);
+    n->loss = reinterpret_cast<double*>(n->zero);
+    for (int l = 0, o = 2; l < n->layers; o += n->out[l++]) n->gb.push_back(n->zero ? n->zero + o : nullptr);
+    n->flat = nalloc<float>(n, n_params(n));
     n->gemm_err = nalloc<unsigned int>(n, 1);
     for (void* p : n->allocs) ok = ok && p;
     if (!ok) {
@@ -887,6 +982,7 @@ lbms_status lbms_net_add_sample(lbms_net* n, lbms_ctx* ctx, int k) {
         const int x = (int)(e % v.nx);
         for (int s = 0; s < 3; ++s)
             t[(size_t)j * 4 + s] = (float)(kTargetScale * (X[(size_t)s * v.N + e] - F.prof[(size_t)s * v.nx + x]));
+        t[(size_t)j * 4 + 3] = 1.0f;
     }
     st = grow(n, n->n_rows + v.nf);
     if (st != LBMS_OK) return st;
@@ -935,12 +1031,12 @@ lbms_status lbms_net_forward(lbms_net* n, const uint16_t* features, int rows, fl
     if (st != LBMS_OK) return st;
     st = forward(n, rows, false);
     if (st != LBMS_OK) return st;
-    std::vector<float> y((size_t)rows * kOutPad);
+    std::vector<float> y((size_t)rows * n->y_ld);
     NCK(cudaMemcpy(y.data(), n->Y, y.size() * sizeof(float), cudaMemcpyDeviceToHost), "read output");
     st = check_gemm(n);
     if (st != LBMS_OK) return st;
     for (int r = 0; r < rows; ++r)
-        for (int s = 0; s < kOut; ++s) out[(size_t)r * kOut + s] = y[(size_t)r * kOutPad + s];
+        for (int s = 0; s < kOut; ++s) out[(size_t)r * kOut + s] = y[(size_t)r * n->y_ld + s];
     return LBMS_OK;
 }
 
@@ -950,8 +1046,10 @@ lbms_status lbms_net_train_batch(lbms_net* n, const uint16_t* features, const fl
     lbms_status st = upload_rows(n, features, rows);
     if (st != LBMS_OK) return st;
     std::vector<float> t((size_t)rows * 4, 0.0f);
-    for (int r = 0; r < rows; ++r)
+    for (int r = 0; r < rows; ++r) {
         for (int s = 0; s < kOut; ++s) t[(size_t)r * 4 + s] = targets[(size_t)r * kOut + s];
+        t[(size_t)r * 4 + 3] = 1.0f;
+    }
     NCK(cudaMemcpy(n->T, t.data(), t.size() * sizeof(float), cudaMemcpyHostToDevice), "targets");
     st = forward(n, rows, true);
     if (st != LBMS_OK) return st;
@@ -965,7 +1063,7 @@ lbms_status lbms_net_set_gemm(lbms_net* n, int kind) {
     if (!n || (kind != LBMS_NET_GEMM_AUTO && kind != LBMS_NET_GEMM_TCGEN05 && kind != LBMS_NET_GEMM_MMA_SYNC))
         return LBMS_EINVAL;
     if (kind == LBMS_NET_GEMM_TCGEN05) {
-        const cudaError_t e = lbms::umma_gemm_init();
+        const cudaError_t e = lbms::umma_init();
         if (e != cudaSuccess) return nfail(n, LBMS_ECUDA, "tcgen05 GEMM unavailable: %s", cudaGetErrorString(e));
     }
     n->gemm_kind = kind;
@@ -984,15 +1082,21 @@ lbms_status lbms_net_get(const lbms_net* cn, int what, float* buf, int64_t count
     if (!n || !buf || (what != 0 && what != 1)) return LBMS_EINVAL;
     if (count < n_params(n)) return nfail(n, LBMS_EINVAL, "buffer holds %lld floats, need %lld", (long long)count,
                                           (long long)n_params(n));
+    // gathered on the device, one copy to the host
+    const std::lock_guard<std::mutex> hold(n->flat_use);
     int64_t off = 0;
+    auto take = [&](const float* p, size_t count) {
+        const cudaError_t e =
+            cudaMemcpyAsync(n->flat + off, p, count * sizeof(float), cudaMemcpyDeviceToDevice, 0);
+        off += (int64_t)count;
+        return e;
+    };
     for (int l = 0; l < n->layers; ++l) {
         const int o = l == n->layers - 1 ? kOut : n->out[l];
-        const size_t nw = (size_t)o * n->in[l];   // the first o rows of [out][in]
-        NCK(cudaMemcpy(buf + off, what ? n->gW[l] : n->W[l], nw * sizeof(float), cudaMemcpyDeviceToHost), "get");
-        off += nw;
-        NCK(cudaMemcpy(buf + off, what ? n->gb[l] : n->b[l], o * sizeof(float), cudaMemcpyDeviceToHost), "get");
-        off += o;
+        NCK(take(what ? n->gW[l] : n->W[l], (size_t)o * n->in[l]), "get");   // the first o rows of [out][in]
+        NCK(take(what ? n->gb[l] : n->b[l], o), "get");
     }
+    NCK(cudaMemcpy(buf, n->flat, (size_t)off * sizeof(float), cudaMemcpyDeviceToHost), "get");
     return LBMS_OK;
 }
 
@@ -1030,7 +1134,7 @@ lbms_status lbms_net_warm_start(lbms_net* n, lbms_ctx* ctx, int k, double* Xout)
             "rows");
         st = forward(n, rows, false);
         if (st != LBMS_OK) return st;
-        predict_post_kernel<<<(rows + 255) / 256, 256>>>(n->Y, F.cell, j0, rows, v.nf, v.nx, F.xtab, F.pred);
+        predict_post_kernel<<<(rows + 255) / 256, 256>>>(n->Y, n->y_ld, F.cell, j0, rows, v.nf, v.nx, F.xtab, F.pred);
         NCK(cudaGetLastError(), "prediction");
     }
     return take_prediction(n, ctx, k, F, Xout);

@@ -303,8 +303,11 @@ struct lbms_unet {
     size_t P_floats = 0;
     int last[4] = {0, 0, 0, 0};  // B, X, Y, Z of the layout the buffers held last
     std::vector<void*> bufs;     // the grown buffers
+    float* zero = nullptr;       // the loss and all bias gradients, cleared together
+    size_t zero_bytes = 0;
     double* loss = nullptr;
     float* flat = nullptr;       // parameters or gradients in the caller's order
+    std::mutex flat_use;
     unsigned int* gemm_err = nullptr;
     struct Sample {
         int X = 0, Y = 0, Z = 0;                // interior extents (multiples of 4)
@@ -642,10 +645,10 @@ lbms_status unet_forward(lbms_unet* u, const Levels& v, bool train, float inv_n)
     lbms::ConvJob j = conv_job(g0, u->d1, h.ci_s, h.Wb, h.rows, 1, 1, lbms::kOutHead);
     j.ep.bias = h.b;
     if (train) {
-        UCK(cudaMemsetAsync(u->loss, 0, sizeof(double), 0), "loss");
-        for (auto& l : L) UCK(cudaMemsetAsync(l.gb, 0, l.co_s * sizeof(float), 0), "bias gradients");
+        UCK(cudaMemsetAsync(u->zero, 0, u->zero_bytes, 0), "loss and bias gradients");
         j.ep.T = u->T;
-        j.ep.inv_n = inv_n;
+        j.ep.grad_scale = 2.0f * inv_n;
+        j.ep.loss_scale = (double)inv_n;
         j.ep.out = u->za[0];
         j.ep.gb = h.gb;
         j.ep.loss = u->loss;
@@ -712,14 +715,14 @@ lbms_status unet_adam(lbms_unet* u, double lr) {
     ++u->step;
     const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)u->step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)u->step)));
-    for (const auto& l : u->L) {
-        const int64_t nw = (int64_t)l.rows * l.K;
-        adam_kernel<<<grid_for(nw), 256>>>(l.W, l.m, l.v, l.g, nw, (float)lr, c1, c2, l.rows, l.K, nullptr, nullptr);
-        adam_kernel<<<grid_for(l.co_s), 256>>>(l.b, l.mb, l.vb, l.gb, l.co_s, (float)lr, c1, c2, l.co_s, 1, nullptr,
-                                               nullptr);
-        UCK(cudaGetLastError(), "adam");
-        UST(cast_layer(u, l));
+    AdamList list = {};
+    for (int i = 0; i < kULayers; ++i) {
+        const auto& l = u->L[i];
+        list.it[2 * i] = {l.W, l.m, l.v, l.g, (int64_t)l.rows * l.K, l.Wb, l.Wt, l.rows, l.K, l.kind == 3 ? l.ci_s : 0};
+        list.it[2 * i + 1] = {l.b, l.mb, l.vb, l.gb, l.co_s, nullptr, nullptr, l.co_s, 1, 0};
     }
+    adam_all_kernel<<<dim3(152, 2 * kULayers), 256>>>(list, (float)lr, c1, c2);
+    UCK(cudaGetLastError(), "adam");
     return LBMS_OK;
 }
 
@@ -839,11 +842,19 @@ lbms_status lbms_unet_create(int width, int64_t max_voxels, uint64_t seed, lbms_
         l.b = ualloc<float>(u, l.co_s);
         l.mb = ualloc<float>(u, l.co_s);
         l.vb = ualloc<float>(u, l.co_s);
-        l.gb = ualloc<float>(u, l.co_s);
         l.Wb = ualloc<bf16>(u, nw);
         l.Wt = ualloc<bf16>(u, l.kind == 3 ? (size_t)l.ci_s * 27 * l.co_s : nw);
     }
-    u->loss = ualloc<double>(u, 1);
+    size_t biases = 0;
+    for (const auto& l : u->L) biases += l.co_s;
+    u->zero_bytes = sizeof(double) + biases * sizeof(float);
+    u->zero = ualloc<float>(u, 2 + biases);
+    u->loss = reinterpret_cast<double*>(u->zero);
+    float* gb = u->zero ? u->zero + 2 : nullptr;
+    for (auto& l : u->L) {
+        l.gb = gb;
+        if (gb) gb += l.co_s;
+    }
     u->flat = ualloc<float>(u, unet_params(u));
     u->gemm_err = ualloc<unsigned int>(u, 1);
     bool ok = true;
@@ -852,7 +863,7 @@ lbms_status lbms_unet_create(int width, int64_t max_voxels, uint64_t seed, lbms_
         lbms_unet_destroy(u);
         return LBMS_ENOMEM;
     }
-    ok = lbms::umma_gemm_init() == cudaSuccess;
+    ok = lbms::umma_init() == cudaSuccess;
     ok = ok && cudaMemset(u->gemm_err, 0, sizeof(unsigned int)) == cudaSuccess;
     // He-uniform weights on the real entries (fan-in 27 ci for the 3x3x3
     // convolutions, ci for the transposed ones), zero head, zero biases
@@ -1167,6 +1178,7 @@ lbms_status lbms_unet_get(const lbms_unet* cu, int what, float* buf, int64_t cou
     if (!u || !buf || (what != 0 && what != 1)) return LBMS_EINVAL;
     if (count < unet_params(u))
         return ufail(u, LBMS_EINVAL, "buffer holds %lld floats, need %lld", (long long)count, (long long)unet_params(u));
+    const std::lock_guard<std::mutex> hold(u->flat_use);
     int64_t off = 0;
     for (const auto& l : u->L) {
         const int64_t n = layer_weights(l);
@@ -1182,6 +1194,7 @@ lbms_status lbms_unet_set(lbms_unet* u, const float* buf, int64_t count) {
     if (!u || !buf) return LBMS_EINVAL;
     if (count < unet_params(u))
         return ufail(u, LBMS_EINVAL, "buffer holds %lld floats, need %lld", (long long)count, (long long)unet_params(u));
+    const std::lock_guard<std::mutex> hold(u->flat_use);
     UCK(cudaMemcpy(u->flat, buf, (size_t)unet_params(u) * sizeof(float), cudaMemcpyHostToDevice), "set");
     int64_t off = 0;
     for (const auto& l : u->L) {
