@@ -431,16 +431,20 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
         }
         if constexpr (KIND == kOutHead) {
             if (ep.T) {
+double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    loss += __shfl_down_sync(0xffffffffu, loss, o);
+                for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) hs[c] += __shfl_down_sync(0xffffffffu, hs[c], o);
-                }
+                    for (int c = 0; c < 4; ++c) sum[c] += __shfl_down_sync(0xffffffffu, sum[c], o);
                 if (lane == 0) {
-                    atomicAdd(ep.loss, loss * ep.loss_scale);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) atomicAdd(&ep.gb[c], hs[c]);
+                    for (int c = 0; c < 4; ++c) atomicAdd(&ep.loss[c], sum[c]);
+                    __threadfence();
+                    if (atomicAdd(ep.done, 1u) + 1u == 4u * gridDim.x) {   // the last epilogue warp
+                        __threadfence();
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) ep.gb[c] = (float)__ldcg(&ep.loss[1 + c]);
+                    }
                 }
             }
         }

@@ -202,7 +202,7 @@ enum ConvOut {
     kOutUp,         // transposed 2x2x2 convolution: column t Cg + n of an interior row, plus bias[n], to the row's
                     //   child t of the finer layout, cat[child][n] (n < w)
     kOutHead        // Y = acc + bias (3 columns): Y[r][4] if given; against T [r][4] = (targets, mask), if given,
-                    //   out[r][n] = BF16(grad_scale (Y - T) mask) (0 for n >= 3), its column sums into gb and
+                    //   out[r][n] = BF16(grad_scale (Y - T) mask) (0 for n >= 3), its column sums (FP64) to gb and
                     //   loss_scale sum((Y - T)^2 mask^2) into loss
 };
 struct ConvEpilogue {
@@ -217,7 +217,8 @@ struct ConvEpilogue {
     float* gb = nullptr;
     const float* T = nullptr;
     float* Y = nullptr;
-    double* loss = nullptr;
+    double* loss = nullptr;       // kOutHead: loss and the three column sums, 0 before
+    unsigned int* done = nullptr; // kOutHead: 0 before
     float grad_scale = 0.0f;
     double loss_scale = 0.0;
     RowLayout g;                  // the product's rows

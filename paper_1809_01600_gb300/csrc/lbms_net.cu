@@ -43,6 +43,7 @@ constexpr int kFUsed = 16;              // features actually set
 constexpr int kOutPad = 64;             // output layer rows (3 used)
 constexpr int kOut = 3;
 constexpr float kTargetScale = 100.0f;  // network output = 100 (X - X_profile)
+constexpr int kZeroHead = 10;           // floats before the bias gradients: loss and sums (4 FP64), a counter
 constexpr int kMaxRows = 32768;         // rows per forward / training batch
 constexpr int kTM = 64, kTN = 64, kTK = 32;
 
@@ -601,6 +602,7 @@ lbms_status forward(lbms_net* n, int R, bool train) {
                 j.ep.out = n->dz[0];
                 j.ep.gb = n->gb[l];
                 j.ep.loss = n->loss;
+                j.ep.done = reinterpret_cast<unsigned int*>(n->loss + 4);
             } else {
                 j.ep.Y = n->Y;
                 n->y_ld = 4;
@@ -894,10 +896,10 @@ lbms_status lbms_net_create(int width, int depth, uint64_t seed, lbms_net** out)
     n->T = nalloc<float>(n, (size_t)kMaxRows * 4);
     size_t biases = 0;
     for (int l = 0; l < n->layers; ++l) biases += n->out[l];
-    n->zero_bytes = sizeof(double) + biases * sizeof(float);
-    n->zero = nalloc<float>(n, 2 + biases);
+    n->zero_bytes = kZeroHead * sizeof(float) + biases * sizeof(float);
+    n->zero = nalloc<float>(n, kZeroHead + biases);
     n->loss = reinterpret_cast<double*>(n->zero);
-    for (int l = 0, o = 2; l < n->layers; o += n->out[l++]) n->gb.push_back(n->zero ? n->zero + o : nullptr);
+    for (int l = 0, o = kZeroHead; l < n->layers; o += n->out[l++]) n->gb.push_back(n->zero ? n->zero + o : nullptr);
     n->flat = nalloc<float>(n, n_params(n));
     n->gemm_err = nalloc<unsigned int>(n, 1);
     for (void* p : n->allocs) ok = ok && p;

@@ -652,6 +652,7 @@ lbms_status unet_forward(lbms_unet* u, const Levels& v, bool train, float inv_n)
         j.ep.out = u->za[0];
         j.ep.gb = h.gb;
         j.ep.loss = u->loss;
+        j.ep.done = reinterpret_cast<unsigned int*>(u->loss + 4);
     } else {
         j.ep.Y = u->Y;
     }
@@ -847,10 +848,10 @@ lbms_status lbms_unet_create(int width, int64_t max_voxels, uint64_t seed, lbms_
     }
     size_t biases = 0;
     for (const auto& l : u->L) biases += l.co_s;
-    u->zero_bytes = sizeof(double) + biases * sizeof(float);
-    u->zero = ualloc<float>(u, 2 + biases);
+    u->zero_bytes = kZeroHead * sizeof(float) + biases * sizeof(float);
+    u->zero = ualloc<float>(u, kZeroHead + biases);
     u->loss = reinterpret_cast<double*>(u->zero);
-    float* gb = u->zero ? u->zero + 2 : nullptr;
+    float* gb = u->zero ? u->zero + kZeroHead : nullptr;
     for (auto& l : u->L) {
         l.gb = gb;
         if (gb) gb += l.co_s;
