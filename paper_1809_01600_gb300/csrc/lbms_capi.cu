@@ -1026,7 +1026,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "pinned readback buffer"));
 
     const int nbw = dim == 2 ? nb_width<D2Q9>() : nb_width<D3Q19>();
-    const size_t fbytes = (size_t)3 * c->Q * L.S * pop_size(L.precision);
+    const size_t fbytes = (size_t)L.S * (L.tiled ? tile_cell_bytes(L.dim, L.precision) : 3 * c->Q * pop_size(L.precision));
     const size_t xbytes = (size_t)3 * L.S * x_size(L.precision);
     const size_t sbytes = (size_t)3 * L.S * sizeof(double);
     const size_t cbytes = (size_t)n_cases * case_bc_size(L.precision);

@@ -32,15 +32,15 @@ constexpr int kVariantPerCell[kStepVariants] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
 // many cells per SM ahead of a block it prefetches, and the blocks per SM its
 // registers are budgeted for.  Measured on the 256x128x128 anode (1.69 M fluid
 // cells, us per step), blocks per SM 5 / 6 / 8 / 9 / 10 / 12: FP32 151 / 151 /
-// 143 / 153 / 140 / 191, FP16 127 / 127 / 112 / 119 / 118 / 151, FP64 2231 /
-// 2253 / 2297 / 2306 / 2306 / 2308; 2-D FP32 (1.22 M cells) 59 up to 10, 56.5
-// at 12.  Prefetch none / 16 / 24 / 48 thousand cells ahead: FP32 155 / 144 /
+// 143 / 153 / 140 / 191, FP64 2231 / 2253 / 2297 / 2306 / 2306 / 2308, FP16 at
+// 8 / 9 / 10 / 12: 105 / 104 / 101 / 125; 2-D FP32 (1.22 M cells) 59 up to 10,
+// 56.5 at 12, FP16 44.8 at any.  Prefetch none / 16 / 24 / 48 thousand cells ahead: FP32 155 / 144 /
 // 143 / 145, FP16 122 / 113 / 112 / 113.
 constexpr int kTile = 64;
 constexpr int kTileBlkCase = 2;
 constexpr int kTilePrefetch = 160;      // 24,320 cells on 152 SMs
 constexpr int tile_min_blocks(int dim, int precision) {
-    return dim == 2 ? (precision == 1 ? 12 : 8) : (precision == 0 ? 5 : (precision == 1 ? 10 : 8));
+    return dim == 2 ? (precision == 1 ? 12 : 8) : (precision == 0 ? 5 : 10);
 }
 // Below this many cells (4 blocks of 64 on each of 152 SMs) a launch does not
 // fill the GPU and the small handles' step is the faster: 37 k cells in FP32
@@ -139,7 +139,8 @@ cudaError_t launch_step(const Launch& L, cudaStream_t st);
 cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st);
 // the same with the grad_forward / outlet_extrap options compiled in
 cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream_t st);
-// the default step (lbms_step_tile.cuh); needs L.tiled
+// the default step (lbms_step_tile.cuh); needs L.tiled; bytes of a cell's populations in its layout
+size_t tile_cell_bytes(int dim, int precision);
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 // the step for a handle whose largest case has max_nf cells, or kNotSmall;
 // L.ncells and sm_count are set

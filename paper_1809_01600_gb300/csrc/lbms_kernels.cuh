@@ -861,11 +861,41 @@ __global__ void fields_kernel(const XS* __restrict__ xcur, const XS* __restrict_
     }
 }
 
-// Element of population (s, k) of cell i: rows of stride S, or the tiled
-// layout of lbms_step_tile.cuh.
+// The tiled population layout (lbms_step_tile.cuh): a tile of kTile cells is
+// kRows rows of kTile units U; row(s, k) is the row of population (s, k), half
+// its 16-bit half of the unit.
+template <class L, typename P>
+struct TileLay {
+    using U = P;
+    static constexpr int kRows = 3 * L::Q;
+    __host__ __device__ static constexpr int row(int s, int k) { return s * L::Q + k; }
+    __host__ __device__ static constexpr int half(int, int) { return 0; }
+};
+// 16-bit populations lie two to a 32-bit unit: species 0 and 1 of a link
+// together, species 2 of link k with that of link k + 2.  The row of the
+// opposite link (k + 1 for odd k) is the next one for every species.
 template <class L>
+struct TileLay<L, __half> {
+    using U = uint32_t;
+    static constexpr int kPairs = (L::Q - 1) / 2;
+    static constexpr int kRest = kPairs / 2 * 6 + kPairs % 2 * 4;    // row of the rest populations of species 0, 1
+    static constexpr int kRows = kRest + 1 + (kPairs % 2 == 0);
+    __host__ __device__ static constexpr int row(int s, int k) {
+        if (k == 0) return s < 2 ? kRest : (kPairs % 2 ? kRest - 2 : kRest + 1);
+        const int q = (k - 1) / 2, o = (k - 1) % 2, m = q / 2 * 6;
+        const bool alone = q == kPairs - 1 && kPairs % 2;            // the last pair of an odd number
+        return s < 2 ? m + q % 2 * 2 + o : m + (alone ? 2 : 4) + o;
+    }
+    __host__ __device__ static constexpr int half(int s, int k) { return s < 2 ? s : (k == 0 ? kPairs % 2 : (k - 1) / 2 % 2); }
+};
+
+// Element of population (s, k) of cell i: rows of stride S, or the tiled layout.
+template <class L, typename P>
 __device__ __forceinline__ int64_t pop_index(bool tiled, int64_t S, int s, int k, int i) {
-    return tiled ? (int64_t)(i / kTile) * (3 * kTile * L::Q) + (s * L::Q + k) * kTile + i % kTile
+    using Lay = TileLay<L, P>;
+    constexpr int per = sizeof(typename Lay::U) / sizeof(P);
+    return tiled ? ((int64_t)(i / kTile) * (kTile * Lay::kRows) + Lay::row(s, k) * kTile + i % kTile) * per +
+                       Lay::half(s, k)
                  : (int64_t)(s * L::Q + k) * S + i;
 }
 
@@ -884,7 +914,7 @@ __global__ void init_kernel(P* __restrict__ h, const XS* __restrict__ x0, XS* __
         v.store(x1, S, s, i);
         snap[s * S + i] = v.to_double();
 #pragma unroll
-        for (int k = 0; k < L::Q; ++k) h[pop_index<L>(tiled, S, s, k, i)] = Pop<T, P>::quant(T(0));
+        for (int k = 0; k < L::Q; ++k) h[pop_index<L, P>(tiled, S, s, k, i)] = Pop<T, P>::quant(T(0));
     }
 }
 
@@ -1129,14 +1159,14 @@ __global__ void __launch_bounds__(kSegThreads) case_boundary_kernel(
 #pragma unroll
                     for (int s = 0; s < 3; ++s)
                         acc[s] += w * Xv<XS>::own(X, S, s, i0).to_double() +
-                                  (double)Pop<T, P>::load(h + pop_index<L>(tiled, S, s, k, i0));
+                                  (double)Pop<T, P>::load(h + pop_index<L, P>(tiled, S, s, k, i0));
                 }
             } else if (ex == -1 && i1 >= 0) {
                 if (nbr[(int64_t)i1 * nb_width<L>() + opp<L>(k) - 1] >= 0) {
 #pragma unroll
                     for (int s = 0; s < 3; ++s)
                         acc[s] -= w * Xv<XS>::own(X, S, s, i1).to_double() +
-                                  (double)Pop<T, P>::load(h + pop_index<L>(tiled, S, s, k, i1));
+                                  (double)Pop<T, P>::load(h + pop_index<L, P>(tiled, S, s, k, i1));
                 }
             }
         }

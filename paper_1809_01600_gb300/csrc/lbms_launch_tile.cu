@@ -41,6 +41,11 @@ cudaError_t tile_t(const Launch& L, cudaStream_t st) {
 
 }  // namespace
 
+size_t tile_cell_bytes(int dim, int precision) {
+    if (precision == 2) return 4 * (dim == 2 ? TileLay<D2Q9, __half>::kRows : TileLay<D3Q19, __half>::kRows);
+    return 3 * (dim == 2 ? D2Q9::Q : D3Q19::Q) * pop_size(precision);
+}
+
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st) {
     if (L.dim == 2) {
         if (L.precision == 0) return tile_t<D2Q9, double, double>(L, st);

@@ -1,9 +1,9 @@
 // The default time step: one thread per fluid cell with the populations of
 // all three species in registers, and the populations in tiles in memory.
 //
-// Tiled layout: population (s, k) of cell j at element
-// (j / 64) 3 Q 64 + (s Q + k) 64 + j % 64, so that all populations of a cell
-// lie at compile-time distances from one address.  A link then costs one
+// Tiled layout (TileLay): population (s, k) of cell j at unit
+// (j / 64) R 64 + row(s, k) 64 + j % 64 of R rows a tile, so that all populations
+// of a cell lie at compile-time distances from one address.  A link then costs one
 // address for its three species and the stores of a cell one address in all,
 // where rows of stride S need one per population; and a tile is one
 // contiguous piece of memory (14.6 KB in FP32), which a single instruction
@@ -13,9 +13,10 @@
 // moves 826 MB a step and takes 140 us, 5.9 TB/s of the 6.8 a copy reaches;
 // with the neighbour decode, the address arithmetic and the boundary rules
 // spread over the links the step before issued 108 M warp instructions and
-// took 181 us, this one issues 66 M.  FP16 moves 441 MB in 112 us (151
-// before): the latency of the gathers at 16 warps an SM and their issue (54 %
-// of the slots).  FP64 takes 2231 us (2548): the FP64 pipe.
+// took 181 us, this one issues 66 M.  FP16 moves 449 MB in 101 us (151
+// before): the latency of the gathers and their issue, so populations share
+// 32-bit units (112 us with a 16-bit access for each, 57 loads and 57 stores a
+// cell instead of 38 and 29).  FP64 takes 2231 us (2548): the FP64 pipe.
 // The same with one thread per (cell, species) and the lookup shared through
 // shared memory took 161 us (FP32) and 137 us (FP16): the L1 data stage, at
 // 72-76 %, from the two-word link records read three times a cell.
@@ -112,19 +113,19 @@ struct Pk<float> {
     }
 };
 
-// Element of population (species 0, link 0) of cell j in the tiled layout.
+// Unit of row 0 of cell j in the tiled layout.
 // Sources are counted from one tile before the first cell (index j + kTile,
 // pointers one tile back), so that the step to the opposite link at a wall
 // stays non-negative; 3 Q (S + kTile) < 2^32 (checked at create).
-template <class L>
+template <class L, typename P>
 __device__ __forceinline__ uint32_t tile_off(int j) {
-    return (uint32_t)j + (uint32_t)(j & ~(kTile - 1)) * (3 * L::Q - 1);
+    return (uint32_t)j + (uint32_t)(j & ~(kTile - 1)) * (TileLay<L, P>::kRows - 1);
 }
 
 // A link's source, counted from one tile before the first cell: the cell
-// whose X it exchanges with (the cell itself at a wall) and the element of
-// the species-0 population to pull less k kTile (bounce-back folded in: the
-// opposite link of the cell itself).
+// whose X it exchanges with (the cell itself at a wall) and the unit to pull
+// from less row(s, k) kTile (bounce-back folded in: the opposite link of the
+// cell itself, one row on or back).
 struct Source {
     uint32_t h;
     int x;
@@ -135,7 +136,7 @@ struct Source {
 // case: .x = fluid flags of voxels 16 w - 8 .. 16 w + 23 of the row (zero
 // outside the grid), .y = kTile + the fluid index that the first fluid voxel
 // at or after 16 w - 8 has (or would have).
-template <class L>
+template <class L, typename P>
 __device__ __forceinline__ void row_sources(uint32_t code, const uint2* __restrict__ tab, int nx, int ny, int nz,
                                             int wpr, int i, Source (&src)[L::Q], bool& at_in, bool& at_out) {
     const bool pad = code == 0xFFFFFFFFu;   // padding cell between cases: walls all round
@@ -150,7 +151,7 @@ __device__ __forceinline__ void row_sources(uint32_t code, const uint2* __restri
     const int plane = ny * wpr;
     const int rz[3] = {(z == 0 ? nz - 1 : z - 1) * plane, z * plane, (z == nz - 1 ? 0 : z + 1) * plane};
     i += kTile;
-    const uint32_t own = tile_off<L>(i);
+    const uint32_t own = tile_off<L, P>(i);
     at_in = x == 0 && !pad;
     at_out = x == nx - 1 && !pad;
 #pragma unroll
@@ -167,7 +168,7 @@ __device__ __forceinline__ void row_sources(uint32_t code, const uint2* __restri
                 const int dx = -L::e(k, 0);
                 const bool fluid = bits & (dx < 0 ? 1u : (dx == 0 ? 2u : 4u));
                 const int j = dx < 0 ? at - 1 : (dx == 0 ? at : at + (int)((bits >> 1) & 1u));
-                src[k].h = fluid ? tile_off<L>(j) : own + (opp<L>(k) - k) * kTile;
+                src[k].h = fluid ? tile_off<L, P>(j) : own + (opp<L>(k) - k) * kTile;
                 src[k].x = fluid ? j : i;
             }
         }
@@ -175,22 +176,41 @@ __device__ __forceinline__ void row_sources(uint32_t code, const uint2* __restri
 }
 
 // The same from the cell's row of the 32-bit table.
-template <class L>
+template <class L, typename P>
 __device__ __forceinline__ void table_sources(const int* __restrict__ nbr, int i, Source (&src)[L::Q], bool& at_in,
                                               bool& at_out) {
     int nb[L::Q];
     load_neighbours<L>(nbr, i, nb);
     i += kTile;
-    const uint32_t own = tile_off<L>(i);
+    const uint32_t own = tile_off<L, P>(i);
     at_in = nb[1] == NB_INLET;      // links 1 and 2 pull from x - 1 and x + 1
     at_out = nb[2] == NB_OUTLET;
 #pragma unroll
     for (int k = 1; k < L::Q; ++k) {
         const bool fluid = nb[k] >= 0;
-        src[k].h = fluid ? tile_off<L>(nb[k] + kTile) : own + (opp<L>(k) - k) * kTile;
+        src[k].h = fluid ? tile_off<L, P>(nb[k] + kTile) : own + (opp<L>(k) - k) * kTile;
         src[k].x = fluid ? nb[k] + kTile : i;
     }
 }
+
+// The populations of link k of the three species from unit a (a source, rows
+// from 0), as stored values.
+template <class L, typename T, typename P>
+__device__ __forceinline__ void load_link(const typename TileLay<L, P>::U* a, int k, T (&v)[3]) {
+    using Lay = TileLay<L, P>;
+    if constexpr (std::is_same<P, __half>::value) {
+        const uint32_t w = a[Lay::row(0, k) * kTile];
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = Pop<T, P>::raw(reinterpret_cast<const __half*>(a + Lay::row(2, k) * kTile) + Lay::half(2, k));
+    } else {
+#pragma unroll
+        for (int s = 0; s < 3; ++s) v[s] = Pop<T, P>::raw(a + Lay::row(s, k) * kTile);
+    }
+}
+
+__device__ __forceinline__ uint32_t half_bits(__half2 h) { return *reinterpret_cast<const uint32_t*>(&h); }
 
 template <class L, typename XS, typename P, typename NBT, int W, int MB>
 __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P> p) {
@@ -198,6 +218,9 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
     using XV = Xv<XS>;
     using PT = Pk<T>;
     static_assert(W == kTile, "a block covers a tile");
+    using Lay = TileLay<L, P>;
+    using U = typename Lay::U;
+    constexpr bool kHalf = std::is_same<P, __half>::value;
     constexpr int Q = L::Q;
     constexpr int DIM = L::DIM;
     constexpr int NP = (Q - 1) / 2;          // link pairs (k, k + 1), opposite to each other
@@ -209,10 +232,10 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
     Source src[Q];
     bool at_in, at_out;
     if constexpr (std::is_same<NBT, RowMaskNb>::value)
-        row_sources<L>(__ldg(p.cell_code + i), p.rowtab + cb.tab, cb.nx, cb.ny, cb.nz,
+        row_sources<L, P>(__ldg(p.cell_code + i), p.rowtab + cb.tab, cb.nx, cb.ny, cb.nz,
                        cb.wpr, i, src, at_in, at_out);
     else
-        table_sources<L>(p.nbr32, i, src, at_in, at_out);
+        table_sources<L, P>(p.nbr32, i, src, at_in, at_out);
     grid_wait();
 
     const int64_t S = p.S;
@@ -221,32 +244,30 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
         const int64_t j = (int64_t)blockIdx.x * W + p.pf_dist;   // a multiple of the tile
         if (j + kTile <= S) {
             if (threadIdx.x == 0)
-                prefetch_bulk(p.hin + j * (3 * Q), 3 * Q * kTile * sizeof(P));
+                prefetch_bulk(reinterpret_cast<const U*>(p.hin) + j * Lay::kRows, Lay::kRows * kTile * sizeof(U));
             else
                 prefetch_bulk(p.xin + (threadIdx.x - 1) * S + j, kTile * sizeof(XS));
         }
     }
     const XS* xh[3] = {p.xin, p.xin + S, p.xin + 2 * S};
-    const uint32_t own = tile_off<L>(i);
-    const P* hi_own = p.hin + own;
-    const P* hin = p.hin - 3 * Q * kTile;
+    const uint32_t own = tile_off<L, P>(i);
+    const U* hin = reinterpret_cast<const U*>(p.hin) - Lay::kRows * kTile;
     XV xo[3];
     T d0[3], g[3][DIM];
     PT d[3][NP];     // f_k(x) - w_k X_old(x) after streaming
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        xo[s] = XV::own_rows(xh[s], p.xin + (int64_t)(3 + s) * S, i);
-        d0[s] = Pop<T, P>::raw(hi_own + s * Q * kTile);
-    }
+    for (int s = 0; s < 3; ++s) xo[s] = XV::own_rows(xh[s], p.xin + (int64_t)(3 + s) * S, i);
+    load_link<L, T, P>(reinterpret_cast<const U*>(p.hin) + own, 0, d0);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
         const int k = 1 + 2 * q;
-        const P* ha = hin + src[k].h;
-        const P* hb = hin + src[k + 1].h;
+        T ha[3], hb[3];
+        load_link<L, T, P>(hin + src[k].h, k, ha);
+        load_link<L, T, P>(hin + src[k + 1].h, k + 1, hb);
         const T w = T(weight<L>(k) * sc);
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-            const PT h = PT::make(Pop<T, P>::raw(ha + (s * Q + k) * kTile), Pop<T, P>::raw(hb + (s * Q + k + 1) * kTile));
+            const PT h = PT::make(ha[s], hb[s]);
             const T nx = -xo[s].exch_base();
             const PT dx = PT::make(xh[s][src[k].x - kTile], xh[s][src[k + 1].x - kTile]) + PT::make(nx, nx);
             d[s][q] = PT::fma(PT::make(w, w), dx, h);
@@ -289,7 +310,9 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
         X[s] = xn.value();
         xn.store_rows(p.xout + s * S, p.xout + (3 + s) * S, i);
     }
-    P* ho = p.hout + own;
+    U* ho = reinterpret_cast<U*>(p.hout) + own;
+    __half2 held[kHalf ? NP : 1];    // species 0, then pairs of species 2, until their units are complete
+    __half held0;
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
         T J[DIM], v[DIM], tau, xinv;
@@ -319,13 +342,42 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
                 first = false;
             }
             const PT hk = PT::fma(PT::fma(w, ndX, d[s][q]), keep2, w * ev);
-            const P q0 = Pop<T, P>::quant_raw(hk.low());
-            const P q1 = Pop<T, P>::quant_raw(hk.high());
-            rest = rest + PT::make(Pop<T, P>::dequant_raw(q0), Pop<T, P>::dequant_raw(q1));
-            step_store(ho + (s * Q + k) * kTile, q0);
-            step_store(ho + (s * Q + k + 1) * kTile, q1);
+            if constexpr (kHalf) {
+                const __half2 h2 = __floats2half2_rn(hk.low(), hk.high());
+                const float2 r = __half22float2(h2);
+                rest = rest + PT::make(r.x, r.y);
+                if (s == 1) {
+                    step_store(ho + Lay::row(0, k) * kTile, half_bits(__lows2half2(held[q], h2)));
+                    step_store(ho + Lay::row(0, k + 1) * kTile, half_bits(__highs2half2(held[q], h2)));
+                } else if (s == 2 && q % 2) {
+                    step_store(ho + Lay::row(2, k) * kTile, half_bits(__lows2half2(held[q - 1], h2)));
+                    step_store(ho + Lay::row(2, k + 1) * kTile, half_bits(__highs2half2(held[q - 1], h2)));
+                } else {
+                    held[q] = h2;
+                }
+            } else {
+                const P q0 = Pop<T, P>::quant_raw(hk.low());
+                const P q1 = Pop<T, P>::quant_raw(hk.high());
+                rest = rest + PT::make(Pop<T, P>::dequant_raw(q0), Pop<T, P>::dequant_raw(q1));
+                step_store(ho + Lay::row(s, k) * kTile, q0);
+                step_store(ho + Lay::row(s, k + 1) * kTile, q1);
+            }
         }
-        step_store(ho + s * Q * kTile, Pop<T, P>::quant_raw(-(rest.low() + rest.high())));
+        const P q0 = Pop<T, P>::quant_raw(-(rest.low() + rest.high()));
+        if constexpr (kHalf) {
+            if (s == 0) {
+                held0 = q0;
+            } else if (s == 1) {
+                step_store(ho + Lay::kRest * kTile, half_bits(__halves2half2(held0, q0)));
+            } else if (NP % 2) {     // with the last pair of species 2
+                step_store(ho + Lay::row(2, 0) * kTile, half_bits(__halves2half2(__low2half(held[NP - 1]), q0)));
+                step_store(ho + (Lay::row(2, 0) + 1) * kTile, half_bits(__highs2half2(held[NP - 1], held[NP - 1])));
+            } else {
+                step_store(ho + Lay::row(2, 0) * kTile, half_bits(__halves2half2(q0, q0)));
+            }
+        } else {
+            step_store(ho + Lay::row(s, 0) * kTile, q0);
+        }
     }
 }
 
