@@ -90,7 +90,9 @@ struct ConvShape {
     static constexpr int kARows = NT == 3 ? 130 : 128;
     static constexpr int kABytes = align1k(kARows * RB);
     static constexpr int kBTile = N * RB;
-    static constexpr int kStage = kABytes + (kResident ? 0 : NT * kBTile);
+    static constexpr int kGps = NT == 3 && RB == 64 ? 3 : 1;   // windows (dz, dy rows) of a stage
+    static constexpr int kStage = kGps * kABytes + (kResident ? 0 : NT * kBTile);
+    static_assert(kGps == 1 || kResident, "a stage holds the weights of one window");
     static constexpr int kResBytes = kResident ? align1k(27 * kBTile) : 0;
     static constexpr int kStageFloats = KIND == kOutSplit ? 4 * 32 * 65 : 0;   // split: rows of each epilogue warp
     static constexpr int kFixed = 1024 + kResBytes + kStageFloats * 4 + N * 4 + 512;
@@ -109,6 +111,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
     using Sh = ConvShape<RB, N, NT, KIND>;
     constexpr int ST = Sh::kStages;
     constexpr int KS = RB / 32;
+    constexpr int GPS = Sh::kGps;
     constexpr uint32_t idesc = umma_idesc(128, N, false);
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -125,7 +128,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
     volatile uint32_t* failed = tmem_slot + 1;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int tiles = (rows + 127) / 128 * ntn;
-    const int per_tile = Sh::kGroups * nblk;   // stages of a tile: (dz, dy) rows x channel blocks
+    const int per_tile = Sh::kGroups / GPS * nblk;   // stages of a tile: (dz, dy) rows x channel blocks
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST; ++s) {
@@ -164,8 +167,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
         bool ok = true;
         for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
             const int m0 = tile / ntn * 128, n0 = tile % ntn * N;
-            for (int g = 0; ok && g < Sh::kGroups; ++g) {
-                const int r = NT == 1 ? m0 : m0 + job.off[3 * g + (back ? 2 : 0)];
+            for (int g = 0; ok && g < Sh::kGroups; g += GPS) {
                 for (int c = 0; c < nblk; ++c) {
                     if (!mbar_wait(&empty[s], ph)) {   // the first pass through the ring finds it free
                         ok = false;
@@ -173,8 +175,11 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                     }
                     if (leader) {
                         uint8_t* sa = stages + s * Sh::kStage;
-                        mbar_expect_tx(&full[s], Sh::kARows * RB + (Sh::kResident ? 0 : NT * Sh::kBTile));
-                        tma_load_2d(sa, &mapA, c * (RB / 2), r, &full[s]);
+                        mbar_expect_tx(&full[s], GPS * Sh::kARows * RB + (Sh::kResident ? 0 : NT * Sh::kBTile));
+#pragma unroll
+                        for (int i = 0; i < GPS; ++i)
+                            tma_load_2d(sa + i * Sh::kABytes, &mapA, c * (RB / 2),
+                                        NT == 1 ? m0 : m0 + job.off[3 * (g + i) + (back ? 2 : 0)], &full[s]);
                         if (!Sh::kResident)
                             for (int d = 0; d < NT; ++d)
                                 tma_load_2d(sa + Sh::kABytes + d * Sh::kBTile, &mapB,
@@ -218,15 +223,19 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                 }
                 fence_after();
                 const uint64_t as = a0 + (uint32_t)((s * Sh::kStage) >> 4);
-                const uint64_t bs = b0 + (uint32_t)((Sh::kResident ? q * 3 * Sh::kBTile : s * Sh::kStage) >> 4);
+                const uint64_t bs = b0 + (uint32_t)((Sh::kResident ? q * GPS * 3 * Sh::kBTile : s * Sh::kStage) >> 4);
                 if (leader) {
 #pragma unroll
-                    for (int d = 0; d < NT; ++d) {
-                        const uint64_t ad = as + (uint32_t)(((back ? 2 - d : d) * RB * (NT == 3)) >> 4);
+                    for (int i = 0; i < GPS; ++i)
 #pragma unroll
-                        for (int j = 0; j < KS; ++j)
-                            umma_f16(d0, ad + 2 * j, bs + ((d * Sh::kBTile) >> 4) + 2 * j, idesc, (q | d | j) != 0);
-                    }
+                        for (int d = 0; d < NT; ++d) {
+                            const uint64_t ad =
+                                as + (uint32_t)((i * Sh::kABytes + (back ? 2 - d : d) * RB * (NT == 3)) >> 4);
+#pragma unroll
+                            for (int j = 0; j < KS; ++j)
+                                umma_f16(d0, ad + 2 * j, bs + (((i * NT + d) * Sh::kBTile) >> 4) + 2 * j, idesc,
+                                         (q | i | d | j) != 0);
+                        }
                     umma_commit(&empty[s]);
                 }
                 __syncwarp();
@@ -628,6 +637,160 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
     if (warp == 0) tmem_dealloc(tmem, cols);
 }
 
+// The weight gradient of a 3x3x3 convolution with at most 64 channels on
+// either side, with the operands' roles turned round: the MMA's 128 rows are
+// the channels of dz at consecutive rows (4 or 2 blocks of them, each one row
+// further into the same window), its columns the channels of x in the three
+// windows of a dz.  With x at row p and dz at row p - 2 + j the product belongs
+// to tap dx = 2 - j.  An MMA reads its 128-row operand from shared memory at 32
+// cycles whatever its columns are, so 96 or 192 columns instead of 32 or 64
+// take a third of the time: 4 volumes of 96^3, 32 by 32 channels WG3_FIGURES.
+template <int RBA, int RBB>
+struct Wgrad3Shape {
+    static constexpr int CA = RBA / 2, CB = RBB / 2;     // channels of x and dz
+    static constexpr int kTpm = 128 / CB;                // rows of dz (taps) of an MMA
+    static constexpr int kMpg = CB == 32 ? 1 : 2;        // MMAs that cover three taps
+    static constexpr int kN = 3 * CA;
+    static constexpr int kRows = 128;                    // rows per stage
+    static constexpr int kABytes = align1k((kRows + 3) * RBB);
+    static constexpr int kBBlock = kRows * RBA;
+    static constexpr int kStage = kABytes + 3 * kBBlock;
+    static constexpr int kTwo = (113 * 1024 - 1536) / kStage;     // stages that leave room for a second CTA on the SM
+    static constexpr int kStages = kTwo >= 2 ? kTwo : std::min(4, (kSmemMax - 1536) / kStage);
+    static constexpr int kSmem = 1024 + kStages * kStage + 512;
+    static constexpr uint32_t kCols = kMpg * kN <= 128 ? 128 : (kMpg * kN <= 256 ? 256 : 512);
+    static_assert(kStages >= 2, "shared memory");
+};
+
+template <int RBA, int RBB>
+__global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ CUtensorMap mapA,
+                                                        const __grid_constant__ CUtensorMap mapB, int chunk,
+                                                        unsigned int* __restrict__ err,
+                                                        const __grid_constant__ WgradJob job) {
+    using Sh = Wgrad3Shape<RBA, RBB>;
+    constexpr int ST = Sh::kStages, WL = Sh::kRows;
+    constexpr uint32_t idesc = umma_idesc(128, Sh::kN, true);
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + ST * Sh::kStage);
+    uint64_t* empty = full + ST;
+    uint64_t* done = empty + ST;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    volatile uint32_t* failed = tmem_slot + 1;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int g0 = blockIdx.x * 3;
+    const int r0 = blockIdx.y * chunk;
+    const int nk = (chunk + WL - 1) / WL;      // the last stage may be half used (chunk: a multiple of 64)
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < ST; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        *failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, Sh::kCols);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        const bool leader = elect_one();
+        int it = 0, s = 0;
+        uint32_t ph = 1u;
+        bool ok = true;
+        for (; it < nk; ++it) {
+            if (!mbar_wait(&empty[s], ph)) {
+                ok = false;
+                break;
+            }
+            if (leader) {
+                uint8_t* sa = base + s * Sh::kStage;
+                const int r = r0 + it * WL;
+                mbar_expect_tx(&full[s], (WL + 3) * RBB + 3 * Sh::kBBlock);
+                tma_load_2d(sa, &mapA, 0, r - 2, &full[s]);
+                for (int g = 0; g < 3; ++g)
+                    tma_load_2d(sa + Sh::kABytes + g * Sh::kBBlock, &mapB, 0, r + job.off[3 * (g0 + g)], &full[s]);
+            }
+            if (++s == ST) {
+                s = 0;
+                ph ^= 1u;
+            }
+        }
+        if (!ok && lane == 0) {
+            *failed = 1;
+            atomicOr(err, 8u);
+        }
+        if (!ok || *failed)
+            for (int i = max(0, it - ST); i < it; ++i) mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u);
+    } else if (warp == 1) {
+        const bool leader = elect_one();
+        int s = 0;
+        uint32_t ph = 0u;
+        const uint64_t a0 = mnmajor_desc(smem_u32(base), RBB, RBB);
+        const uint64_t b0 = mnmajor_desc(smem_u32(base) + Sh::kABytes, Sh::kBBlock, RBA);
+        for (int it = 0; it < nk; ++it) {
+            if (!mbar_wait(&full[s], ph)) {
+                if (lane == 0) {
+                    *failed = 1;
+                    atomicOr(err, 16u);
+                }
+                break;
+            }
+            fence_after();
+            const uint64_t as = a0 + (uint32_t)((s * Sh::kStage) >> 4);
+            const uint64_t bs = b0 + (uint32_t)((s * Sh::kStage) >> 4);
+            const int slices = min(WL, chunk - it * WL) / 16;
+            if (leader) {
+#pragma unroll
+                for (int j = 0; j < WL / 16; ++j)
+                    if (j < slices)
+#pragma unroll
+                        for (int m = 0; m < Sh::kMpg; ++m)
+                            umma_f16(tmem + m * Sh::kN, as + (m * Sh::kTpm + 16 * j) * (RBB / 16),
+                                     bs + 16 * j * (RBA / 16), idesc, (it | j) != 0);
+                umma_commit(&empty[s]);
+            }
+            __syncwarp();
+            if (++s == ST) {
+                s = 0;
+                ph ^= 1u;
+            }
+        }
+        if (leader) umma_commit(done);
+        __syncwarp();
+    } else if (warp >= 2) {
+        if (!mbar_wait(done, 0)) {
+            if (lane == 0) atomicOr(err, 32u);
+        } else {
+            fence_after();
+            const int quarter = warp & 3;
+            const int l = 32 * quarter + lane;
+            const int co = l % Sh::CB;
+            for (int m = 0; m < Sh::kMpg; ++m) {
+                const int d = 2 - (m * Sh::kTpm + l / Sh::CB);     // the same for all lanes of the warp
+                if (d < 0) continue;
+                const uint32_t taddr = tmem + m * Sh::kN + ((uint32_t)(32 * quarter) << 16);
+                for (int n = 0; n < Sh::kN; n += 32) {
+                    uint32_t u[32];
+                    tmem_ld32(taddr + n, u);
+                    tmem_wait_ld();
+                    float* dst = job.P + ((long long)blockIdx.y * 27 * Sh::CA +
+                                          (long long)(3 * (g0 + n / Sh::CA) + d) * Sh::CA + n % Sh::CA) * Sh::CB + co;
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) dst[q * Sh::CB] = __uint_as_float(u[q]);
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, Sh::kCols);
+}
+
 // ------------------------------------------------------------------ launch
 int g_sms = 0;
 
@@ -676,6 +839,22 @@ struct WgradK {
     }
 };
 
+template <int RBA, int RBB>
+struct Wgrad3K {
+    using Sh = Wgrad3Shape<RBA, RBB>;
+    static cudaError_t init() {
+        return cudaFuncSetAttribute(wgrad3_kernel<RBA, RBB>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::kSmem);
+    }
+    static cudaError_t launch(const WgradJob& j, unsigned int* err, cudaStream_t st) {
+        CUtensorMap ma, mb;
+        if (!make_map(&ma, j.dz, j.N, j.rows, j.N, RBB, Sh::kRows + 3) ||
+            !make_map(&mb, j.x, j.C, j.rows, j.C, RBA, Sh::kRows))
+            return cudaErrorInvalidValue;
+        wgrad3_kernel<RBA, RBB><<<dim3(3, j.S), 192, Sh::kSmem, st>>>(ma, mb, j.rows / j.S, err, j);
+        return cudaGetLastError();
+    }
+};
+
 // Every shape the network uses (C, N stored channels).
 #define LBMS_CONV_SHAPES(F)                                                                              \
     F(64, 32, 3, kOutRelu) F(64, 64, 3, kOutRelu) F(128, 64, 3, kOutRelu) F(128, 128, 3, kOutRelu)        \
@@ -685,7 +864,7 @@ struct WgradK {
     F(128, 64, 1, kOutReluBack) F(64, 32, 1, kOutHead) F(64, 32, 1, kOutReluBack)                         \
     F(128, 64, 1, kOutRelu) F(128, 64, 1, kOutHead)
 #define LBMS_WGRAD_SHAPES(F)                                                                        \
-    F(64, 1, 64, 1, 3) F(64, 1, 128, 1, 3) F(128, 1, 64, 1, 3) F(128, 1, 128, 1, 3) F(128, 1, 128, 2, 3) \
+    F(128, 1, 128, 2, 3)                                                                              \
     F(128, 2, 128, 1, 3) F(128, 2, 128, 2, 3) F(64, 1, 64, 1, 1) F(128, 2, 128, 1, 1) F(128, 2, 128, 2, 1)
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -700,6 +879,10 @@ cudaError_t conv_init() {
     if (e == cudaSuccess) e = ConvK<RB, N, NT, KIND>::init();
     LBMS_CONV_SHAPES(LBMS_INIT)
 #undef LBMS_INIT
+    if (e == cudaSuccess) e = Wgrad3K<64, 64>::init();
+    if (e == cudaSuccess) e = Wgrad3K<64, 128>::init();
+    if (e == cudaSuccess) e = Wgrad3K<128, 64>::init();
+    if (e == cudaSuccess) e = Wgrad3K<128, 128>::init();
 #define LBMS_INIT(A, NA, B, NB, NT) \
     if (e == cudaSuccess) e = WgradK<A, NA, B, NB, NT>::init();
     LBMS_WGRAD_SHAPES(LBMS_INIT)
@@ -745,6 +928,10 @@ cudaError_t umma_wgrad(const WgradJob& j, unsigned int* err, cudaStream_t st) {
     if ((j.C != 32 && j.C % 64) || (j.N != 32 && j.N % 64) || j.C < 32 || j.N < 32 ||
         (nt == 3 && (j.C > 128 || j.N > 128 || j.C % (rba / 2 * nba) || j.N % (rbb / 2 * nbb))))
         return cudaErrorInvalidValue;
+    if (nt == 3 && j.C <= 64 && j.N <= 64) {
+        if (j.C == 32) return j.N == 32 ? Wgrad3K<64, 64>::launch(j, err, st) : Wgrad3K<64, 128>::launch(j, err, st);
+        return j.N == 32 ? Wgrad3K<128, 64>::launch(j, err, st) : Wgrad3K<128, 128>::launch(j, err, st);
+    }
 #define LBMS_TRY(A, NA, B, NB, NT) \
     if (rba == A && nba == NA && rbb == B && nbb == NB && nt == NT) return WgradK<A, NA, B, NB, NT>::launch(j, err, st);
     LBMS_WGRAD_SHAPES(LBMS_TRY)

@@ -247,7 +247,9 @@ cudaError_t umma_conv(const ConvJob& j, unsigned int* err, cudaStream_t st);
 // P[z][t C + c][n] = sum over the rows r of chunk z of x[r + off[t]][c]
 // dz[r][n] (taps = 27, off[3 g + d] = off[3 g] + d), or P[z][c][n] with
 // taps = 1; x [rows][C], dz [rows][N], S chunks of rows / S (a multiple of 64)
-// rows each.
+// rows each.  With taps = 27 the last two rows of dz are zero, and at most 64
+// channels on either side a chunk takes the products whose x row off[3 g] on
+// from dz lies in it.
 struct WgradJob {
     const void* x = nullptr;
     const void* dz = nullptr;

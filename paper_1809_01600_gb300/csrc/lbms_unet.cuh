@@ -6,10 +6,13 @@
 // Layout.  Activations are channels-last BF16 rows [row][C] (C = 32, 64 or
 // 128 at the three levels, the smallest that holds the real channels; the
 // real channels first, zeros after).  Each volume of X x Y x Z voxels is
-// stored with a zero halo of one voxel per side, in Xp x Yp x Zp rows (Xp =
-// X + 2 rounded up to a multiple of 8, Yp = Y + 2, Zp = Z + 2), volumes one
-// after the other; the row count is padded to a multiple of 64 S (S chunks of
-// the reductions over rows).  The neighbour of a voxel at tap (dz, dy, dx) is
+// stored with a zero halo of one voxel in front of each row, plane and volume,
+// in Xp x Yp x Zp = (X + 1) x (Y + 1) x (Z + 1) rows, volumes one after the other:
+// the halo behind a row is the one in front of the next, and behind the last
+// volume come padding rows (zeros) and what TMA fills in (zeros).  A halo on
+// both sides and rows of a multiple of 8 took 9 % more rows at 96^3 and 18 % at
+// 64x32x32.  The row count is padded to a multiple of 64 S (S chunks of the
+// reductions over rows).  The neighbour of a voxel at tap (dz, dy, dx) is
 // then off = (dz Yp + dy) Xp + dx rows away, so a 3x3x3 convolution is an
 // implicit GEMM on the tensor cores (lbms_conv.cu).  What follows a product
 // is done on its accumulators: bias, ReLU, zero halo and the copy into the
@@ -31,10 +34,10 @@ constexpr int kULayers = 13;
 // Layout of one resolution level of a batch (all row counts below 2^31).
 struct Geo {
     int B = 0, X = 0, Y = 0, Z = 0;   // volumes; interior extents of one volume
-    int Xp = 0, Yp = 0, Zp = 0;       // extents with the halo (Xp a multiple of 8)
+    int Xp = 0, Yp = 0, Zp = 0;       // extents with the halo
     int64_t V = 0;                    // interior voxels of the batch
     int64_t R = 0;                    // rows of the layout, B Xp Yp Zp
-    int64_t Rp = 0;                   // rows processed: R padded to a multiple of 64 S
+    int64_t Rp = 0;                   // rows processed: R + 2 or more, a multiple of 64 S
     int S = 1;                        // chunks of the reductions over rows
 };
 
@@ -363,6 +366,10 @@ T* ualloc(lbms_unet* u, size_t count) {
 constexpr int64_t kChunkRows = 16384;
 constexpr int64_t kGemmMaxRows = 65535ll * 128;   // grid limit of the GEMM's row tiles
 
+// Zero rows behind the last volume that the weight gradients of the 3x3x3
+// convolutions need (they reach dz up to two rows late).
+constexpr int64_t kTailRows = 2;
+
 int64_t splits_for(int64_t R) { return std::max<int64_t>(1, (R + kChunkRows - 1) / kChunkRows); }
 int64_t padded_rows(int64_t R) {
     const int64_t q = 64 * splits_for(R);
@@ -375,13 +382,13 @@ Geo make_geo(int B, int X, int Y, int Z) {
     g.X = X;
     g.Y = Y;
     g.Z = Z;
-    g.Xp = (X + 2 + 7) / 8 * 8;
-    g.Yp = Y + 2;
-    g.Zp = Z + 2;
+    g.Xp = X + 1;
+    g.Yp = Y + 1;
+    g.Zp = Z + 1;
     g.V = (int64_t)B * X * Y * Z;
     g.R = (int64_t)B * g.Xp * g.Yp * g.Zp;
-    g.S = (int)splits_for(g.R);
-    g.Rp = padded_rows(g.R);
+    g.S = (int)splits_for(g.R + kTailRows);
+    g.Rp = padded_rows(g.R + kTailRows);
     return g;
 }
 
