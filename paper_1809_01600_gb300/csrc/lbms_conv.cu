@@ -2,8 +2,8 @@
 // (the 3-D U-Net), plain products (the pointwise network), input gradients and
 // weight gradients, with what follows each product done on its accumulators.
 //
-// Activations are stored in a layout with a zero halo of one voxel per side,
-// so the neighbour of every interior voxel at tap t = (dz, dy, dx) lies a
+// Activations are stored in a layout with a zero halo of one voxel between
+// rows, planes and volumes, so the neighbour of every interior voxel at tap t = (dz, dy, dx) lies a
 // fixed number of rows off(t) away and a convolution is an implicit GEMM: the
 // A tile of tap t is the activation matrix [rows][C] read at shifted rows
 // (TMA zero-fills rows outside it).  The three taps of a (dz, dy) row differ
@@ -15,12 +15,12 @@
 // memory per MMA whatever N is, so at N = 32 (the full resolution) an MMA
 // takes about 50 cycles where its arithmetic takes 8; storing 32 channels
 // instead of 64 there quartered the MMAs.  A training step on 4 volumes of
-// 96^3 takes 9.3 ms, on 8 of 64x32x32 2.85 ms (43.5 and 7.45 with 64 channels
+// 96^3 takes 6.6 ms, on 8 of 64x32x32 1.7 ms (43.5 and 7.45 with 64 channels
 // stored, FP32 products in memory, transposed copies for the weight gradients
-// and row-wise kernels between the products).  Of the 9.3 ms the 32-channel
-// convolutions take 0.40 ms each, their input gradients 0.36, their weight
-// gradients 0.43; reading the timer on every barrier wait and issuing from a
-// single lane's branch cost twice that (17.2 ms a step).
+// and row-wise kernels between the products).  Of the 6.6 ms the 32-channel
+// convolutions take 0.35 ms each (66 cycles an MMA), their input gradients
+// 0.28, their weight gradients 0.22.  Reading the timer on every barrier wait
+// and issuing from a single lane's branch cost twice that.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -34,6 +34,7 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kSmemMax = 227 * 1024;
+constexpr int kConvThreads = 64 + 2 * 128;
 constexpr int align1k(int b) { return (b + 1023) / 1024 * 1024; }
 
 // Interior coordinates of row r; false for halo and padding rows.
@@ -80,7 +81,11 @@ __device__ __forceinline__ float column_sum(float (&v)[32], int lane) {
 //
 // A persistent CTA per SM takes 128-row tiles in turn: warp 0 issues the TMA
 // loads of a ring of stages, warp 1 the MMAs into one of two TMEM
-// accumulators, warps 2-5 the epilogue of the other.  The weights stay in
+// accumulators, warps 2-5 the epilogues of the tiles in the first, warps 6-9 of
+// those in the second; what an epilogue reads from memory it loads before the
+// wait for its accumulator.  Plain products are bound by their epilogues: the
+// head of 4 volumes of 96^3 takes 0.144 ms and its input gradient 0.156, with
+// one set of epilogue warps 0.197 and 0.235.  The weights stay in
 // shared memory for the whole launch where they fit (27 N RB <= 108 KB, the
 // layers at full resolution), else each stage brings its three taps'.
 template <int RB, int N, int NT, int KIND>
@@ -90,11 +95,11 @@ struct ConvShape {
     static constexpr int kARows = NT == 3 ? 130 : 128;
     static constexpr int kABytes = align1k(kARows * RB);
     static constexpr int kBTile = N * RB;
-    static constexpr int kGps = NT == 3 && RB == 64 ? 3 : 1;   // windows (dz, dy rows) of a stage
+    static constexpr int kGps = NT == 3 && RB == 64 && KIND != kOutSplit ? 3 : 1;   // windows (dz, dy rows) of a stage
     static constexpr int kStage = kGps * kABytes + (kResident ? 0 : NT * kBTile);
     static_assert(kGps == 1 || kResident, "a stage holds the weights of one window");
     static constexpr int kResBytes = kResident ? align1k(27 * kBTile) : 0;
-    static constexpr int kStageFloats = KIND == kOutSplit ? 4 * 32 * 65 : 0;   // split: rows of each epilogue warp
+    static constexpr int kStageFloats = KIND == kOutSplit ? 8 * 32 * 65 : 0;   // split: rows of each epilogue warp
     static constexpr int kFixed = 1024 + kResBytes + kStageFloats * 4 + N * 4 + 512;
     static constexpr int kFit = (kSmemMax - kFixed) / kStage;
     static constexpr int kStages = kFit < 8 ? kFit : 8;
@@ -104,7 +109,7 @@ struct ConvShape {
 };
 
 template <int RB, int N, int NT, int KIND>
-__global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CUtensorMap mapA,
+__global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const __grid_constant__ CUtensorMap mapA,
                                                       const __grid_constant__ CUtensorMap mapB, int rows, int nblk,
                                                       int ntn, unsigned int* __restrict__ err,
                                                       const __grid_constant__ ConvJob job) {
@@ -143,7 +148,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
         *failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int c = threadIdx.x; c < N; c += 192) cs[c] = 0.0f;
+    for (int c = threadIdx.x; c < N; c += kConvThreads) cs[c] = 0.0f;
     if (warp == 0) tmem_alloc(tmem_slot, Sh::kCols);
     fence_before();
     __syncthreads();
@@ -255,23 +260,31 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
     } else if (warp >= 2) {
         const ConvEpilogue& ep = job.ep;
         const int quarter = warp & 3;               // TMEM lanes this warp may read
-        int nt = 0;
+        const int b = (warp - 2) >> 2;              // its accumulator
+        int nt = b;
         double loss = 0.0;
         float hs[3] = {0.0f, 0.0f, 0.0f};
-        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++nt) {
+        for (int tile = blockIdx.x + b * gridDim.x; tile < tiles; tile += 2 * gridDim.x, nt += 2) {
             const int m0 = tile / ntn * 128, n0 = tile % ntn * N;
-            const int b = nt & 1;
-            if (!mbar_wait(&acc_full[b], (uint32_t)(nt >> 1) & 1u)) {
-                if (lane == 0) atomicOr(err, 4u);
-                break;
-            }
-            fence_after();
             const long long row = m0 + 32 * quarter + lane;
             const bool valid = row < rows;
             int x = 0, y = 0, z = 0, vb = 0;
             const bool in = KIND == kOutRelu && NT == 1 ? valid   // a plain layer: every row
                             : KIND != kOutReluBack && KIND != kOutStore && KIND != kOutHead &&
                                   voxel_of(ep.g, row, x, y, z, vb);
+            uint4 acts[KIND == kOutReluBack ? N / 8 : 1];
+            float4 target = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if constexpr (KIND == kOutReluBack) {
+                const uint4* act = reinterpret_cast<const uint4*>(static_cast<const bf16*>(ep.act) + row * job.N + n0);
+#pragma unroll
+                for (int q = 0; q < N / 8; ++q) acts[q] = valid ? __ldg(act + q) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            if (KIND == kOutHead && ep.T && valid) target = __ldg(reinterpret_cast<const float4*>(ep.T) + row);
+            if (!mbar_wait(&acc_full[b], (uint32_t)(nt >> 1) & 1u)) {
+                if (lane == 0) atomicOr(err, 4u);
+                break;
+            }
+            fence_after();
             const uint32_t taddr = tmem + b * N + ((uint32_t)(32 * quarter) << 16);
             constexpr int kChunks = KIND == kOutHead ? 1 : N / 32;
 #pragma unroll
@@ -319,11 +332,10 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                     }
                 } else if constexpr (KIND == kOutReluBack) {
                     float v[32];
-                    const uint4* act = reinterpret_cast<const uint4*>(static_cast<const bf16*>(ep.act) + row * job.N + n0 + c0);
                     uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(ep.out) + row * job.N + n0 + c0);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const uint4 av = valid ? __ldg(act + q) : make_uint4(0u, 0u, 0u, 0u);
+                        const uint4 av = acts[4 * ch + q];
                         const uint32_t aw[4] = {av.x, av.y, av.z, av.w};
                         uint32_t o[4];
 #pragma unroll
@@ -415,11 +427,10 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
                             for (int c = 0; c < 3; ++c) ep.Y[row * 4 + c] = yv[c];
                         }
                         if (ep.T) {
-                            const float4 t = __ldg(reinterpret_cast<const float4*>(ep.T) + row);
-                            const float tv[3] = {t.x, t.y, t.z};
+                            const float tv[3] = {target.x, target.y, target.z};
 #pragma unroll
                             for (int c = 0; c < 3; ++c) {
-                                const float d = (yv[c] - tv[c]) * t.w;
+                                const float d = (yv[c] - tv[c]) * target.w;
                                 loss += (double)d * d;
                                 gv[c] = ep.grad_scale * d;
                                 hs[c] += gv[c];
@@ -434,7 +445,7 @@ __global__ void __launch_bounds__(192, 1) conv_kernel(const __grid_constant__ CU
             }
         }
         if constexpr (KIND == kOutReluBack || KIND == kOutSplit) {
-            asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // the epilogue warps
             const int e = (int)threadIdx.x - 64;
             if (e < N && (KIND == kOutReluBack ? ntn == 1 : e < ep.w)) atomicAdd(&ep.gb[e], cs[e]);
         }
@@ -449,7 +460,7 @@ double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
 #pragma unroll
                     for (int c = 0; c < 4; ++c) atomicAdd(&ep.loss[c], sum[c]);
                     __threadfence();
-                    if (atomicAdd(ep.done, 1u) + 1u == 4u * gridDim.x) {   // the last epilogue warp
+                    if (atomicAdd(ep.done, 1u) + 1u == 8u * gridDim.x) {   // the last epilogue warp
                         __threadfence();
 #pragma unroll
                         for (int c = 0; c < 3; ++c) ep.gb[c] = (float)__ldcg(&ep.loss[1 + c]);
@@ -468,50 +479,45 @@ double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
 // channels, i.e. MN-major with K running over the rows: no transposed copies.
 // RBA, NBA: row bytes and number of the A blocks of a window (32 channels: 64,
 // 1; 64: 128, 1; 128: 128, 2); RBB, NBB the same of dz.  An MMA's 128 rows are
-// the channels of 4, 2 or 1 consecutive dx taps: the next block of M starts
-// one row further into the same window (the leading offset of the
-// descriptor), and the blocks past the third tap are not stored.
+// the channels of 2 or 1 consecutive dx taps: the next block of M starts one
+// row further into the same window (the leading offset of the descriptor), and
+// the block past the third tap is not stored.
 //
-// A CTA reduces one chunk of rows for GR of the nine (dz, dy) rows of taps
-// (plain product: GR of its 128-channel tiles), all accumulators in TMEM, in
-// the order of the rows.  GR is the launch's choice: large where the chunks
-// alone fill the GPU (dz is then read once), 1 where they do not.
+// A CTA reduces one chunk of rows for one of the nine (dz, dy) rows of taps
+// (plain product: one of its 128-channel tiles) in the order of the rows.
 constexpr int kWL = 64;                  // rows per stage
 constexpr int kWRows = kWL + 3;          // window rows (taps up to 3 rows on)
 
 template <int RBA, int NBA, int RBB, int NBB, int NT>
 struct WgradShape {
-    static constexpr int kTpm = NT == 1 ? 1 : (NBA == 2 ? 1 : (RBA == 128 ? 2 : 4));   // taps per MMA
-    static constexpr int kMpg = NT == 1 ? 1 : (3 + kTpm - 1) / kTpm;                   // MMAs per group
+    static constexpr int kTpm = NT == 1 ? 1 : (NBA == 2 ? 1 : 2);   // taps per MMA
+    static constexpr int kMpg = NT == 1 ? 1 : (3 + kTpm - 1) / kTpm;    // MMAs per K slice
     static constexpr int kN = RBB / 2 * NBB;
     static constexpr int kABlock = align1k(kWRows * RBA);
     static constexpr int kBBlock = kWL * RBB;
-    static constexpr int kGroupCols = kMpg * kN;
-    __host__ __device__ static constexpr int stage(int gr) { return gr * NBA * kABlock + NBB * kBBlock; }
-    static constexpr int max_groups() {
-        return 9 * kGroupCols <= 512 && 3 * stage(9) + 2048 <= kSmemMax ? 9 : (3 * kGroupCols <= 512 ? 3 : 1);
-    }
-    static int stages(int gr) { return std::min(8, (kSmemMax - 2048) / stage(gr)); }
+    static constexpr uint32_t kCols = kMpg * kN <= 32 ? 32 : (kMpg * kN <= 128 ? 128 : (kMpg * kN <= 256 ? 256 : 512));
+    static constexpr int kStage = NBA * kABlock + NBB * kBBlock;
+    static constexpr int kStages = std::min(8, (kSmemMax - 2048) / kStage);
 };
 
 template <int RBA, int NBA, int RBB, int NBB, int NT>
 __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ CUtensorMap mapA,
-                                                       const __grid_constant__ CUtensorMap mapB, int chunk, int GR,
-                                                       int ST, uint32_t cols, unsigned int* __restrict__ err,
+                                                       const __grid_constant__ CUtensorMap mapB, int chunk, int ST,
+                                                       unsigned int* __restrict__ err,
                                                        const __grid_constant__ WgradJob job) {
     using Sh = WgradShape<RBA, NBA, RBB, NBB, NT>;
     constexpr uint32_t idesc = umma_idesc(128, Sh::kN, true);
     constexpr int CA = RBA / 2 * NBA;        // channels of a window
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int stage = Sh::stage(GR);
+    constexpr int stage = Sh::kStage;
     uint64_t* full = reinterpret_cast<uint64_t*>(base + ST * stage);
     uint64_t* empty = full + ST;
     uint64_t* done = empty + ST;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* failed = tmem_slot + 1;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int g0 = blockIdx.x * GR;
+    const int g = blockIdx.x;
     const int n0 = blockIdx.z * Sh::kN;
     const int r0 = blockIdx.y * chunk;
     const int nk = chunk / kWL;
@@ -525,7 +531,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
         *failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(tmem_slot, cols);
+    if (warp == 0) tmem_alloc(tmem_slot, Sh::kCols);
     fence_before();
     __syncthreads();
     fence_after();
@@ -544,14 +550,12 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
             if (leader) {
                 uint8_t* sa = base + s * stage;
                 const int r = r0 + it * kWL;
-                mbar_expect_tx(&full[s], GR * NBA * kWRows * RBA + NBB * Sh::kBBlock);
-                for (int g = 0; g < GR; ++g)
-                    for (int c = 0; c < NBA; ++c)
-                        tma_load_2d(sa + (g * NBA + c) * Sh::kABlock, &mapA,
-                                    (NT == 1 ? (g0 + g) * CA : 0) + c * (RBA / 2),
-                                    NT == 1 ? r : r + job.off[3 * (g0 + g)], &full[s]);
+                mbar_expect_tx(&full[s], NBA * kWRows * RBA + NBB * Sh::kBBlock);
+                for (int c = 0; c < NBA; ++c)
+                    tma_load_2d(sa + c * Sh::kABlock, &mapA, (NT == 1 ? g * CA : 0) + c * (RBA / 2),
+                                NT == 1 ? r : r + job.off[3 * g], &full[s]);
                 for (int c = 0; c < NBB; ++c)
-                    tma_load_2d(sa + GR * NBA * Sh::kABlock + c * Sh::kBBlock, &mapB, n0 + c * (RBB / 2), r, &full[s]);
+                    tma_load_2d(sa + NBA * Sh::kABlock + c * Sh::kBBlock, &mapB, n0 + c * (RBB / 2), r, &full[s]);
             }
             if (++s == ST) {
                 s = 0;
@@ -569,7 +573,7 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
         int s = 0;
         uint32_t ph = 0u;
         const uint64_t a0 = mnmajor_desc(smem_u32(base), NBA == 2 ? Sh::kABlock : RBA, RBA);
-        const uint64_t b0 = mnmajor_desc(smem_u32(base) + GR * NBA * Sh::kABlock, Sh::kBBlock, RBB);
+        const uint64_t b0 = mnmajor_desc(smem_u32(base) + NBA * Sh::kABlock, Sh::kBBlock, RBB);
         for (int it = 0; it < nk; ++it) {
             if (!mbar_wait(&full[s], ph)) {
                 if (lane == 0) {
@@ -579,20 +583,17 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
                 break;
             }
             fence_after();
+            const uint64_t as = a0 + (uint32_t)((s * stage) >> 4);
             const uint64_t bs = b0 + (uint32_t)((s * stage) >> 4);
-            for (int g = 0; g < GR; ++g) {
-                const uint64_t as = a0 + (uint32_t)((s * stage + g * NBA * Sh::kABlock) >> 4);
-                if (leader) {
+            if (leader) {
 #pragma unroll
-                    for (int m = 0; m < Sh::kMpg; ++m)
+                for (int m = 0; m < Sh::kMpg; ++m)
 #pragma unroll
-                        for (int j = 0; j < kWL / 16; ++j)
-                            umma_f16(tmem + g * Sh::kGroupCols + m * Sh::kN, as + (m * Sh::kTpm + 16 * j) * (RBA / 16),
-                                     bs + 16 * j * (RBB / 16), idesc, (it | j) != 0);
-                }
-                __syncwarp();
+                    for (int j = 0; j < kWL / 16; ++j)
+                        umma_f16(tmem + m * Sh::kN, as + (m * Sh::kTpm + 16 * j) * (RBA / 16), bs + 16 * j * (RBB / 16),
+                                 idesc, (it | j) != 0);
+                umma_commit(&empty[s]);
             }
-            if (leader) umma_commit(&empty[s]);
             __syncwarp();
             if (++s == ST) {
                 s = 0;
@@ -610,31 +611,30 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
             const int l = 32 * quarter + lane;
             const int tb = l / CA, c = l % CA;       // tap within the MMA, channel
             const int K = NT == 1 ? job.C : 27 * job.C;
-            for (int g = 0; g < GR; ++g)
-                for (int m = 0; m < Sh::kMpg; ++m) {
-                    const int d = m * Sh::kTpm + tb;
-                    const bool keep = NT == 1 ? (g0 + g) * CA + l < job.C && tb == 0 : d < 3;
-                    const long long prow = NT == 1 ? (long long)(g0 + g) * CA + c : (long long)(3 * (g0 + g) + d) * job.C + c;
-                    float4* dst = reinterpret_cast<float4*>(job.P + ((long long)blockIdx.y * K + prow) * job.N + n0);
-                    const uint32_t taddr = tmem + g * Sh::kGroupCols + m * Sh::kN + ((uint32_t)(32 * quarter) << 16);
+            for (int m = 0; m < Sh::kMpg; ++m) {
+                const int d = m * Sh::kTpm + tb;
+                const bool keep = NT == 1 ? g * CA + l < job.C && tb == 0 : d < 3;
+                const long long prow = NT == 1 ? (long long)g * CA + c : (long long)(3 * g + d) * job.C + c;
+                float4* dst = reinterpret_cast<float4*>(job.P + ((long long)blockIdx.y * K + prow) * job.N + n0);
+                const uint32_t taddr = tmem + m * Sh::kN + ((uint32_t)(32 * quarter) << 16);
 #pragma unroll
-                    for (int n = 0; n < Sh::kN; n += 32) {
-                        uint32_t u[32];
-                        tmem_ld32(taddr + n, u);
-                        tmem_wait_ld();
-                        if (keep && n0 + n < job.N) {
+                for (int n = 0; n < Sh::kN; n += 32) {
+                    uint32_t u[32];
+                    tmem_ld32(taddr + n, u);
+                    tmem_wait_ld();
+                    if (keep && n0 + n < job.N) {
 #pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                dst[n / 4 + q] = make_float4(__uint_as_float(u[4 * q]), __uint_as_float(u[4 * q + 1]),
-                                                             __uint_as_float(u[4 * q + 2]), __uint_as_float(u[4 * q + 3]));
-                        }
+                        for (int q = 0; q < 8; ++q)
+                            dst[n / 4 + q] = make_float4(__uint_as_float(u[4 * q]), __uint_as_float(u[4 * q + 1]),
+                                                         __uint_as_float(u[4 * q + 2]), __uint_as_float(u[4 * q + 3]));
                     }
                 }
+            }
         }
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, cols);
+    if (warp == 0) tmem_dealloc(tmem, Sh::kCols);
 }
 
 // The weight gradient of a 3x3x3 convolution with at most 64 channels on
@@ -644,30 +644,31 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
 // windows of a dz.  With x at row p and dz at row p - 2 + j the product belongs
 // to tap dx = 2 - j.  An MMA reads its 128-row operand from shared memory at 32
 // cycles whatever its columns are, so 96 or 192 columns instead of 32 or 64
-// take a third of the time: 4 volumes of 96^3, 32 by 32 channels WG3_FIGURES.
-template <int RBA, int RBB>
+// take a third of the MMAs: 4 volumes of 96^3, 32 by 32 channels 0.43 -> 0.22 ms.
+// W windows a CTA: 3, or 1 where three would leave half the SMs without work.
+template <int RBA, int RBB, int W>
 struct Wgrad3Shape {
     static constexpr int CA = RBA / 2, CB = RBB / 2;     // channels of x and dz
     static constexpr int kTpm = 128 / CB;                // rows of dz (taps) of an MMA
     static constexpr int kMpg = CB == 32 ? 1 : 2;        // MMAs that cover three taps
-    static constexpr int kN = 3 * CA;
+    static constexpr int kN = W * CA;
     static constexpr int kRows = 128;                    // rows per stage
     static constexpr int kABytes = align1k((kRows + 3) * RBB);
     static constexpr int kBBlock = kRows * RBA;
-    static constexpr int kStage = kABytes + 3 * kBBlock;
+    static constexpr int kStage = kABytes + W * kBBlock;
     static constexpr int kTwo = (113 * 1024 - 1536) / kStage;     // stages that leave room for a second CTA on the SM
-    static constexpr int kStages = kTwo >= 2 ? kTwo : std::min(4, (kSmemMax - 1536) / kStage);
+    static constexpr int kStages = kTwo >= 2 ? std::min(4, kTwo) : std::min(4, (kSmemMax - 1536) / kStage);
     static constexpr int kSmem = 1024 + kStages * kStage + 512;
     static constexpr uint32_t kCols = kMpg * kN <= 128 ? 128 : (kMpg * kN <= 256 ? 256 : 512);
     static_assert(kStages >= 2, "shared memory");
 };
 
-template <int RBA, int RBB>
+template <int RBA, int RBB, int W>
 __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ CUtensorMap mapA,
                                                         const __grid_constant__ CUtensorMap mapB, int chunk,
                                                         unsigned int* __restrict__ err,
                                                         const __grid_constant__ WgradJob job) {
-    using Sh = Wgrad3Shape<RBA, RBB>;
+    using Sh = Wgrad3Shape<RBA, RBB, W>;
     constexpr int ST = Sh::kStages, WL = Sh::kRows;
     constexpr uint32_t idesc = umma_idesc(128, Sh::kN, true);
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ 
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* failed = tmem_slot + 1;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int g0 = blockIdx.x * 3;
+    const int g0 = blockIdx.x * W;
     const int r0 = blockIdx.y * chunk;
     const int nk = (chunk + WL - 1) / WL;      // the last stage may be half used (chunk: a multiple of 64)
 
@@ -710,9 +711,9 @@ __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ 
             if (leader) {
                 uint8_t* sa = base + s * Sh::kStage;
                 const int r = r0 + it * WL;
-                mbar_expect_tx(&full[s], (WL + 3) * RBB + 3 * Sh::kBBlock);
+                mbar_expect_tx(&full[s], (WL + 3) * RBB + W * Sh::kBBlock);
                 tma_load_2d(sa, &mapA, 0, r - 2, &full[s]);
-                for (int g = 0; g < 3; ++g)
+                for (int g = 0; g < W; ++g)
                     tma_load_2d(sa + Sh::kABytes + g * Sh::kBBlock, &mapB, 0, r + job.off[3 * (g0 + g)], &full[s]);
             }
             if (++s == ST) {
@@ -807,7 +808,7 @@ struct ConvK {
             !make_map(&mb, j.W, j.taps * j.C, j.N, j.taps * j.C, RB, N))
             return cudaErrorInvalidValue;
         const int tiles = (j.rows + 127) / 128 * ntn;
-        conv_kernel<RB, N, NT, KIND><<<std::min(tiles, g_sms), 192, Sh::kSmem, st>>>(ma, mb, j.rows, nblk, ntn, err, j);
+        conv_kernel<RB, N, NT, KIND><<<std::min(tiles, g_sms), kConvThreads, Sh::kSmem, st>>>(ma, mb, j.rows, nblk, ntn, err, j);
         return cudaGetLastError();
     }
 };
@@ -822,36 +823,42 @@ struct WgradK {
     static cudaError_t launch(const WgradJob& j, unsigned int* err, cudaStream_t st) {
         constexpr int CA = RBA / 2 * NBA;
         const int groups = NT == 1 ? (j.C + CA - 1) / CA : 9;
-        int gr = NT == 1 ? 1 : Sh::max_groups();
-        while (gr > 1 && j.S * (9 / gr) < 2 * g_sms) gr /= 3;
         CUtensorMap ma, mb;
         if (!make_map(&ma, j.x, j.C, j.rows, j.C, RBA, kWRows) || !make_map(&mb, j.dz, j.N, j.rows, j.N, RBB, kWL))
             return cudaErrorInvalidValue;
         // two CTAs an SM for the plain products of the pointwise network, whose chunks are a few stages long
         const int nk = j.rows / j.S / kWL;
-        const int st_n = NT == 1 && nk <= 16 ? std::min(3, Sh::stages(gr)) : Sh::stages(gr);
-        const int smem = 1024 + st_n * Sh::stage(gr) + 512;
-        uint32_t cols = 32;
-        while ((int)cols < gr * Sh::kGroupCols) cols *= 2;
-        wgrad_kernel<RBA, NBA, RBB, NBB, NT><<<dim3(groups / gr, j.S, (j.N + Sh::kN - 1) / Sh::kN), 192, smem, st>>>(
-            ma, mb, j.rows / j.S, gr, st_n, cols, err, j);
+        const int st_n = NT == 1 && nk <= 16 ? std::min(3, Sh::kStages) : Sh::kStages;
+        wgrad_kernel<RBA, NBA, RBB, NBB, NT>
+            <<<dim3(groups, j.S, (j.N + Sh::kN - 1) / Sh::kN), 192, 1024 + st_n * Sh::kStage + 512, st>>>(
+                ma, mb, j.rows / j.S, st_n, err, j);
         return cudaGetLastError();
     }
 };
 
 template <int RBA, int RBB>
 struct Wgrad3K {
-    using Sh = Wgrad3Shape<RBA, RBB>;
-    static cudaError_t init() {
-        return cudaFuncSetAttribute(wgrad3_kernel<RBA, RBB>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::kSmem);
+    template <int W>
+    static cudaError_t init_w() {
+        return cudaFuncSetAttribute(wgrad3_kernel<RBA, RBB, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    Wgrad3Shape<RBA, RBB, W>::kSmem);
     }
-    static cudaError_t launch(const WgradJob& j, unsigned int* err, cudaStream_t st) {
+    static cudaError_t init() {
+        const cudaError_t e = init_w<1>();
+        return e == cudaSuccess ? init_w<3>() : e;
+    }
+    template <int W>
+    static cudaError_t launch_w(const WgradJob& j, unsigned int* err, cudaStream_t st) {
+        using Sh = Wgrad3Shape<RBA, RBB, W>;
         CUtensorMap ma, mb;
         if (!make_map(&ma, j.dz, j.N, j.rows, j.N, RBB, Sh::kRows + 3) ||
             !make_map(&mb, j.x, j.C, j.rows, j.C, RBA, Sh::kRows))
             return cudaErrorInvalidValue;
-        wgrad3_kernel<RBA, RBB><<<dim3(3, j.S), 192, Sh::kSmem, st>>>(ma, mb, j.rows / j.S, err, j);
+        wgrad3_kernel<RBA, RBB, W><<<dim3(9 / W, j.S), 192, Sh::kSmem, st>>>(ma, mb, j.rows / j.S, err, j);
         return cudaGetLastError();
+    }
+    static cudaError_t launch(const WgradJob& j, unsigned int* err, cudaStream_t st) {
+        return 6 * j.S < g_sms ? launch_w<1>(j, err, st) : launch_w<3>(j, err, st);
     }
 };
 

@@ -294,6 +294,7 @@ struct lbms_unet {
     int64_t vcap = 0;            // interior voxels of one batch at most
     // activations and scratch, sized for the largest batch layout so far (grown on demand)
     int64_t cap[3] = {0, 0, 0};  // rows per level the buffers hold
+    size_t splits[3] = {0, 0, 0};   // and chunks of the reductions the partials hold
     bf16 *x0 = nullptr, *e1a = nullptr, *e1 = nullptr, *c1 = nullptr, *d1a = nullptr, *d1 = nullptr;
     bf16 *p1 = nullptr, *e2a = nullptr, *e2 = nullptr, *c2 = nullptr, *d2a = nullptr, *d2 = nullptr;
     bf16 *p2 = nullptr, *e3a = nullptr, *e3 = nullptr;
@@ -360,9 +361,11 @@ T* ualloc(lbms_unet* u, size_t count) {
     return static_cast<T*>(p);
 }
 
-// The reductions over rows (weight gradients) are split in S chunks of at
-// most kChunkRows (+ 63) rows, so that one CTA of the tensor-core GEMM
-// streams a few MB and ends far inside the GEMM's bound on each wait.
+// The reductions over rows (weight gradients) are split in S chunks, of as many
+// voxels as 16384 rows hold where the halo lies on both sides of a row (of a
+// multiple of 8), a plane and a volume.  The tensor cores' FP32 accumulators
+// truncate, so a chunk's length is its error: 2e-5 to 3e-5 of a gradient at this
+// length, and 3.5e-5 more with chunks 2.4 times as long.
 constexpr int64_t kChunkRows = 16384;
 constexpr int64_t kGemmMaxRows = 65535ll * 128;   // grid limit of the GEMM's row tiles
 
@@ -370,10 +373,9 @@ constexpr int64_t kGemmMaxRows = 65535ll * 128;   // grid limit of the GEMM's ro
 // convolutions need (they reach dz up to two rows late).
 constexpr int64_t kTailRows = 2;
 
-int64_t splits_for(int64_t R) { return std::max<int64_t>(1, (R + kChunkRows - 1) / kChunkRows); }
-int64_t padded_rows(int64_t R) {
-    const int64_t q = 64 * splits_for(R);
-    return (R + q - 1) / q * q;
+int64_t splits_for(int B, int X, int Y, int Z) {
+    const int64_t R = (int64_t)B * ((X + 9) / 8 * 8) * (Y + 2) * (Z + 2);
+    return std::max<int64_t>(1, (R + kChunkRows - 1) / kChunkRows);
 }
 
 Geo make_geo(int B, int X, int Y, int Z) {
@@ -387,8 +389,9 @@ Geo make_geo(int B, int X, int Y, int Z) {
     g.Zp = Z + 1;
     g.V = (int64_t)B * X * Y * Z;
     g.R = (int64_t)B * g.Xp * g.Yp * g.Zp;
-    g.S = (int)splits_for(g.R + kTailRows);
-    g.Rp = padded_rows(g.R + kTailRows);
+    g.S = (int)splits_for(B, X, Y, Z);
+    const int64_t q = 64 * (int64_t)g.S;
+    g.Rp = (g.R + kTailRows + q - 1) / q * q;
     return g;
 }
 
@@ -412,18 +415,20 @@ bool levels_fit(const Levels& v) {
 // Grows the activation and scratch buffers to hold the layout of `v`.
 lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
     int64_t c[3];
+    size_t sp[3];
     bool grow = false;
     for (int l = 0; l < 3; ++l) {
         c[l] = std::max(u->cap[l], v.g[l].Rp);
-        grow = grow || c[l] > u->cap[l];
+        sp[l] = std::max<size_t>(u->splits[l], v.g[l].S);
+        grow = grow || c[l] > u->cap[l] || sp[l] > u->splits[l];
     }
     if (!grow) return LBMS_OK;
     UCK(cudaDeviceSynchronize(), "U-Net buffers");
     for (void* p : u->bufs) cudaFree(p);
     u->bufs.clear();
-    for (int l = 0; l < 3; ++l) u->cap[l] = 0;
+    for (int l = 0; l < 3; ++l) u->cap[l] = u->splits[l] = 0;
     const size_t c0 = c[0], c1 = c[1], c2 = c[2];
-    const size_t s0 = splits_for(c0), s1 = splits_for(c1), s2 = splits_for(c2);
+    const size_t s0 = sp[0], s1 = sp[1], s2 = sp[2];
     u->P_floats = std::max({s0 * 64 * 864, s1 * 128 * 1728, s2 * 128 * 3456, s1 * 256 * 64, s2 * 512 * 128});
     bool ok = true;
     auto get = [&](size_t bytes) {
@@ -474,7 +479,10 @@ lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
         u->bufs.clear();
         return ufail(u, LBMS_ENOMEM, "U-Net buffers for %lld rows", (long long)c0);
     }
-    for (int l = 0; l < 3; ++l) u->cap[l] = c[l];
+    for (int l = 0; l < 3; ++l) {
+        u->cap[l] = c[l];
+        u->splits[l] = sp[l];
+    }
     return LBMS_OK;
 }
 
