@@ -235,6 +235,12 @@ def variant_key(info):
     return f"{info.tile_cells}x{info.tile_min_blocks}/t{info.threads_per_cell}/nb{info.neighbour_bits}"
 
 
+def step_kernel_name(forced_variant, threads_per_cell):
+    if forced_variant:
+        return "step_kernel_cell" if threads_per_cell == 1 else "step_kernel"
+    return "step_tile_kernel" if threads_per_cell == 1 else "step_small_kernel"
+
+
 def ncu_traffic(workload, precision, variant):
     """DRAM bytes per launch of the step kernel variant in use, from the
     committed ncu summary; valid only while the kernel sources are unchanged."""
@@ -542,7 +548,7 @@ def main():
                 "peak_source": peak_kind, "bytes_per_fluid_cell": bpc, "variant": variant_key(tinfo),
                 "algorithmic_bytes_per_launch": nf * bpc,
                 "kernel": "%s<%s, X %s, h %s>" % (
-                    "step_kernel_cell" if tinfo.threads_per_cell == 1 else "step_kernel",
+                    step_kernel_name(args.step_variant, tinfo.threads_per_cell),
                     "D3Q19" if case.dim == 3 else "D2Q9",
                     "double" if args.precision == "fp64" else "float pair",
                     {"fp64": "double", "fp32": "float", "fp16": "__half"}[args.precision])}

@@ -34,8 +34,9 @@ constexpr int kVariantPerCell[kStepVariants] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 1};
 // cells, us per step), blocks per SM 5 / 6 / 8 / 9 / 10 / 12: FP32 151 / 151 /
 // 143 / 153 / 140 / 191, FP64 2231 / 2253 / 2297 / 2306 / 2306 / 2308, FP16 at
 // 8 / 9 / 10 / 12: 105 / 104 / 101 / 125; 2-D FP32 (1.22 M cells) 59 up to 10,
-// 56.5 at 12, FP16 44.8 at any.  Prefetch none / 16 / 24 / 48 thousand cells ahead: FP32 155 / 144 /
-// 143 / 145, FP16 122 / 113 / 112 / 113.
+// 56.5 at 12, FP16 44.8 at any.  Prefetch none / 16 / 24 / 48 thousand cells
+// ahead: FP32 155 / 144 / 143 / 145, FP16 (a 16-bit row per population) 122 /
+// 113 / 112 / 113.
 constexpr int kTile = 64;
 constexpr int kTileBlkCase = 2;
 constexpr int kTilePrefetch = 160;      // 24,320 cells on 152 SMs

@@ -1,6 +1,6 @@
 // The convolutional warm start (declared in include/lbms_net.h): a 3-D U-Net
 // over the anode's voxels, trained and run with this file's kernels and the
-// tcgen05 kernels of lbms_umma.cu.  Included at the end of lbms_net.cu, whose
+// tcgen05 kernels of lbms_conv.cu.  Included at the end of lbms_net.cu, whose
 // feature builder, split-K sum, Adam and weight-cast kernels it shares.
 //
 // Layout.  Activations are channels-last BF16 rows [row][C] (C = 32, 64 or
