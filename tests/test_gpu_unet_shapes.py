@@ -115,3 +115,29 @@ def test_several_chunks_and_changing_grids(L):
     for k, (Z, Y, X) in enumerate([(24, 24, 36), (8, 12, 16), (24, 24, 36)]):
         _check(net, params, _inputs(1, Z, Y, X, 300 + k), k)
     net.close()
+
+
+@pytest.mark.parametrize("copies", [4, 32])
+def test_copies_of_a_volume(L, copies):
+    """The gradients of a batch of equal volumes are those of the volume: the
+    scale divides by a power of two, the sums are exact.  One volume has 8
+    chunks of rows at full resolution; 4 copies have 32 (three windows a CTA of
+    the weight gradients instead of one), 32 copies also at half resolution."""
+    Z, Y, X = 40, 40, 64
+    net = L.UNet(width=28, max_voxels=copies * Z * Y * X, seed=4)
+    params = _sparse_params(net.shapes(), 17)
+    net.set(params)
+    x = _inputs(1, Z, Y, X, 400)
+    y = net.forward(x)
+    rng = np.random.default_rng(5)
+    d = np.zeros(y.shape, dtype=np.float32)
+    d.reshape(-1)[rng.choice(d.size, 64, replace=False)] = rng.choice([-1.0, 1.0], 64)
+    loss = net.train_batch(x, y - d, lr=0.0)
+    one = net.get(1)
+    many_loss = net.train_batch(np.repeat(x, copies, 0), np.repeat(y - d, copies, 0), lr=0.0)
+    assert many_loss == pytest.approx(loss, rel=1e-12)
+    for i, (g, r) in enumerate(zip(net.get(1), one)):
+        assert np.abs(r).max() > 0
+        # the head's bias gradient sums FP32 values before their rounding to BF16
+        assert np.allclose(g, r, rtol=1e-6, atol=0) if i == 25 else np.array_equal(g, r), i
+    net.close()
