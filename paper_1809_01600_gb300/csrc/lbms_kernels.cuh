@@ -393,7 +393,9 @@ __device__ __forceinline__ void ms_relax(const T (&X)[3], const T (&gs)[DIM], co
 // What a collision needs of the coupling of species s: 1 / tau and the drift
 // velocity.  FP64: the quotients of ms_flux, ms_relax and 1 / tau through one
 // reciprocal of the product of their denominators (the FP64 pipe bounds the
-// FP64 steps, and a division costs it about ten operations).
+// FP64 steps, and a division costs it about ten operations).  Whatever the
+// signs, tau is clamped to the side ms_relax clamps it to; the product of five
+// denominators holds for |X| from 1e-40 (unless 0) to 1e40.
 template <typename T, int DIM>
 __device__ __forceinline__ void ms_couple(const T (&X)[3], const T (&g)[3][DIM], const T (&gs)[DIM],
                                           const MsConst<T>& c, int s, T& it, T (&v)[DIM]) {
@@ -419,19 +421,24 @@ __device__ __forceinline__ void ms_couple(const double (&X)[3], const double (&g
         den0 = (s == 0 ? X[1] * c.i12 + X[2] * c.i13
                        : (s == 1 ? X[0] * c.i12 + X[2] * c.i23 : X[0] * c.i13 + X[1] * c.i23)) +
                kMixDelta * c.h[s];
+        if (den0 < 0.0) {
+            num = -num;
+            den0 = -den0;
+        }
     }
     const double d30 = s == 2 ? X[0] * c.i13 + X[1] * c.i23 : 1.0;
     const bool det_ok = det0 > 0.0, den_ok = den0 > 0.0, d3_ok = d30 > 0.0;
     const double det = det_ok ? det0 : 1.0, den = den_ok ? den0 : 1.0, d3 = d3_ok ? d30 : 1.0;
     const double e2 = 3.0 * num + 0.5 * den;                // tau = e2 / den
+    const double e2p = e2 > 0.0 ? e2 : 1.0;                 // not needed where tau is clamped below
     const double xq = Xs * Xs + kEpsX * kEpsX;
-    const double p1 = det * den, p2 = e2 * xq, p1d = p1 * d3;
+    const double p1 = det * den, p2 = e2p * xq, p1d = p1 * d3;
     const double R = 1.0 / (p1d * p2);
     const double Rp2 = R * p2, Rp1 = R * p1d;
     const double idet = det_ok ? Rp2 * (den * d3) : 0.0;
-    const double xinv = Xs * (Rp1 * e2);
+    const double xinv = Xs * (Rp1 * e2p);
     double Dt;
-    if (!den_ok || e2 > c.tau_max * den) {
+    if ((!den_ok && !(num < 0.0)) || e2 > c.tau_max * den) {
         it = c.it_max;
         Dt = (c.tau_max - 0.5) * (1.0 / 3.0);
     } else if (e2 < c.tau_min * den) {
