@@ -53,6 +53,7 @@ struct lbms_ctx {
     std::vector<unsigned char> case_bc;  // packed CaseBC images of all cases
     bool initialized = false;         // every case has boundary data
     bool tuned = false;
+    bool dense_refused = false;       // no memory was left for L.b.dense: conversions stay on the host
     int64_t steps = 0;
     uint64_t h2d = 0, d2h = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -93,8 +94,8 @@ void* dev_alloc(lbms_ctx* c, size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (c->opt.alloc) {
         p = c->opt.alloc(bytes, c->stream, c->opt.alloc_user);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        p = nullptr;
+    } else {
+        dev_malloc(&p, bytes);
     }
     if (p) {
         c->allocs.emplace_back(p, bytes);
@@ -320,14 +321,15 @@ constexpr int64_t kDenseSpecies = 1 << 28;   // bytes up to which the three spec
 
 // Device room for the dense grid of the largest case, three species of it
 // (one beyond kDenseSpecies bytes), kept from its first use; null if the
-// handle has no coordinate words, the case is small, or no memory is left:
-// the caller then converts on the host.
+// handle has no coordinate words, the case is small, or no memory was left
+// when it was first asked for: the caller then converts on the host.
 double* dense_scratch(lbms_ctx* c, const CaseHost& cs, int& species) {
-    if (!c->L.b.cell_code || cs.N < kDenseMin) return nullptr;
+    if (!c->L.b.cell_code || cs.N < kDenseMin || c->dense_refused) return nullptr;
     int64_t n = 0;
     for (const auto& q : c->cases) n = std::max(n, q.N);
     species = n * 3 * (int64_t)sizeof(double) <= kDenseSpecies ? 3 : 1;
     if (!c->L.b.dense) c->L.b.dense = static_cast<double*>(dev_alloc(c, (size_t)species * n * sizeof(double)));
+    c->dense_refused = !c->L.b.dense;
     return c->L.b.dense;
 }
 

@@ -122,6 +122,19 @@ struct CaseHostBC {
     int tab;            // first row-table entry of the case
 };
 
+// cudaMalloc that leaves no error behind: a refused allocation is the caller's
+// to report or to do without, and must not come back from the
+// cudaGetLastError of a later launch.  *p is null then.
+template <typename T>
+inline cudaError_t dev_malloc(T** p, size_t bytes) {
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        (void)cudaGetLastError();
+    }
+    return e;
+}
+
 // First touch of freshly mapped host memory by the CPU: a device copy into
 // untouched 64 KB pages takes a fault of some 25 us for each.
 inline void touch_pages(double* p, int64_t n) {

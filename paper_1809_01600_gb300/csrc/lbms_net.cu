@@ -517,7 +517,7 @@ lbms_status nfail(lbms_net* n, lbms_status s, const char* fmt, ...) {
 template <typename T>
 T* nalloc(lbms_net* n, size_t count) {
     void* p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) p = nullptr;
+    lbms::dev_malloc(&p, std::max<size_t>(count, 1) * sizeof(T));
     n->allocs.push_back(p);
     return static_cast<T*>(p);
 }
@@ -755,11 +755,7 @@ lbms_status case_features(lbms_net* n, lbms_ctx* ctx, int k, CaseFeatures& F) {
         cudaFree(n->room);
         n->room = nullptr;
         n->room_bytes = 0;
-        if (cudaMalloc(&n->room, need) != cudaSuccess) {
-            n->room = nullptr;
-            cudaGetLastError();
-            return nfail(n, LBMS_ENOMEM, "feature buffers");
-        }
+        if (lbms::dev_malloc(&n->room, need) != cudaSuccess) return nfail(n, LBMS_ENOMEM, "feature buffers");
         n->room_bytes = need;
     }
     lay_out(n->room);
@@ -827,8 +823,8 @@ lbms_status grow(lbms_net* n, int64_t need) {
     int64_t cap = std::max<int64_t>(need, 2 * n->cap);
     bf16* f = nullptr;
     float* t = nullptr;
-    NCK(cudaMalloc(&f, (size_t)cap * kF * sizeof(bf16)), "training rows");
-    if (cudaMalloc(&t, (size_t)cap * 4 * sizeof(float)) != cudaSuccess) {
+    NCK(lbms::dev_malloc(&f, (size_t)cap * kF * sizeof(bf16)), "training rows");
+    if (lbms::dev_malloc(&t, (size_t)cap * 4 * sizeof(float)) != cudaSuccess) {
         cudaFree(f);
         return nfail(n, LBMS_ENOMEM, "training targets");
     }

@@ -356,7 +356,7 @@ lbms_status ufail(lbms_unet* u, lbms_status s, const char* fmt, ...) {
 template <typename T>
 T* ualloc(lbms_unet* u, size_t count) {
     void* p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) p = nullptr;
+    lbms::dev_malloc(&p, std::max<size_t>(count, 1) * sizeof(T));
     u->allocs.push_back(p);
     return static_cast<T*>(p);
 }
@@ -433,7 +433,7 @@ lbms_status ensure_buffers(lbms_unet* u, const Levels& v) {
     bool ok = true;
     auto get = [&](size_t bytes) {
         void* p = nullptr;
-        if (ok && cudaMalloc(&p, std::max<size_t>(bytes, 16)) == cudaSuccess) {
+        if (ok && lbms::dev_malloc(&p, std::max<size_t>(bytes, 16)) == cudaSuccess) {
             u->bufs.push_back(p);
             ok = cudaMemset(p, 0, std::max<size_t>(bytes, 16)) == cudaSuccess;
         } else {
@@ -954,8 +954,8 @@ lbms_status lbms_unet_add_sample(lbms_unet* u, lbms_ctx* ctx, int k) {
     s.rows = R;
     s.nfluid = v.nf;
     int64_t* prow = F.row;
-    if (cudaMalloc(&s.in, (size_t)R * kUInC * sizeof(bf16)) != cudaSuccess) return ufail(u, LBMS_ENOMEM, "sample");
-    if (cudaMalloc(&s.tg, (size_t)R * 4 * sizeof(float)) != cudaSuccess) {
+    if (lbms::dev_malloc(&s.in, (size_t)R * kUInC * sizeof(bf16)) != cudaSuccess) return ufail(u, LBMS_ENOMEM, "sample");
+    if (lbms::dev_malloc(&s.tg, (size_t)R * 4 * sizeof(float)) != cudaSuccess) {
         cudaFree(s.in);
         return ufail(u, LBMS_ENOMEM, "sample");
     }
@@ -994,9 +994,9 @@ lbms_status lbms_unet_add_volume(lbms_unet* u, const float* x, const float* t, i
     s.nfluid = (int64_t)std::llround(nf);
     float* dev = nullptr;
     const size_t nin = (size_t)g.V * kUInReal, ntg = (size_t)g.V * 3;
-    if (cudaMalloc(&dev, (nin + ntg) * sizeof(float)) != cudaSuccess) return ufail(u, LBMS_ENOMEM, "volume upload");
-    cudaError_t e = cudaMalloc(&s.in, (size_t)g.R * kUInC * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc(&s.tg, (size_t)g.R * 4 * sizeof(float));
+    if (lbms::dev_malloc(&dev, (nin + ntg) * sizeof(float)) != cudaSuccess) return ufail(u, LBMS_ENOMEM, "volume upload");
+    cudaError_t e = lbms::dev_malloc(&s.in, (size_t)g.R * kUInC * sizeof(bf16));
+    if (e == cudaSuccess) e = lbms::dev_malloc(&s.tg, (size_t)g.R * 4 * sizeof(float));
     if (e == cudaSuccess) e = cudaMemcpy(dev, x, nin * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dev + nin, t, ntg * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(s.in, 0, (size_t)g.R * kUInC * sizeof(bf16));
@@ -1134,7 +1134,7 @@ lbms_status upload_batch(lbms_unet* u, const float* x, const float* t, int B, in
     if (nfluid) *nfluid = nf;
     float* dev = nullptr;
     const size_t nin = (size_t)V * kUInReal, ntg = t ? (size_t)V * 3 : 0;
-    UCK(cudaMalloc(&dev, (nin + ntg) * sizeof(float)), "batch upload");
+    UCK(lbms::dev_malloc(&dev, (nin + ntg) * sizeof(float)), "batch upload");
     lbms_status st = LBMS_OK;
     cudaError_t e = cudaMemcpy(dev, x, nin * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && t) e = cudaMemcpy(dev + nin, t, ntg * sizeof(float), cudaMemcpyHostToDevice);
