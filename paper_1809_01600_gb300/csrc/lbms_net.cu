@@ -1135,7 +1135,15 @@ lbms_status lbms_net_warm_start(lbms_net* n, lbms_ctx* ctx, int k, double* Xout)
         predict_post_kernel<<<(rows + 255) / 256, 256>>>(n->Y, n->y_ld, F.cell, j0, rows, v.nf, v.nx, F.xtab, F.pred);
         NCK(cudaGetLastError(), "prediction");
     }
+    st = check_gemm(n);   // before the handle's state is replaced
+    if (st != LBMS_OK) return st;
     return take_prediction(n, ctx, k, F, Xout);
+}
+
+// For tests: leaves the network as a product whose wait ran out does.
+int lbms_internal_net_timeout(lbms_net* n) {
+    const unsigned int f = 1u;
+    return cudaMemcpy(n->gemm_err, &f, sizeof(f), cudaMemcpyHostToDevice);
 }
 
 }  // extern "C"
