@@ -73,6 +73,15 @@ __device__ __forceinline__ float column_sum(float (&v)[32], int lane) {
     return v[0];
 }
 
+// After a wait that ran out, once no warp of the CTA issues any more: the
+// copies into the last stages land (or are waited for as long as any) before
+// the CTA gives its shared memory back.  `issued` stages of the ring of ST in
+// all; `once`: a barrier of copies issued once, or null.
+__device__ __noinline__ void drain_copies(uint64_t* full, int ST, int issued, uint64_t* once) {
+    for (int i = max(0, issued - ST); i < issued; ++i) mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u);
+    if (once) mbar_wait(once, 0);
+}
+
 // ---------------------------------------------------------------------------
 // Convolution and plain product.  RB: bytes of an operand row in shared
 // memory (64: 32 channels, 128: 64 channels; nblk such blocks make up C).
@@ -161,13 +170,14 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const __grid_cons
     // instruction itself, so that descriptors and addresses stay in uniform
     // registers: issued from a single lane's branch an MMA took 150 cycles.
     const bool back = NT == 3 && job.off[2] < job.off[0];
+    int it = 0;      // stages whose loads are issued (warp 0)
     if (warp == 0) {
         const bool leader = elect_one();
         if (Sh::kResident && leader) {
             mbar_expect_tx(res_full, 27 * Sh::kBTile);
             for (int t = 0; t < 27; ++t) tma_load_2d(resB + t * Sh::kBTile, &mapB, t * (RB / 2), 0, res_full);
         }
-        int it = 0, s = 0;
+        int s = 0;
         uint32_t ph = 1u;
         bool ok = true;
         for (int tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
@@ -201,10 +211,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const __grid_cons
         if (!ok && lane == 0) {
             *failed = 1;
             atomicOr(err, 1u);
-        }
-        if (!ok || *failed) {   // copies still in flight land before the CTA exits
-            for (int i = max(0, it - ST); i < it; ++i) mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u);
-            if (Sh::kResident) mbar_wait(res_full, 0);
         }
     } else if (warp == 1) {
         const bool leader = elect_one();
@@ -451,7 +457,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv_kernel(const __grid_cons
         }
         if constexpr (KIND == kOutHead) {
             if (ep.T) {
-double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
+                double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -471,7 +477,10 @@ double sum[4] = {loss * ep.loss_scale, hs[0], hs[1], hs[2]};
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, Sh::kCols);
+    if (warp == 0) {
+        if (*failed) drain_copies(full, ST, it, Sh::kResident ? res_full : nullptr);
+        tmem_dealloc(tmem, Sh::kCols);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -537,9 +546,10 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    int it = 0;      // stages whose loads are issued (warp 0)
     if (warp == 0) {
         const bool leader = elect_one();
-        int it = 0, s = 0;
+        int s = 0;
         uint32_t ph = 1u;
         bool ok = true;
         for (; it < nk; ++it) {
@@ -566,8 +576,6 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
             *failed = 1;
             atomicOr(err, 8u);
         }
-        if (!ok || *failed)
-            for (int i = max(0, it - ST); i < it; ++i) mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u);
     } else if (warp == 1) {
         const bool leader = elect_one();
         int s = 0;
@@ -634,7 +642,10 @@ __global__ void __launch_bounds__(192, 1) wgrad_kernel(const __grid_constant__ C
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, Sh::kCols);
+    if (warp == 0) {
+        if (*failed) drain_copies(full, ST, it, nullptr);
+        tmem_dealloc(tmem, Sh::kCols);
+    }
 }
 
 // The weight gradient of a 3x3x3 convolution with at most 64 channels on
@@ -698,9 +709,10 @@ __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ 
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    int it = 0;      // stages whose loads are issued (warp 0)
     if (warp == 0) {
         const bool leader = elect_one();
-        int it = 0, s = 0;
+        int s = 0;
         uint32_t ph = 1u;
         bool ok = true;
         for (; it < nk; ++it) {
@@ -725,8 +737,6 @@ __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ 
             *failed = 1;
             atomicOr(err, 8u);
         }
-        if (!ok || *failed)
-            for (int i = max(0, it - ST); i < it; ++i) mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u);
     } else if (warp == 1) {
         const bool leader = elect_one();
         int s = 0;
@@ -789,7 +799,10 @@ __global__ void __launch_bounds__(192, 1) wgrad3_kernel(const __grid_constant__ 
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, Sh::kCols);
+    if (warp == 0) {
+        if (*failed) drain_copies(full, ST, it, nullptr);
+        tmem_dealloc(tmem, Sh::kCols);
+    }
 }
 
 // ------------------------------------------------------------------ launch
