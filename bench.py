@@ -235,10 +235,13 @@ def variant_key(info):
     return f"{info.tile_cells}x{info.tile_min_blocks}/t{info.threads_per_cell}/nb{info.neighbour_bits}"
 
 
-def step_kernel_name(forced_variant, threads_per_cell):
+def step_kernel_name(forced_variant, info):
+    """The step kernel of a handle with the default outlet and gradient options."""
     if forced_variant:
-        return "step_kernel_cell" if threads_per_cell == 1 else "step_kernel"
-    return "step_tile_kernel" if threads_per_cell == 1 else "step_small_kernel"
+        return "step_kernel_cell" if info.threads_per_cell == 1 else "step_kernel"
+    if info.threads_per_cell == 1:
+        return "step_tile_kernel"
+    return "step_small_kernel" if info.tile_cells == 32 else "block_steps_kernel"
 
 
 def ncu_traffic(workload, precision, variant):
@@ -548,7 +551,7 @@ def main():
                 "peak_source": peak_kind, "bytes_per_fluid_cell": bpc, "variant": variant_key(tinfo),
                 "algorithmic_bytes_per_launch": nf * bpc,
                 "kernel": "%s<%s, X %s, h %s>" % (
-                    step_kernel_name(args.step_variant, tinfo.threads_per_cell),
+                    step_kernel_name(args.step_variant, tinfo),
                     "D3Q19" if case.dim == 3 else "D2Q9",
                     "double" if args.precision == "fp64" else "float pair",
                     {"fp64": "double", "fp32": "float", "fp16": "__half"}[args.precision])}
@@ -612,7 +615,8 @@ def main():
                                    f"{'one thread per cell' if tinfo.threads_per_cell == 1 else 'one thread per cell and species'}, "
                                    f"{tinfo.tile_min_blocks} blocks/SM, " + (
                                        "neighbours decoded from per-row fluid bitmasks" if tinfo.neighbour_bits == 1
-                                       else f"{tinfo.neighbour_bits}-bit neighbour table") + " (autotuned)",
+                                       else f"{tinfo.neighbour_bits}-bit neighbour table") + (
+                                       " (forced)" if args.step_variant else " (by size)"),
                            "l2": "state larger than L2 (no flush needed)" if nf * bpc > 129e6 * 2
                            else "state fits in L2"},
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk,

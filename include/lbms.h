@@ -183,7 +183,7 @@ typedef struct {
     uint64_t h2d_bytes;         /* host-to-device bytes copied so far */
     uint64_t d2h_bytes;         /* device-to-host bytes copied so far */
     int n_cases;                /* cases in the handle (1 unless made by lbms_create_batch) */
-    int tile_cells;             /* step-kernel tile picked by the autotuner: cells per block */
+    int tile_cells;             /* the step kernel chosen by size or by the autotuner: cells per block */
     int tile_min_blocks;        /*   and its register budget (resident blocks per SM) */
     int neighbour_bits;         /*   and its neighbour lookup: 32 (indices), 16 (offsets) or 1 (row bitmasks) */
     int threads_per_cell;       /*   and its thread mapping: 3 (one per species) or 1 */

@@ -1490,6 +1490,13 @@ lbms_status lbms_get_info(const lbms_ctx* c, lbms_info* info) {
         info->threads_per_cell = 1;
         return LBMS_OK;
     }
+    if (c->L.small) {   // a block per case reads its links once a launch, from the 32-bit table
+        info->tile_cells = kSmallCells[c->L.small];
+        info->tile_min_blocks = kSmallMinBlocks[c->L.small];
+        info->neighbour_bits = c->L.small == kSmall && c->L.b.rowtab ? 1 : 32;
+        info->threads_per_cell = 3;
+        return LBMS_OK;
+    }
     info->tile_cells = kVariantCells[c->L.variant];
     info->tile_min_blocks = kVariantMinBlocks[c->L.variant];
     info->neighbour_bits = kVariantNb[c->L.variant] == kNbOffset16 ? 16 : (kVariantNb[c->L.variant] == kNbRowMask ? 1 : 32);

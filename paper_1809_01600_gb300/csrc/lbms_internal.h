@@ -51,6 +51,8 @@ constexpr int kTileMinCells = 38913;
 // Steps of handles that do not fill the GPU (lbms_step_small.cuh): many steps
 // of a block per case of at most 64, 128 or 320 cells, or a launch a step.
 enum { kNotSmall = 0, kBlock64, kBlock128, kBlock320, kSmall };
+constexpr int kSmallCells[] = {0, 64, 128, 320, 32};        // cells per block of each
+constexpr int kSmallMinBlocks[] = {0, 1, 1, 1, 4};          // and blocks per SM its registers are budgeted for
 constexpr int kBlockSteps = 65536;   // steps of one launch at most
 
 // Limits of the per-cell coordinate word of kNbRowMask (x | y << 11 | z << 21).
@@ -64,7 +66,7 @@ struct DevBuffers {
     int16_t* nbr16 = nullptr;          // [S][nb16_width] offsets, when they all fit (else null)
     uint32_t* cell_code = nullptr;     // [S] x | y << 11 | z << 21 of each fluid cell (kNbRowMask; else null)
     uint4* rowtab = nullptr;           // per case [rows][words]: 64-bit fluid window + index (kNbRowMask); with
-                                       // Launch::tiled uint2 windows of 32 voxels (lbms_step_tile.cuh)
+                                       // Launch::windows16 uint2 windows of 32 voxels (lbms_step_tile.cuh)
     int* rows = nullptr;               // [3][total rows]: x = 0, x = 1, x = nx-1 cell of each row (-1 if solid)
     int2* case_rows = nullptr;         // [cases]: first row, row count
     void* cases = nullptr;             // [cases] CaseBC<XS> (inlet values, outlet flux, range)

@@ -39,7 +39,7 @@ cudaError_t block_w(const Launch& L, int n, cudaStream_t st) {
 
 template <class Lat, typename XS, typename P>
 cudaError_t small_t(const Launch& L, cudaStream_t st) {
-    constexpr int W = 32;
+    constexpr int W = kSmallCells[kSmall];
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(L.ncells / W));
     cfg.blockDim = dim3(3 * W);
@@ -55,9 +55,9 @@ cudaError_t small_t(const Launch& L, cudaStream_t st) {
 template <class Lat, typename XS, typename P>
 cudaError_t block_t(const Launch& L, int n, cudaStream_t st) {
     switch (L.small) {
-        case kBlock64: return block_w<Lat, XS, P, 64>(L, n, st);
-        case kBlock128: return block_w<Lat, XS, P, 128>(L, n, st);
-        case kBlock320: return block_w<Lat, XS, P, 320>(L, n, st);
+        case kBlock64: return block_w<Lat, XS, P, kSmallCells[kBlock64]>(L, n, st);
+        case kBlock128: return block_w<Lat, XS, P, kSmallCells[kBlock128]>(L, n, st);
+        case kBlock320: return block_w<Lat, XS, P, kSmallCells[kBlock320]>(L, n, st);
         default: return cudaErrorInvalidValue;
     }
 }

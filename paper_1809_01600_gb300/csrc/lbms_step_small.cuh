@@ -267,7 +267,7 @@ __device__ __forceinline__ void share_table(const int* __restrict__ nbr, int i, 
 // FP64 12.0 / 9.8; 3-D 4.8 k FP32 2.9 / 2.6, 26 k FP32 4.6 / 3.9, FP16 4.7 / 3.9,
 // FP64 47 / 41, 37 k FP32 4.7 / 4.0.
 template <class L, typename XS, typename P, int W>
-__global__ void __launch_bounds__(3 * W, 4) step_small_kernel(const SmallParams<XS, P> p) {
+__global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_kernel(const SmallParams<XS, P> p) {
     using T = typename Xv<XS>::T;
     using XV = Xv<XS>;
     constexpr int Q = L::Q;

@@ -1,0 +1,50 @@
+"""lbms_get_info names the step that a handle takes: cells per block, blocks
+per SM, neighbour lookup and threads per cell, on both sides of the sizes
+between which the step changes."""
+import pytest
+
+from test_gpu_step_small import _box
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1809_01600_gb300 import lbms
+    lbms.load()
+    return lbms
+
+
+def _info(L, cs, precision, **kw):
+    b = L.Batch.from_cases(cs, precision=precision, **kw)
+    for k, c in enumerate(cs):                 # a forced variant takes effect with the boundary data
+        b.set_bc(c.x_in, 0.0 if c.periodic_x else c.current_A_cm2, case=k)
+    i = b.info()
+    b.close()
+    return i.tile_cells, i.tile_min_blocks, i.neighbour_bits, i.threads_per_cell
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+@pytest.mark.parametrize("fluid,want", [(64, (64, 1, 32, 3)), (65, (128, 1, 32, 3)), (128, (128, 1, 32, 3)),
+                                        (129, (320, 1, 32, 3)), (320, (320, 1, 32, 3)), (321, (32, 4, 1, 3))])
+def test_small_handles(L, precision, fluid, want):
+    assert _info(L, [_box(2, fluid)], precision) == want
+
+
+def test_periodic_boxes_read_the_table(L):
+    assert _info(L, [_box(2, 700, periodic=True)], "fp32") == (32, 4, 32, 3)
+    assert _info(L, [_box(2, 700), _box(2, 700, periodic=True)], "fp32") == (32, 4, 32, 3)
+
+
+@pytest.mark.parametrize("precision,blocks", [("fp32", 10), ("fp16", 10)])
+def test_around_the_tiled_step(L, precision, blocks):
+    assert _info(L, [_box(3, 38912)], precision) == (32, 4, 1, 3)
+    assert _info(L, [_box(3, 38913)], precision) == (64, blocks, 1, 1)
+
+
+def test_forced_variants(L):
+    assert _info(L, [_box(2, 64)], "fp32", step_variant=1) == (32, 8, 32, 3)
+    assert _info(L, [_box(2, 64)], "fp32", step_variant=9) == (64, 8, 1, 1)
