@@ -159,7 +159,7 @@ cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream
 size_t tile_cell_bytes(int dim, int precision);
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 // the step for a handle whose largest case has max_nf cells, or kNotSmall;
-// L.ncells and sm_count are set
+// L.ncells, n_cases and sm_count are set
 int choose_small(const Launch& L, int max_nf);
 cudaError_t launch_step_small(const Launch& L, cudaStream_t st);
 // n <= kBlockSteps steps of a kBlock* handle; cur turns n & 1 times

@@ -57,17 +57,43 @@ cudaError_t block_t(const Launch& L, int n, cudaStream_t st) {
     switch (L.small) {
         case kBlock64: return block_w<Lat, XS, P, kSmallCells[kBlock64]>(L, n, st);
         case kBlock128: return block_w<Lat, XS, P, kSmallCells[kBlock128]>(L, n, st);
-        case kBlock320: return block_w<Lat, XS, P, kSmallCells[kBlock320]>(L, n, st);
+        case kBlock320:
+            if constexpr (sizeof(XS) == 8) return cudaErrorInvalidValue;   // not chosen
+            else return block_w<Lat, XS, P, kSmallCells[kBlock320]>(L, n, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
+namespace {
+
+// Whether a block per case is the faster step of small cases.  FP32 and FP16:
+// a step is latency, so it is, but for 3-D cases of more than 128 cells while
+// they leave most SMs idle (us per step of 1 / 15 / 30 / 45 / 60 cases of 300
+// cells, block 3.0 at any, launches 2.2 / 2.4 / 2.8 / 3.1 / 3.3; FP16 3.2
+// and 2.1 / 2.4 / 2.8 / 3.0 / 3.3).  FP64: the pipe of the fullest SM is the step,
+// and a block puts a whole case on one (2-D, 1 case of 64, 120, 300 cells: 8.5,
+// 16.7, 41.5 us, launches 6.7 at any), so it must not give that SM more warps
+// than the launches would (80 cases of 64: 8.5, launches 9.9; 152 of 120: 16.7
+// and 22); with 320 cells its registers spill and it was ahead nowhere.
+bool block_pays(const Launch& L, int block) {
+    if (L.precision != 0) return block != kBlock320 || L.dim == 2 || 8 * L.n_cases >= 3 * L.sm_count;
+    if (block == kBlock320) return false;
+    const int warps = 3 * kSmallCells[block] / 32, resident = block == kBlock64 ? 2 : 1;
+    const int64_t a = L.sm_count, n = L.n_cases;
+    const int64_t of_blocks = n <= a ? warps : (n + resident * a - 1) / (resident * a) * resident * warps;
+    return of_blocks <= 3 * ((L.ncells / kSmallCells[kSmall] + a - 1) / a);
+}
+
+}  // namespace
+
 int choose_small(const Launch& L, int max_nf) {
-    if (max_nf <= 64) return kBlock64;
-    if (max_nf <= 128) return kBlock128;
-    if (max_nf <= 320) return kBlock320;
+    for (int block : {kBlock64, kBlock128, kBlock320})
+        if (max_nf <= kSmallCells[block]) {
+            if (block_pays(L, block)) return block;
+            break;
+        }
     return L.ncells < kTileMinCells ? kSmall : kNotSmall;
 }
 

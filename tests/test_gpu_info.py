@@ -48,3 +48,18 @@ def test_around_the_tiled_step(L, precision, blocks):
 def test_forced_variants(L):
     assert _info(L, [_box(2, 64)], "fp32", step_variant=1) == (32, 8, 32, 3)
     assert _info(L, [_box(2, 64)], "fp32", step_variant=9) == (64, 8, 1, 1)
+
+
+# a block per case while it gives no SM more FP64 warps than the launches do,
+# and in 3-D FP32 / FP16 from 128 cells on only with enough cases
+@pytest.mark.parametrize("dim,precision,fluid,cases_,want", [
+    (2, "fp64", 64, 1, 32), (2, "fp64", 64, 76, 32), (2, "fp64", 64, 77, 64), (3, "fp64", 60, 152, 64),
+    (3, "fp64", 60, 153, 32), (2, "fp64", 60, 229, 64), (2, "fp64", 60, 320, 32), (2, "fp64", 128, 114, 32),
+    (2, "fp64", 128, 115, 128), (3, "fp64", 120, 153, 32), (2, "fp64", 300, 1, 32), (3, "fp64", 300, 100, 32),
+    (3, "fp32", 128, 1, 128), (3, "fp32", 129, 1, 32), (3, "fp32", 300, 56, 32), (3, "fp32", 300, 57, 320),
+    (3, "fp16", 300, 56, 32), (3, "fp16", 300, 57, 320), (2, "fp32", 300, 1, 320), (2, "fp16", 320, 300, 320)])
+def test_a_block_per_case_where_it_pays(L, dim, precision, fluid, cases_, want):
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the counts are for 152 SMs")
+    assert _info(L, [_box(dim, fluid)] * cases_, precision)[0] == want
