@@ -421,16 +421,16 @@ __device__ __forceinline__ void ms_couple(const double (&X)[3], const double (&g
         den0 = (s == 0 ? X[1] * c.i12 + X[2] * c.i13
                        : (s == 1 ? X[0] * c.i12 + X[2] * c.i23 : X[0] * c.i13 + X[1] * c.i23)) +
                kMixDelta * c.h[s];
-        if (den0 < 0.0) {
-            num = -num;
-            den0 = -den0;
-        }
+        // both signs turned over where den0 < 0 (bits: a comparison takes the FP64 pipe)
+        const int sign = __double2hiint(den0) & (int)0x80000000;
+        num = __hiloint2double(__double2hiint(num) ^ sign, __double2loint(num));
+        den0 = fabs(den0);
     }
     const double d30 = s == 2 ? X[0] * c.i13 + X[1] * c.i23 : 1.0;
     const bool det_ok = det0 > 0.0, den_ok = den0 > 0.0, d3_ok = d30 > 0.0;
     const double det = det_ok ? det0 : 1.0, den = den_ok ? den0 : 1.0, d3 = d3_ok ? d30 : 1.0;
     const double e2 = 3.0 * num + 0.5 * den;                // tau = e2 / den
-    const double e2p = e2 > 0.0 ? e2 : 1.0;                 // not needed where tau is clamped below
+    const double e2p = __double2hiint(e2) > 0 ? e2 : 1.0;                // not needed where tau is clamped below
     const double xq = Xs * Xs + kEpsX * kEpsX;
     const double p1 = det * den, p2 = e2p * xq, p1d = p1 * d3;
     const double R = 1.0 / (p1d * p2);
@@ -438,7 +438,7 @@ __device__ __forceinline__ void ms_couple(const double (&X)[3], const double (&g
     const double idet = det_ok ? Rp2 * (den * d3) : 0.0;
     const double xinv = Xs * (Rp1 * e2p);
     double Dt;
-    if ((!den_ok && !(num < 0.0)) || e2 > c.tau_max * den) {
+    if ((!den_ok && __double2hiint(num) >= 0) || e2 > c.tau_max * den) {
         it = c.it_max;
         Dt = (c.tau_max - 0.5) * (1.0 / 3.0);
     } else if (e2 < c.tau_min * den) {
