@@ -6,6 +6,27 @@
 namespace lbms {
 namespace {
 
+// How the launches of step_small_kernel overlap.  Blocks of the next step are
+// placed wherever there is room, so where there is room beside some blocks of
+// this step and not beside others they pile up on few SMs.
+//  FP64, whose step is the pipe of the fullest SM: 2-D (6 blocks of an SM
+// resident) with 3 to 5 blocks an SM, 3-D (5 resident) with 2.5 to 4 took 18.4 ->
+// 24.2 us (16.8 k cells) and 24.0 -> 33.2 us (13.4 k cells) a step with
+// overlapped launches.  Below, two steps fit side by side, above, next to
+// nothing of the next one does: there overlapping gains 0.9 us.
+//  FP32 and FP16, whose step is latency: ahead at any size by 0.4 to 0.6 us;
+// in 2-D up to two blocks an SM the next step may be placed as early as can be
+// (8.3 k cells 2.37 -> 2.00 us; beyond, 18 k cells 2.65 -> 2.83).
+struct Overlap {
+    bool on, early;
+};
+Overlap small_overlap(const Launch& L) {
+    const int64_t blocks = L.ncells / kSmallCells[kSmall], sms = L.sm_count;
+    if (L.precision != 0) return {true, L.dim == 2 && blocks <= 2 * sms};
+    const int resident = L.dim == 2 ? 6 : 5;
+    return {2 * blocks <= resident * sms || blocks > (resident - 1) * sms, false};
+}
+
 template <class Lat, typename XS, typename P>
 SmallParams<XS, P> params(const Launch& L, int n) {
     SmallParams<XS, P> p;
@@ -15,6 +36,7 @@ SmallParams<XS, P> params(const Launch& L, int n) {
     }
     p.cur = L.cur;
     p.n = n;
+    p.early = small_overlap(L).early;
     p.nbr32 = L.b.nbr;
     p.cell_code = L.b.cell_code;
     p.rowtab = reinterpret_cast<const uint2*>(L.b.rowtab);
@@ -48,7 +70,7 @@ cudaError_t small_t(const Launch& L, cudaStream_t st) {
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = small_overlap(L).on ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, step_small_kernel<Lat, XS, P, W>, params<Lat, XS, P>(L, 1));
 }
 

@@ -2,8 +2,22 @@
 #include "lbms_step_launch.cuh"
 #include "lbms_step_tile.cuh"
 
+#include <algorithm>
+
 namespace lbms {
 namespace {
+
+// Whether consecutive launches overlap (programmatic dependent launch).  Blocks
+// of the next step are placed wherever there is room; while this step leaves
+// room on some SMs and not on others, they pile up there and the next step runs
+// unevenly.  us per step without and with: 3-D FP32 41 k cells 5.5 and 6.9, 67 k
+// 6.5 and 7.5, 79 k 7.52 and 7.53, 91 k 7.9 and 7.5; FP16 67 k 5.9 and 6.6, 79 k
+// 7.0 and 6.6; 2-D FP32 60 k 4.0 and 4.4, 90 k 4.6 and 4.6, FP64 43 k 42.9 and 63.8,
+// 67 k 60.0 and 65.3; 3-D FP64 (5 blocks an SM resident) 41 k 69.6 and 79.5, 49 k
+// 80.0 and 79.8.  So from 8 blocks an SM on, or as many as are resident.
+bool tile_overlaps(const Launch& L) {
+    return L.ncells >= (int64_t)std::min(8, tile_min_blocks(L.dim, L.precision)) * kTile * L.sm_count;
+}
 
 template <class Lat, typename XS, typename P, typename NBT>
 cudaError_t tile_w(const Launch& L, cudaStream_t st) {
@@ -30,7 +44,7 @@ cudaError_t tile_w(const Launch& L, cudaStream_t st) {
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = tile_overlaps(L) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, step_tile_kernel<Lat, XS, P, NBT, kTile, MB>, p);
 }
 

@@ -8,7 +8,9 @@
 //    dependent launch).  The three threads of a cell split its source rows
 //    (row windows: 9 rows of D3Q19 as 3 + 2 + 4, 6 links each) or its row of
 //    the 32-bit table and leave the links in shared memory, before the wait for
-//    the preceding step: no step writes those tables.
+//    the preceding step: no step writes those tables.  When the next step may
+//    be placed, and where launches overlap at all: small_overlap
+//    (lbms_launch_small.cu).
 // Keeping all blocks resident with a grid-wide barrier, or with flags between
 // the blocks that exchange, was no faster than overlapped launches where FP32
 // is the arithmetic: 26 k cells took 4.3 and 5.0 us per step.
@@ -28,6 +30,7 @@ struct SmallParams {
     XS* x[2];
     int cur;                            // lattice holding the state
     int n;                              // steps (block_steps_kernel)
+    bool early;                         // the next step may be placed from the start (step_small_kernel)
     const int* nbr32;
     const uint32_t* cell_code;
     const uint2* rowtab;                // windows of the tiled step, or null: nbr32
@@ -276,6 +279,7 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
     __shared__ int sF[W];
     __shared__ T sXv[3][W];
     __shared__ T sG[3][DIM][W];
+    if (p.early) grid_launch_next();
     const int s = threadIdx.x / W;
     const int c = threadIdx.x - s * W;
     const int i = blockIdx.x * W + c;    // the cells of all cases are a multiple of 64
@@ -332,9 +336,10 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
 #pragma unroll
         for (int a = 0; a < DIM; ++a) gall[r][a] = sG[r][a][c];
     }
-    // Not earlier: blocks of the next step placed while these have just begun
-    // crowd onto the SMs they find, and the FP64 pipe of a crowded SM is the
-    // whole step (9.3 k cells 2-D FP64: 9.8 us here, 23.5 from the start).
+    // Unless small_overlap says so, not earlier: blocks of the next step placed
+    // while these have just begun crowd onto the SMs they find, and the FP64
+    // pipe of a crowded SM is the whole step (9.3 k cells 2-D FP64: 9.8 us
+    // here, 23.5 from the start).
     grid_launch_next();
     P q[Q];
     collide<L, XS, P>(p.c, s, X, gall, g, dX, d, q);
