@@ -9,22 +9,26 @@ namespace {
 // How the launches of step_small_kernel overlap.  Blocks of the next step are
 // placed wherever there is room, so where there is room beside some blocks of
 // this step and not beside others they pile up on few SMs.
-//  FP64, whose step is the pipe of the fullest SM: 2-D (6 blocks of an SM
-// resident) with 3 to 5 blocks an SM, 3-D (5 resident) with 2.5 to 4 took 18.4 ->
-// 24.2 us (16.8 k cells) and 24.0 -> 33.2 us (13.4 k cells) a step with
-// overlapped launches.  Below, two steps fit side by side, above, next to
-// nothing of the next one does: there overlapping gains 0.9 us.
-//  FP32 and FP16, whose step is latency: ahead at any size by 0.4 to 0.6 us;
-// in 2-D up to two blocks an SM the next step may be placed as early as can be
-// (8.3 k cells 2.37 -> 2.00 us; beyond, 18 k cells 2.65 -> 2.83).
+//  Two steps fit side by side (twice the blocks are resident): the next one is
+// let in as soon as the wait of this one is over, not before, when a third and a
+// fourth would come too.  us per step, let in after the gathers / after the
+// wait / from the start: 2-D FP32 8.3 k cells 2.42 / 1.92 / 2.03, 18 k 2.65 / 2.2 /
+// 2.8, 27 k 2.75 / 2.50 / 2.93; beyond, 30 k, 2.81 / 3.33 / 3.33; 3-D FP32 9.7 k 2.89 /
+// 2.50 / 2.85, 19 k 3.37 / 2.94 / 3.36, 23.5 k (beyond) 3.63 / 3.91 / 3.91.
+//  Else after the gathers, but in FP64, whose step is the pipe of the fullest
+// SM, only where next to nothing of the next step finds room: with 3 to 5 blocks
+// an SM in 2-D (6 resident) and 2.5 to 4 in 3-D (5 resident) overlapped launches
+// took 24.2 us (16.8 k cells) and 33.2 us (13.4 k), ordinary ones 18.4 and 24.0;
+// with more they gain 0.9 us.
 struct Overlap {
-    bool on, early;
+    bool on, side;
 };
 Overlap small_overlap(const Launch& L) {
     const int64_t blocks = L.ncells / kSmallCells[kSmall], sms = L.sm_count;
-    if (L.precision != 0) return {true, L.dim == 2 && blocks <= 2 * sms};
-    const int resident = L.dim == 2 ? 6 : 5;
-    return {2 * blocks <= resident * sms || blocks > (resident - 1) * sms, false};
+    // by the registers of the kernels: 96 / 126 (FP64), 56 / 80
+    const int resident = L.precision == 0 ? (L.dim == 2 ? 6 : 5) : (L.dim == 2 ? 12 : 8);
+    const bool side = 2 * blocks <= resident * sms;
+    return {L.precision != 0 || side || blocks > (resident - 1) * sms, side};
 }
 
 template <class Lat, typename XS, typename P>
@@ -36,7 +40,7 @@ SmallParams<XS, P> params(const Launch& L, int n) {
     }
     p.cur = L.cur;
     p.n = n;
-    p.early = small_overlap(L).early;
+    p.side = small_overlap(L).side;
     p.nbr32 = L.b.nbr;
     p.cell_code = L.b.cell_code;
     p.rowtab = reinterpret_cast<const uint2*>(L.b.rowtab);

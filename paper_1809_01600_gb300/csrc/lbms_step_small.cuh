@@ -30,7 +30,7 @@ struct SmallParams {
     XS* x[2];
     int cur;                            // lattice holding the state
     int n;                              // steps (block_steps_kernel)
-    bool early;                         // the next step may be placed from the start (step_small_kernel)
+    bool side;                          // the next step fits beside this one (step_small_kernel)
     const int* nbr32;
     const uint32_t* cell_code;
     const uint2* rowtab;                // windows of the tiled step, or null: nbr32
@@ -279,7 +279,6 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
     __shared__ int sF[W];
     __shared__ T sXv[3][W];
     __shared__ T sG[3][DIM][W];
-    if (p.early) grid_launch_next();
     const int s = threadIdx.x / W;
     const int c = threadIdx.x - s * W;
     const int i = blockIdx.x * W + c;    // the cells of all cases are a multiple of 64
@@ -304,6 +303,7 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
             share_table<L, 2, W>(p.nbr32, i, S32, c, sN, sF);
     }
     grid_wait();
+    if (p.side) grid_launch_next();
     const P* hs = p.h[p.cur] + (int64_t)s * Q * S;
     const XS* xh = p.x[p.cur] + s * S;
     XV xo = XV::own_rows(xh, p.x[p.cur] + (3 + s) * S, i);
@@ -336,10 +336,8 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
 #pragma unroll
         for (int a = 0; a < DIM; ++a) gall[r][a] = sG[r][a][c];
     }
-    // Unless small_overlap says so, not earlier: blocks of the next step placed
-    // while these have just begun crowd onto the SMs they find, and the FP64
-    // pipe of a crowded SM is the whole step (9.3 k cells 2-D FP64: 9.8 us
-    // here, 23.5 from the start).
+    // Unless two steps fit side by side, not earlier: blocks of the next step
+    // placed while these have just begun crowd onto the SMs they find.
     grid_launch_next();
     P q[Q];
     collide<L, XS, P>(p.c, s, X, gall, g, dX, d, q);
