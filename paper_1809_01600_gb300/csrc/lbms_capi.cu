@@ -994,6 +994,7 @@ lbms_status lbms_create_batch(int n_cases, const lbms_geometry* geoms, const lbm
         for (const auto& cs : c->cases) max_nf = std::max(max_nf, cs.nf);
         L.small = choose_small(L, max_nf);
         L.tiled = !L.small && 3 * (int64_t)c->Q * (L.S + kTile) < (int64_t)1 << 32;
+        L.fine = L.tiled && tile_fine(L);
     }
 
     // reduction segments and block -> case tables
@@ -1484,8 +1485,8 @@ lbms_status lbms_get_info(const lbms_ctx* c, lbms_info* info) {
     info->d2h_bytes = c->d2h;
     info->n_cases = (int)c->cases.size();
     if (c->L.tiled) {
-        info->tile_cells = kTile;
-        info->tile_min_blocks = tile_min_blocks(c->dim, c->opt.precision);
+        info->tile_cells = c->L.fine ? kFineCells : kTile;
+        info->tile_min_blocks = c->L.fine ? kFineMinBlocks : tile_min_blocks(c->dim, c->opt.precision);
         info->neighbour_bits = c->L.b.rowtab ? 1 : 32;
         info->threads_per_cell = 1;
         return LBMS_OK;

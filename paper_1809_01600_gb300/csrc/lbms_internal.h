@@ -43,10 +43,16 @@ constexpr int kTilePrefetch = 160;      // 24,320 cells on 152 SMs
 constexpr int tile_min_blocks(int dim, int precision) {
     return dim == 2 ? (precision == 1 ? 12 : 8) : (precision == 0 ? 5 : 10);
 }
-// Below this many cells (4 blocks of 64 on each of 152 SMs) a launch does not
-// fill the GPU and the small handles' step is the faster: 37 k cells in FP32
-// take 4.0 us, 46 k with the tiled step 4.7 (26 k: 3.9 against 5.5).
-constexpr int kTileMinCells = 38913;
+// Blocks of a tile that its registers let an SM hold (FP64 in 3-D: 6 of 168
+// registers a thread, though 5 are asked for).
+constexpr int tile_resident(int dim, int precision) {
+    return dim == 2 ? (precision == 0 ? 8 : 12) : (precision == 0 ? 6 : 10);
+}
+// FP64 in 3-D where a second wave of such blocks would be less than half full
+// takes blocks of half a tile instead, 20 an SM with 96 registers a thread, all
+// of them at once: 60 k cells 107 -> 95 us, 67 k 107 -> 99, but 55 k (one wave) 80
+// -> 83, 74 k 107 -> 110 and 1.7 M 2230 -> 2300 us (16 an SM), from its spills.
+constexpr int kFineCells = kTile / 2, kFineMinBlocks = 20;
 
 // Steps of handles that do not fill the GPU (lbms_step_small.cuh): many steps
 // of a block per case of at most 64, 128 or 320 cells, or a launch a step.
@@ -100,6 +106,7 @@ struct Launch {
     int variant = 0;                   // chosen step-kernel tile shape
     bool tiled = false;                // the step of lbms_step_tile.cuh and its population layout, instead of a variant
     int small = kNotSmall;             // which of the small handles' steps, instead of a variant
+    bool fine = false;                 // the tiled step's blocks are half tiles
     bool windows16() const { return tiled || small != kNotSmall; }   // the row table's form (no 16-bit table then)
     int cur = 0;                       // lattice holding the latest post-collision state
     DevBuffers b;
@@ -157,6 +164,7 @@ cudaError_t launch_step_variant(const Launch& L, int variant, cudaStream_t st);
 cudaError_t launch_step_variant_literal(const Launch& L, int variant, cudaStream_t st);
 // the default step (lbms_step_tile.cuh); needs L.tiled; bytes of a cell's populations in its layout
 size_t tile_cell_bytes(int dim, int precision);
+bool tile_fine(const Launch& L);   // whether it takes kFineCells a block; L.ncells and sm_count are set
 cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 // the step for a handle whose largest case has max_nf cells, or kNotSmall;
 // L.ncells, n_cases and sm_count are set

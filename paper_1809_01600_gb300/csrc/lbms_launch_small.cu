@@ -112,6 +112,20 @@ bool block_pays(const Launch& L, int block) {
     return of_blocks <= 3 * ((L.ncells / kSmallCells[kSmall] + a - 1) / a);
 }
 
+// Whether a launch of blocks of 32 cells and three threads a cell is the faster
+// step, against the tiled one; `per` cells make one block of a tile on each SM.
+// us per step, this / tiled: FP32 3-D 36 k cells 4.0 / 5.1, 42 k 5.4 / 5.1, 2-D 37 k
+// 3.0 / 3.4, 44 k 3.2 / 3.1.  FP64, bound by the pipe of the fullest SM, gains from the
+// finer blocks while there are few: 2-D 40 k cells 38 / 43, 57 k 50 / 50, 67 k 62 / 60, and
+// once more where the tiled step starts a second wave of 8 blocks an SM: 81 k 71 /
+// 80, 92 k 82 / 80; 3-D 41 k 60 / 70, 49 k 73 / 80, 52 k 73 / 80, 54 k 80 / 80.
+bool small_pays(const Launch& L) {
+    const int64_t n = L.ncells, per = (int64_t)kTile * L.sm_count;
+    if (L.precision != 0) return n <= 4 * per;
+    if (L.dim == 2) return n <= 6 * per || (n > 8 * per && n <= 9 * per);
+    return 2 * n <= 11 * per;
+}
+
 }  // namespace
 
 int choose_small(const Launch& L, int max_nf) {
@@ -120,7 +134,7 @@ int choose_small(const Launch& L, int max_nf) {
             if (block_pays(L, block)) return block;
             break;
         }
-    return L.ncells < kTileMinCells ? kSmall : kNotSmall;
+    return small_pays(L) ? kSmall : kNotSmall;
 }
 
 cudaError_t launch_steps_block(const Launch& L, int n, cudaStream_t st) {

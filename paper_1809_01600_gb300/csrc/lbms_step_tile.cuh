@@ -59,6 +59,7 @@ struct TileParams {
     const CaseBC<XS>* cases;
     const int* blk_case;
     int64_t S;
+    bool side;                          // the next step fits beside this one: let in after the wait
     int pf_dist;                        // cells ahead to prefetch into L2
     MsConst<typename Xv<XS>::T> c;
 };
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
     using T = typename Xv<XS>::T;
     using XV = Xv<XS>;
     using PT = Pk<T>;
-    static_assert(W == kTile, "a block covers a tile");
+    static_assert(kTile % W == 0, "a block lies in a tile");
     using Lay = TileLay<L, P>;
     using U = typename Lay::U;
     constexpr bool kHalf = std::is_same<P, __half>::value;
@@ -226,9 +227,9 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
     constexpr int NP = (Q - 1) / 2;          // link pairs (k, k + 1), opposite to each other
     constexpr T sc = T(Pop<T, P>::kStore);   // d, dX and the collision work in storage units (h * kStore)
 
-    grid_launch_next();
+    if (!p.side) grid_launch_next();
     const int i = blockIdx.x * W + threadIdx.x;
-    const CaseBC<XS>& cb = p.cases[__ldg(p.blk_case + blockIdx.x)];
+    const CaseBC<XS>& cb = p.cases[__ldg(p.blk_case + blockIdx.x / (kTile / W))];
     Source src[Q];
     bool at_in, at_out;
     if constexpr (std::is_same<NBT, RowMaskNb>::value)
@@ -237,9 +238,10 @@ __global__ void __launch_bounds__(W, MB) step_tile_kernel(const TileParams<XS, P
     else
         table_sources<L, P>(p.nbr32, i, src, at_in, at_out);
     grid_wait();
+    if (p.side) grid_launch_next();
 
     const int64_t S = p.S;
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 4 && blockIdx.x % (kTile / W) == 0) {
         // the tile and the X rows that blocks a third of a wave later start from
         const int64_t j = (int64_t)blockIdx.x * W + p.pf_dist;   // a multiple of the tile
         if (j + kTile <= S) {

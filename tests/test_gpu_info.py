@@ -63,3 +63,41 @@ def test_a_block_per_case_where_it_pays(L, dim, precision, fluid, cases_, want):
     if torch.cuda.get_device_properties(0).multi_processor_count != 152:
         pytest.skip("the counts are for 152 SMs")
     assert _info(L, [_box(dim, fluid)] * cases_, precision)[0] == want
+
+
+def _channel(nx, ny, nz, fluid):
+    """A channel with `fluid` fluid cells, end planes fluid."""
+    import numpy as np
+    from workloads import cases
+    c = cases.open_channel(nx, ny, nz, current_A_cm2=1.0)
+    inner = c.solid[:, :, 1:-1]
+    drop = np.random.default_rng(fluid).permutation(inner.size)[:c.solid.size - fluid]
+    z, y, x = np.unravel_index(drop, inner.shape)
+    inner[z, y, x] = True
+    assert c.n_fluid == fluid
+    return c
+
+
+# cells per block, threads per cell: launches of 32 cells (three threads each),
+# tiles of 64, or halves of them where a second wave of tiles would be short
+FP64 = [((300, 220, 1), 58368, (32, 3)), ((300, 220, 1), 58369, (64, 1)), ((400, 220, 1), 77824, (64, 1)),
+        ((400, 220, 1), 77825, (32, 3)), ((400, 220, 1), 87552, (32, 3)), ((400, 220, 1), 87553, (64, 1)),
+        ((60, 40, 32), 53504, (32, 3)), ((60, 40, 32), 53505, (64, 1)), ((60, 40, 32), 58368, (64, 1)),
+        ((60, 40, 32), 58369, (32, 1)), ((60, 40, 32), 72960, (32, 1)), ((60, 40, 32), 72961, (64, 1))]
+
+
+@pytest.mark.parametrize("shape,fluid,want", FP64)
+def test_fp64_by_size(L, shape, fluid, want):
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the sizes are for 152 SMs")
+    cells, _, bits, threads = _info(L, [_channel(*shape, fluid)], "fp64")
+    assert (cells, threads) == want and bits == 1
+
+
+@pytest.mark.parametrize("shape,fluid", [((300, 220, 1), 50001), ((400, 220, 1), 80001), ((60, 40, 32), 50001),
+                                         ((60, 40, 32), 58369), ((60, 40, 32), 66001), ((60, 40, 32), 72960)])
+@pytest.mark.parametrize("periodic", [False, True])
+def test_fp64_steps_against_a_forced_variant(L, shape, fluid, periodic):
+    from test_gpu_step_small import _same
+    _same(L, [_channel(*shape, fluid).with_(periodic_x=periodic)], "fp64", 1e-12, (33, 2))
