@@ -265,7 +265,11 @@ lbms_status lbms_batch_run_to_residual(lbms_ctx *ctx, double tol, int64_t max_st
 /* Fields of the last step on the dense grid, solid voxels zero (case 0).
  * X: 3*N mole fractions.  u: 3*dim*N component velocities (m/s,
  * [species][axis][z][y][x], Eq. 20) or NULL.  tau: 3*N relaxation times
- * (Eq. 25) or NULL. */
+ * (Eq. 25) or NULL.
+ * Setting and reading the fields of grids of 16384 cells or more takes device
+ * memory for the dense grid: 24 bytes a cell of the handle's largest grid, kept
+ * from the first such call; beyond 256 MB, 8 bytes a cell for the call alone.
+ * Where there is none left the host converts. */
 lbms_status lbms_get_fields(lbms_ctx *ctx, double *X, double *u, double *tau);
 
 /* As lbms_get_fields for case k (arrays sized for that case's grid). */

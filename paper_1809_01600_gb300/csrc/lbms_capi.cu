@@ -319,10 +319,11 @@ lbms_status autotune(lbms_ctx* c) {
 constexpr int64_t kDenseMin = 16384;
 constexpr int64_t kDenseSpecies = 1 << 28;   // bytes up to which the three species go in one copy
 
-// Device room for the dense grid of the largest case, three species of it
-// (one beyond kDenseSpecies bytes), kept from its first use; null if the
-// handle has no coordinate words, the case is small, or no memory was left
-// when it was first asked for: the caller then converts on the host.
+// Device room for the dense grid of the largest case, three species of it and
+// kept from its first use, or one species beyond kDenseSpecies bytes and given
+// back by dense_done; null if the handle has no coordinate words, the case is
+// small, or no memory was left when it was first asked for: the caller then
+// converts on the host.
 double* dense_scratch(lbms_ctx* c, const CaseHost& cs, int& species) {
     if (!c->L.b.cell_code || cs.N < kDenseMin || c->dense_refused) return nullptr;
     int64_t n = 0;
@@ -331,6 +332,15 @@ double* dense_scratch(lbms_ctx* c, const CaseHost& cs, int& species) {
     if (!c->L.b.dense) c->L.b.dense = static_cast<double*>(dev_alloc(c, (size_t)species * n * sizeof(double)));
     c->dense_refused = !c->L.b.dense;
     return c->L.b.dense;
+}
+
+// After the conversions of a call (and the stream's work): what a handle keeps
+// of it is kDenseSpecies bytes at most.  A larger room costs a millisecond to
+// ask for, the copy of such a grid a hundred.
+void dense_done(lbms_ctx* c, int species) {
+    if (species == 3) return;
+    dev_free(c, c->L.b.dense);
+    c->L.b.dense = nullptr;
 }
 
 // Copies a dense host field of case k (3 * N doubles) into X[cur] and
@@ -350,6 +360,7 @@ lbms_status upload_field(lbms_ctx* c, int k, const double* X) {
         c->h2d += (size_t)3 * cs.N * sizeof(double);
         CK(launch_init(c->L, cs.base, cs.nf, c->stream), "init kernel");
         CK(cudaStreamSynchronize(c->stream), "init");
+        dense_done(c, per);
         return LBMS_OK;
     }
     const int rows = x_rows(prec);
@@ -1360,6 +1371,7 @@ lbms_status lbms_batch_get_fields(lbms_ctx* c, int k, double* X, double* u, doub
         }
         CK(cudaStreamSynchronize(c->stream), "read X");
         c->d2h += (size_t)3 * cs.N * sizeof(double);
+        dense_done(c, per);
     } else if (X) {
         const int rows = x_rows(prec);
         const size_t word = x_word(prec);

@@ -487,8 +487,8 @@ struct lbms_net {
     int gemm_kind = LBMS_NET_GEMM_AUTO;
     int64_t tcgen05_calls = 0, mma_sync_calls = 0;
     std::vector<void*> allocs;
-    char* room = nullptr;                   // working memory of the case at hand, kept and grown on demand
-    size_t room_bytes = 0;
+    char* room = nullptr;                   // working memory of the case at hand, grown on demand and kept
+    size_t room_bytes = 0;                  //   up to kRoomKept bytes
     std::string err;
 };
 
@@ -703,10 +703,24 @@ lbms_status backward_step(lbms_net* n, int R, double lr, double* loss) {
     return LBMS_OK;
 }
 
+// Working memory that a network keeps between calls (about 43 bytes a voxel and
+// 168 a fluid cell: grids of 5 M voxels); what a larger case took goes back at
+// the end of its call, which takes ten milliseconds or more.
+constexpr size_t kRoomKept = (size_t)512 << 20;
+
 // Feature rows (device, [rows_pad][kF], zero padded) and the per-x table of
 // one case, with room for a prediction; rows_pad = nf rounded up to 64.  All
 // of it lies in the net's working memory, valid until its next case.
 struct CaseFeatures {
+    explicit CaseFeatures(lbms_net* n) : net(n) {}
+    CaseFeatures(const CaseFeatures&) = delete;
+    ~CaseFeatures() {
+        if (net->room_bytes <= kRoomKept) return;
+        cudaFree(net->room);                // waits for the device
+        net->room = nullptr;
+        net->room_bytes = 0;
+    }
+    lbms_net* net;
     bf16* rows = nullptr;
     float* xtab = nullptr;
     int64_t* cell = nullptr;         // dense index of each fluid cell
@@ -957,7 +971,7 @@ lbms_status lbms_net_features(lbms_net* n, lbms_ctx* ctx, int k, uint16_t* rows,
     if (!lbms::case_view(ctx, k, &v)) return nfail(n, LBMS_EINVAL, "case index %d out of range", k);
     if (n_rows != v.nf) return nfail(n, LBMS_EINVAL, "case %d has %d fluid cells, the buffer holds %lld rows", k, v.nf,
                                      (long long)n_rows);
-    CaseFeatures F;
+    CaseFeatures F(n);
     lbms_status st = case_features(n, ctx, k, F);
     if (st != LBMS_OK) return st;
     NCK(cudaMemcpy(rows, F.rows, (size_t)v.nf * kF * sizeof(bf16), cudaMemcpyDeviceToHost), "feature rows");
@@ -966,7 +980,7 @@ lbms_status lbms_net_features(lbms_net* n, lbms_ctx* ctx, int k, uint16_t* rows,
 
 lbms_status lbms_net_add_sample(lbms_net* n, lbms_ctx* ctx, int k) {
     if (!n || !ctx) return LBMS_EINVAL;
-    CaseFeatures F;
+    CaseFeatures F(n);
     lbms_status st = case_features(n, ctx, k, F);
     if (st != LBMS_OK) return st;
     lbms::CaseView v;
@@ -1120,7 +1134,7 @@ lbms_status lbms_net_set(lbms_net* n, const float* buf, int64_t count) {
 
 lbms_status lbms_net_warm_start(lbms_net* n, lbms_ctx* ctx, int k, double* Xout) {
     if (!n || !ctx) return LBMS_EINVAL;
-    CaseFeatures F;
+    CaseFeatures F(n);
     lbms_status st = case_features(n, ctx, k, F);
     if (st != LBMS_OK) return st;
     lbms::CaseView v;

@@ -925,7 +925,7 @@ lbms_status lbms_unet_gemm_calls(const lbms_unet* u, int64_t* tcgen05_calls) {
 
 lbms_status lbms_unet_add_sample(lbms_unet* u, lbms_ctx* ctx, int k) {
     if (!u || !ctx) return LBMS_EINVAL;
-    CaseFeatures F;
+    CaseFeatures F(&u->feat);
     lbms_status st = case_features(&u->feat, ctx, k, F);
     if (st != LBMS_OK) return ufail(u, st, "%s", u->feat.err.c_str());
     lbms::CaseView v;
@@ -1087,7 +1087,7 @@ lbms_status lbms_unet_train(lbms_unet* u, int iters, int max_batch, double lr, d
 
 lbms_status lbms_unet_warm_start(lbms_unet* u, lbms_ctx* ctx, int k, double* Xout) {
     if (!u || !ctx) return LBMS_EINVAL;
-    CaseFeatures F;
+    CaseFeatures F(&u->feat);
     lbms_status st = case_features(&u->feat, ctx, k, F);
     if (st != LBMS_OK) return ufail(u, st, "%s", u->feat.err.c_str());
     lbms::CaseView v;

@@ -99,9 +99,11 @@ def test_one_species_at_a_time(L, precision):
     c = _tube(2048, 72, 77)                          # 11.4 M voxels: three species pass 256 MB
     X = _field(c)
     s = L.Solver.from_case(c, precision=precision)
+    held = s.info().device_bytes
     s.set_bc(c.x_in, c.current_A_cm2)
     s.set_fields(X)
     got = s.fields()
+    assert s.info().device_bytes == held             # given back after each call
     assert np.abs(got - X)[:, ~c.solid].max() <= (0.0 if precision == "fp64" else 2.0 ** -48)
     assert np.all(got[:, c.solid] == 0.0)
     s.close()
@@ -119,4 +121,37 @@ def test_training_goes_on_after_a_batch_that_did_not_fit(L):
         assert e.value.status == L.LBMS_ENOMEM
         assert np.array_equal(net.forward(small), want)
     assert np.array_equal(net.forward(small), want)
+    net.close()
+
+
+def test_what_a_handle_keeps(L):
+    c = _tube(256, 64, 64)                           # 1.05 M voxels: 25 MB for three species
+    s = L.Solver.from_case(c)
+    held = s.info().device_bytes
+    for _ in range(2):
+        s.set_bc(c.x_in, c.current_A_cm2)
+        s.set_fields(_field(c))
+        s.fields()
+    assert s.info().device_bytes - held == 24 * c.solid.size <= 256 << 20
+    s.close()
+
+
+def test_what_a_network_keeps(L):
+    net = L.Net(width=64, depth=1, seed=1)
+    s = []
+    for shape, most in (((256, 64, 64), 64 << 20), ((2048, 96, 80), 512 << 20)):   # 45 MB and 680 MB of working memory
+        c = _tube(*shape)
+        s.append(L.Solver.from_case(c, torch_allocator=False))
+        s[-1].set_bc(c.x_in, c.current_A_cm2)
+        s[-1].fields()                               # the handle's own room, kernels loaded
+        net.features(s[0], int((~_tube(256, 64, 64).solid).sum()))
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(2):
+            X = net.warm_start(s[-1])
+        assert free - torch.cuda.mem_get_info()[0] <= (2 << 20) + (0 if shape[0] == 2048 else most)
+        assert np.abs(X.sum(0)[~c.solid] - 1.0).max() <= 1e-12
+        del X
+    for h in s:
+        h.close()
     net.close()
