@@ -221,10 +221,13 @@ def measured_peak_hbm():
 
 
 def kernel_source_sha():
+    """Hash of every source that the step kernels and their choice are built from."""
+    csrc = os.path.join(ROOT, "paper_1809_01600_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("lbms_kernels.cuh", "lbms_lattice.cuh", "lbms_launch.cu", "lbms_step_launch.cuh"):
-        with open(os.path.join(ROOT, "paper_1809_01600_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+    for f in sorted(os.listdir(csrc)):
+        if f.startswith(("lbms_kernels", "lbms_lattice", "lbms_launch", "lbms_step", "lbms_internal")):
+            with open(os.path.join(csrc, f), "rb") as fh:
+                h.update(fh.read())
     return h.hexdigest()[:16]
 
 

@@ -1,5 +1,7 @@
-"""The kernel that the benchmark names from a handle's step description."""
+"""The kernel that the benchmark names from a handle's step description, and the
+hash that its committed traffic figures are valid for."""
 import os
+import shutil
 import sys
 
 import pytest
@@ -16,3 +18,17 @@ import bench  # noqa: E402
 def test_step_kernel_name(forced, cells, threads, want):
     info = type("I", (), dict(tile_cells=cells, threads_per_cell=threads))()
     assert bench.step_kernel_name(forced, info) == want
+
+
+def test_the_source_hash_covers_every_step_kernel(tmp_path, monkeypatch):
+    csrc = os.path.join(bench.ROOT, "paper_1809_01600_gb300", "csrc")
+    copy = tmp_path / "paper_1809_01600_gb300" / "csrc"
+    shutil.copytree(csrc, copy)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    shas = {bench.kernel_source_sha()}
+    steps = ["lbms_kernels.cuh", "lbms_step_tile.cuh", "lbms_step_small.cuh", "lbms_launch_tile.cu",
+             "lbms_launch_small.cu", "lbms_launch.cu", "lbms_step_launch.cuh", "lbms_lattice.cuh", "lbms_internal.h"]
+    for f in steps:
+        (copy / f).write_text((copy / f).read_text() + "// changed\n")
+        shas.add(bench.kernel_source_sha())
+    assert len(shas) == 1 + len(steps)
