@@ -1,6 +1,6 @@
 // C ABI of the solver (declared in include/lbms.h): validation, host
 // properties, fluid-cell indexing, batching of cases into one index space,
-// device state, tile autotuning, CUDA-graph stepping, residual loops and
+// device state, choice of the step, CUDA-graph stepping, residual loops and
 // the FP64 post-processing of Eq. 43.  A single-case solver is a batch of 1.
 #include <algorithm>
 #include <cmath>
@@ -313,9 +313,9 @@ lbms_status autotune(lbms_ctx* c) {
 
 // The conversion between a case's dense grid (the caller's) and its fluid
 // cells runs on the device from kDenseMin cells on: reading 96^3 cells takes
-// 0.2 ms where host loops took 1.4, 256x128x128 7.6 ms where they took 16 (5 of
-// either is the first touch of the caller's pages).  Below, a copy of the
-// cells and a host loop are one launch less.
+// 0.2 ms where host loops took 1.4, 256x128x128 3.9 ms where they took 16 (most
+// of it the first touch of the caller's pages).  Below, a copy of the cells and a
+// host loop are one launch less.
 constexpr int64_t kDenseMin = 16384;
 constexpr int64_t kDenseSpecies = 1 << 28;   // bytes up to which the three species go in one copy
 

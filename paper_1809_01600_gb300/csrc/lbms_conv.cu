@@ -14,13 +14,14 @@
 // What bounds these products: an operand A of 128 rows is 4 KB of shared
 // memory per MMA whatever N is, so at N = 32 (the full resolution) an MMA
 // takes about 50 cycles where its arithmetic takes 8; storing 32 channels
-// instead of 64 there quartered the MMAs.  A training step on 4 volumes of
-// 96^3 takes 6.6 ms, on 8 of 64x32x32 1.7 ms (43.5 and 7.45 with 64 channels
-// stored, FP32 products in memory, transposed copies for the weight gradients
-// and row-wise kernels between the products).  Of the 6.6 ms the 32-channel
-// convolutions take 0.35 ms each (66 cycles an MMA), their input gradients
-// 0.28, their weight gradients 0.22.  Reading the timer on every barrier wait
-// and issuing from a single lane's branch cost twice that.
+// instead of 64 there quartered the MMAs.  The kernels of a training step on 4
+// volumes of 96^3 take 6.5 ms, on 8 of 64x32x32 1.5 ms (calls that read the
+// gradients 6.95 and 1.92; 48.5 and 13.2 with 64 channels stored, FP32 products
+// in memory, transposed copies for the weight gradients and row-wise kernels
+// between the products).  Of the 6.5 ms the 32-channel convolutions take 0.35 ms
+// each (66 cycles an MMA), their input gradients 0.28, their weight gradients
+// 0.22.  Reading the timer on every barrier wait and issuing from a single
+// lane's branch cost twice that.
 #include <cuda_bf16.h>
 
 #include <algorithm>

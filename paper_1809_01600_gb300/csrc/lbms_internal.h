@@ -55,7 +55,8 @@ constexpr int tile_resident(int dim, int precision) {
 constexpr int kFineCells = kTile / 2, kFineMinBlocks = 20;
 
 // Steps of handles that do not fill the GPU (lbms_step_small.cuh): many steps
-// of a block per case of at most 64, 128 or 320 cells, or a launch a step.
+// of a block per case of at most 64, 128 or 320 cells, or a launch a step.  The
+// rules stand in lbms_launch_small.cu.
 enum { kNotSmall = 0, kBlock64, kBlock128, kBlock320, kSmall };
 constexpr int kSmallCells[] = {0, 64, 128, 320, 32};        // cells per block of each
 constexpr int kSmallMinBlocks[] = {0, 1, 1, 1, 4};          // and blocks per SM its registers are budgeted for
@@ -169,7 +170,7 @@ cudaError_t launch_step_tile(const Launch& L, cudaStream_t st);
 // the step for a handle whose largest case has max_nf cells, or kNotSmall;
 // L.ncells, n_cases and sm_count are set
 int choose_small(const Launch& L, int max_nf);
-cudaError_t launch_step_small(const Launch& L, cudaStream_t st);
+cudaError_t launch_step_small(const Launch& L, cudaStream_t st);   // kSmall
 // n <= kBlockSteps steps of a kBlock* handle; cur turns n & 1 times
 cudaError_t launch_steps_block(const Launch& L, int n, cudaStream_t st);
 cudaError_t launch_init(const Launch& L, int first, int count, cudaStream_t st);
@@ -227,8 +228,8 @@ enum ConvOut {
     kOutUp,         // transposed 2x2x2 convolution: column t Cg + n of an interior row, plus bias[n], to the row's
                     //   child t of the finer layout, cat[child][n] (n < w)
     kOutHead        // Y = acc + bias (3 columns): Y[r][4] if given; against T [r][4] = (targets, mask), if given,
-                    //   out[r][n] = BF16(grad_scale (Y - T) mask) (0 for n >= 3), its column sums (FP64) to gb and
-                    //   loss_scale sum((Y - T)^2 mask^2) into loss
+                    //   out[r][n] = BF16(grad_scale (Y - T) mask) (0 for n >= 3), its column sums (FP32 over a
+                    //   thread's rows, FP64 over the threads) to gb and loss_scale sum((Y - T)^2 mask^2) into loss
 };
 struct ConvEpilogue {
     const float* bias = nullptr;

@@ -149,7 +149,6 @@ cudaError_t launch_steps_block(const Launch& L, int n, cudaStream_t st) {
 }
 
 cudaError_t launch_step_small(const Launch& L, cudaStream_t st) {
-    if (L.small != kSmall) return launch_steps_block(L, 1, st);
     if (L.dim == 2) {
         if (L.precision == 0) return small_t<D2Q9, double, double>(L, st);
         if (L.precision == 1) return small_t<D2Q9, float, float>(L, st);

@@ -3,7 +3,7 @@
 // again.  One thread per (species, cell), as in step_kernel.
 //  * block_steps_kernel: every case fits a block, which keeps the case's whole
 //    state in shared memory over many steps; a step costs two block barriers.
-//    15 strips of 64 nodes in FP32: 0.60 us per step, 1.86 with a launch each.
+//    15 strips of 64 nodes in FP32: 0.61 us per step, 1.79 with a launch each.
 //  * step_small_kernel: one step per launch, launches overlapped (programmatic
 //    dependent launch).  The three threads of a cell split its source rows
 //    (row windows: 9 rows of D3Q19 as 3 + 2 + 4, 6 links each) or its row of
@@ -13,7 +13,7 @@
 //    (lbms_launch_small.cu).
 // Keeping all blocks resident with a grid-wide barrier, or with flags between
 // the blocks that exchange, was no faster than overlapped launches where FP32
-// is the arithmetic: 26 k cells took 4.3 and 5.0 us per step.
+// is the arithmetic: 26 k cells took 4.3 and 5.0 us per step, launches 3.9.
 #pragma once
 
 #include "lbms_internal.h"
@@ -266,9 +266,9 @@ __device__ __forceinline__ void share_table(const int* __restrict__ nbr, int i, 
 
 // One step of blocks of W = 32 cells (blocks of 16 and 64 were slower on one or
 // another of 2-D and 3-D handles of 2 to 37 k cells in FP64, FP32 and FP16).
-// us per step, before / now: 2-D 2.1 k cells FP64 8.8 / 6.7, FP32 2.2 / 1.9; 9 k
-// FP64 12.0 / 9.8; 3-D 4.8 k FP32 2.9 / 2.6, 26 k FP32 4.6 / 3.9, FP16 4.7 / 3.9,
-// FP64 47 / 41, 37 k FP32 4.7 / 4.0.
+// us per step, with step_kernel / now: 2-D 2.2 k cells FP64 8.3 / 6.8, 2.4 k FP32
+// 2.1 / 1.7; 9 k FP64 12.0 / 9.9; 3-D 5.2 k FP32 2.6 / 2.2, 26 k FP32 4.1 / 3.7, FP64 47 /
+// 41, 36 k FP32 4.6 / 4.0.
 template <class L, typename XS, typename P, int W>
 __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_kernel(const SmallParams<XS, P> p) {
     using T = typename Xv<XS>::T;

@@ -10,7 +10,8 @@
 // prefetches into L2.  X keeps its rows of stride S.
 //
 // What bounds it (256x128x128 anode, 1,689,574 fluid cells, D3Q19): FP32
-// moves 826 MB a step and takes 140 us, 5.9 TB/s of the 6.8 a copy reaches;
+// moves 826 MB a step and takes 140 to 149 us on one GB300 or another, 5.6 to
+// 5.9 TB/s of the 6.8 a copy reaches;
 // with the neighbour decode, the address arithmetic and the boundary rules
 // spread over the links the step before issued 108 M warp instructions and
 // took 181 us, this one issues 66 M.  FP16 moves 449 MB in 101 us (151

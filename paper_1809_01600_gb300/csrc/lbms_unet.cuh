@@ -202,7 +202,7 @@ __global__ void conv_cast_kernel(const float* __restrict__ W, int co_s, int ci_s
 }
 
 // A batch given as FP32 [B][17][Z][Y][X] (channel 16 the fluid mask) into
-// the interior rows of x0 [rows][64] (BF16) and the mask column of T [rows][4]
+// the interior rows of x0 [rows][kUInC] (BF16) and the mask column of T [rows][4]
 // (both cleared before); one warp per voxel.
 __global__ void vol_in_kernel(const float* __restrict__ in, Geo g, bf16* __restrict__ x0, float* __restrict__ T) {
     const int lane = threadIdx.x & 31;
@@ -316,7 +316,7 @@ struct lbms_unet {
     struct Sample {
         int X = 0, Y = 0, Z = 0;                // interior extents (multiples of 4)
         int64_t rows = 0, nfluid = 0;           // rows of its layout; fluid voxels
-        bf16* in = nullptr;                     // [rows][64]
+        bf16* in = nullptr;                     // [rows][kUInC]
         float* tg = nullptr;                    // [rows][4]: 100 (X - profile), fluid mask
     };
     std::vector<Sample> samples;
@@ -367,7 +367,9 @@ T* ualloc(lbms_unet* u, size_t count) {
 // truncate, so a chunk's length is its error: 2e-5 to 3e-5 of a gradient at this
 // length, and 3.5e-5 more with chunks 2.4 times as long.
 constexpr int64_t kChunkRows = 16384;
-constexpr int64_t kGemmMaxRows = 65535ll * 128;   // grid limit of the GEMM's row tiles
+// Rows of a level at most: what batches were always limited to (the kernels'
+// row numbers are 32-bit, and rows times channels fit 63 bits far beyond it).
+constexpr int64_t kGemmMaxRows = 65535ll * 128;
 
 // Zero rows behind the last volume that the weight gradients of the 3x3x3
 // convolutions need (they reach dz up to two rows late).
