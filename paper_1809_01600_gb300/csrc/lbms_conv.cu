@@ -18,10 +18,11 @@
 // volumes of 96^3 take 6.5 ms, on 8 of 64x32x32 1.5 ms (calls that read the
 // gradients 6.95 and 1.92; 48.5 and 13.2 with 64 channels stored, FP32 products
 // in memory, transposed copies for the weight gradients and row-wise kernels
-// between the products).  Of the 6.5 ms the 32-channel convolutions take 0.35 ms
-// each (66 cycles an MMA), their input gradients 0.28, their weight gradients
-// 0.22.  Reading the timer on every barrier wait and issuing from a single
-// lane's branch cost twice that.
+// between the products).  Of the 6.5 ms the 32-channel convolutions take 0.28 ms
+// each (52 cycles an MMA, shared memory at 74 %) and the one that copies into a
+// concatenation 0.5 (its stores), their input gradients 0.28, their weight
+// gradients 0.22.  Reading the timer on every barrier wait and issuing from a
+// single lane's branch cost twice that.
 #include <cuda_bf16.h>
 
 #include <algorithm>
