@@ -40,7 +40,6 @@ SmallParams<XS, P> params(const Launch& L, int n) {
     }
     p.cur = L.cur;
     p.n = n;
-    p.side = small_overlap(L).side;
     p.nbr32 = L.b.nbr;
     p.cell_code = L.b.cell_code;
     p.rowtab = reinterpret_cast<const uint2*>(L.b.rowtab);
@@ -74,8 +73,11 @@ cudaError_t small_t(const Launch& L, cudaStream_t st) {
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = small_overlap(L).on ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, step_small_kernel<Lat, XS, P, W>, params<Lat, XS, P>(L, 1));
+    const Overlap over = small_overlap(L);
+    cfg.numAttrs = over.on ? 1 : 0;
+    return cudaLaunchKernelEx(
+        &cfg, over.side ? step_small_kernel<Lat, XS, P, W, true> : step_small_kernel<Lat, XS, P, W, false>,
+        params<Lat, XS, P>(L, 1));
 }
 
 template <class Lat, typename XS, typename P>

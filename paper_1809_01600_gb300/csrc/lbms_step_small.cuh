@@ -30,7 +30,6 @@ struct SmallParams {
     XS* x[2];
     int cur;                            // lattice holding the state
     int n;                              // steps (block_steps_kernel)
-    bool side;                          // the next step fits beside this one (step_small_kernel)
     const int* nbr32;
     const uint32_t* cell_code;
     const uint2* rowtab;                // windows of the tiled step, or null: nbr32
@@ -269,7 +268,8 @@ __device__ __forceinline__ void share_table(const int* __restrict__ nbr, int i, 
 // us per step, with step_kernel / now: 2-D 2.2 k cells FP64 8.3 / 6.8, 2.4 k FP32
 // 2.1 / 1.7; 9 k FP64 12.0 / 9.9; 3-D 5.2 k FP32 2.6 / 2.2, 26 k FP32 4.1 / 3.7, FP64 47 /
 // 41, 36 k FP32 4.6 / 4.0.
-template <class L, typename XS, typename P, int W>
+// SIDE: the next step fits beside this one (small_overlap).
+template <class L, typename XS, typename P, int W, bool SIDE>
 __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_kernel(const SmallParams<XS, P> p) {
     using T = typename Xv<XS>::T;
     using XV = Xv<XS>;
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
             share_table<L, 2, W>(p.nbr32, i, S32, c, sN, sF);
     }
     grid_wait();
-    if (p.side) grid_launch_next();
+    if constexpr (SIDE) grid_launch_next();
     const P* hs = p.h[p.cur] + (int64_t)s * Q * S;
     const XS* xh = p.x[p.cur] + s * S;
     XV xo = XV::own_rows(xh, p.x[p.cur] + (3 + s) * S, i);
@@ -336,9 +336,9 @@ __global__ void __launch_bounds__(3 * W, kSmallMinBlocks[kSmall]) step_small_ker
 #pragma unroll
         for (int a = 0; a < DIM; ++a) gall[r][a] = sG[r][a][c];
     }
-    // Unless two steps fit side by side, not earlier: blocks of the next step
-    // placed while these have just begun crowd onto the SMs they find.
-    grid_launch_next();
+    // Not earlier: blocks of the next step placed while these have just begun
+    // crowd onto the SMs they find.
+    if constexpr (!SIDE) grid_launch_next();
     P q[Q];
     collide<L, XS, P>(p.c, s, X, gall, g, dX, d, q);
     P* ho = p.h[p.cur ^ 1] + (int64_t)s * Q * S;
